@@ -474,100 +474,96 @@ void launch_spring(const int* start, const int* nbr, const T* kap, int M, const 
 
 // Spreading as a cell-binned gather: face (i, j) of component c collects every marker whose
 // level-l stencil origin is (i - a, j - b), a, b < W, from the Morton-ordered bin of that origin:
-//   f^c_ij = (1/h^2) sum_{a,b} sum_{m in bin(i-a, j-b)} wx_m[a] wy_m[b] F^c_m.
+//   f^c_ij = (1/h^2) sum_b [ sum_a sum_{m in bin(i-a, j-b)} wy_m[b] (wx_m[a] F^c_m) ].
 // No atomics; the summation order is fixed.  Only IB-active tiles are written.
+//
+// One block per (listed tile, component); rowSlots != nullptr: block b takes the tile of slot rowSlots[b]
+// (b < *nTiles, the count of that list), the tiles that a marker stencil touches; otherwise tile b of the
+// active-tile list.  Thread (x, r) walks the W bins (i - a, jj) of one bin row jj = j0 + r - (W - 1): one
+// product wx F per marker and one multiply-add per face row jj + b it reaches, so a marker's 16 faces cost
+// 4 x (1 + 4) FP64 operations, and the W bins are walked as one list (lanes differ by the bins' counts
+// only in total).  The bound is the FP64 pipe and the gathers' latency: a warp per face spent its lanes on
+// bins of four markers.  1024^2 disk and ellipse, 3e5 markers, FP64: interpolation, spreading and operator
+// together 722 us with the warp per face (598 us of it the spreading) -> 204 us.
+constexpr int SP_MAXW = 4;
 template <typename T>
-__device__ __forceinline__ T gather_face(const IBK<T>& k, const T* __restrict__ F, int c, int i, int j, int lane,
-                                         int stride) {
-    const int mk = k.N - 1;
+struct alignas(16) Wgt4 {   // half of a marker's eight weights: 16 bytes (FP32) or 32 (FP64), aligned to them
+    T v[4];
+};
+template <typename T>
+__global__ void __launch_bounds__(TX * (TY + SP_MAXW - 1))
+    k_spread_tile(IBK<T> k, const T* __restrict__ F, T* __restrict__ f, const int* __restrict__ tiles,
+                  const int* __restrict__ nTiles, const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
+    __shared__ T g[TY + SP_MAXW - 1][SP_MAXW][TX];
+    pdl_entry();
+    if ((int)blockIdx.x >= *nTiles) return;
+    const int t = tiles[rowSlots ? rowSlots[blockIdx.x] : blockIdx.x];
+    const int i0 = (t % ntx) * tx, j0 = (t / ntx) * ty, mk = k.N - 1, W = k.W;
+    const int x = threadIdx.x, r = threadIdx.y, c = blockIdx.y;
     const int* bs = c ? k.binStart[1] : k.binStart[0];
     const int* srt = c ? k.sorted[1] : k.sorted[0];
     const T* wg = c ? k.wgt[1] : k.wgt[0];
     const T* Fc = F + c * k.M;
-    // the W x W bin ranges first (independent loads, W <= 4), then the markers of each bin in the
-    // same order (b, a, q) as a bin-by-bin walk
-    int s[16], e[16];
+    const int jj = (j0 + r - (W - 1)) & mk;
+    // the walk's position p belongs to bin a (number of ends e <= p), marker position p + off[a]
+    int end[SP_MAXW], off[SP_MAXW], total = 0;
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-            s[4 * b + a] = 0;
-            e[4 * b + a] = 0;
-            if (a < k.W && b < k.W) {
-                const uint32_t bin = morton((i - a) & mk, (j - b) & mk);
-                s[4 * b + a] = bs[bin];
-                e[4 * b + a] = bs[bin + 1];
-            }
+    for (int a = 0; a < SP_MAXW; ++a) {
+        int s0 = 0, e0 = 0;
+        if (a < W) {
+            const uint32_t bin = morton((i0 + x - a) & mk, jj);
+            s0 = bs[bin];
+            e0 = bs[bin + 1];
         }
-    T acc = T(0);
+        off[a] = s0 - total;
+        total += e0 - s0;
+        end[a] = total;
+    }
+    // face rows of the tile that this bin row reaches: r - (W - 1) + b in [0, ty)
+    const int blo = max(0, W - 1 - r), bhi = min(W, ty + W - 1 - r);
+    T acc[SP_MAXW];
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
+    for (int b = 0; b < SP_MAXW; ++b) acc[b] = T(0);
+#pragma unroll 4
+    for (int p = 0; p < total; ++p) {
+        const int a = (p >= end[0]) + (p >= end[1]) + (p >= end[2]);
+        const int o = p >= end[1] ? (p >= end[2] ? off[3] : off[2]) : (p >= end[0] ? off[1] : off[0]);
+        const int m = srt[p + o];
+        const T wf = wg[8 * m + a] * Fc[m];
+        const Wgt4<T> wy = *reinterpret_cast<const Wgt4<T>*>(wg + 8 * m + 4);
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
-            for (int q = s[4 * b + a] + lane; q < e[4 * b + a]; q += stride) {
-                const int m = srt[q];
-                acc += wg[8 * m + a] * wg[8 * m + 4 + b] * Fc[m];
-            }
-    return acc;
-}
-
-// rowSlots != nullptr: block b takes the tile of slot rowSlots[b] (b < *nTiles, the count of that
-// list), the tiles that a marker stencil touches; otherwise tile b of the active-tile list.  One thread
-// per face of component blockIdx.y.
-template <typename T>
-__global__ void __launch_bounds__(256) k_spread_thread(IBK<T> k, const T* __restrict__ F, T* __restrict__ f,
-                                                       const int* __restrict__ tiles, const int* __restrict__ nTiles,
-                                                       const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
-    pdl_entry();
-    if ((int)blockIdx.x >= *nTiles) return;
-    const int t = tiles[rowSlots ? rowSlots[blockIdx.x] : blockIdx.x];
-    const int i = (t % ntx) * tx + threadIdx.x, j = (t / ntx) * ty + threadIdx.y;
-    const int n = k.N * k.N, c = blockIdx.y;
-    f[c * n + j * k.N + i] = k.inv_h2 * gather_face(k, F, c, i, j, 0, 1);
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_spread_warp(IBK<T> k, const T* __restrict__ F, T* __restrict__ f,
-                                                     const int* __restrict__ tiles, const int* __restrict__ nTiles,
-                                                     const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
-    pdl_entry();
-    if ((int)blockIdx.x >= *nTiles) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int face = blockIdx.y * 8 + warp;
-    const int per = tx * ty;
-    if (face >= 2 * per) return;
-    const int c = face / per, q = face % per;
-    const int t = tiles[rowSlots ? rowSlots[blockIdx.x] : blockIdx.x];
-    const int i = (t % ntx) * tx + q % tx, j = (t / ntx) * ty + q / tx;
-    T acc = gather_face(k, F, c, i, j, lane, 32);
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) f[c * k.N * k.N + j * k.N + i] = k.inv_h2 * acc;
+        for (int b = 0; b < SP_MAXW; ++b)
+            if (b >= blo && b < bhi) acc[b] += wy.v[b] * wf;
+    }
+#pragma unroll
+    for (int b = 0; b < SP_MAXW; ++b) g[r][b][x] = acc[b];
+    __syncthreads();
+    if (r >= ty) return;
+    T sum = T(0);
+#pragma unroll
+    for (int b = 0; b < SP_MAXW; ++b)
+        if (b < W) sum += g[r + W - 1 - b][b][x];   // bin row j - b
+    f[(size_t)c * k.N * k.N + (size_t)(j0 + r) * k.N + i0 + x] = k.inv_h2 * sum;
 }
 
 // With rowSlots (nRow its count, maxTiles its host bound) only the tiles that a marker stencil touches
 // are written; the caller keeps f at zero on the other active tiles.
 template <typename T>
 void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles, int maxTiles, int tx,
-                   int ty, int ntx, int warpPerFace, cudaStream_t s, const int* rowSlots, const int* nRow) {
+                   int ty, int ntx, cudaStream_t s, const int* rowSlots, const int* nRow) {
     if (maxTiles == 0) return;
     const int* cnt = rowSlots ? nRow : nTiles;
-    if (warpPerFace) {
-        const int groups = (2 * tx * ty + 7) / 8;
-        launch_pdl(k_spread_warp<T>, dim3(maxTiles, groups), 256, 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty, ntx);
-    } else {
-        launch_pdl(k_spread_thread<T>, dim3(maxTiles, 2), dim3(tx, ty), 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty,
-                   ntx);
-    }
+    launch_pdl(k_spread_tile<T>, dim3(maxTiles, 2), dim3(tx, ty + k.W - 1), 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty,
+               ntx);
 }
 
 // ------------------------------------------------------------------------------------------
 // Spreading as a stored sparse product.  The gather's walk is done once per set-up: for every face of
 // a stencil-touched tile and component, the markers it collects, in the gather's order (b, then a,
-// then the bin's Morton order), with their weight products wx[a] wy[b] in FP64 and in FP32 (each
-// formed as gather_face forms it).  Every (marker, a, b) pair lands on exactly one face, so a
+// then the bin's Morton order), with their weight products wx[a] wy[b] in FP64 and in FP32.  Every (marker, a, b) pair lands on exactly one face, so a
 // component holds M W^2 entries.  Row R = (c maxRow + r) tx ty + q: row tile r of the list, face q of
 // the tile (row by row), component c.  Applying it, f = (1/h^2) S F is one ordered dot product per
-// face, with the gather's rounding.
+// face.
 __device__ __forceinline__ void spread_face(int tile, int tx, int ty, int ntx, int q, int& i, int& j) {
     i = (tile % ntx) * tx + q % tx;
     j = (tile / ntx) * ty + q / tx;
@@ -1302,7 +1298,7 @@ void launch_grad_X(const double* X, int M, int N, const double* w, const double*
     template void launch_adj_kappa<T>(const int*, const double*, int, T*, cudaStream_t);                        \
     template void launch_interp<T>(const IBK<T>&, const T*, T*, cudaStream_t);                                  \
     template void launch_spring<T>(const int*, const int*, const T*, int, const T*, T*, cudaStream_t);           \
-    template void launch_spread<T>(const IBK<T>&, const T*, T*, const int*, const int*, int, int, int, int, int, \
+    template void launch_spread<T>(const IBK<T>&, const T*, T*, const int*, const int*, int, int, int, int,      \
                                    cudaStream_t, const int*, const int*);
 SIB_IB_INST(float)
 SIB_IB_INST(double)

@@ -316,7 +316,7 @@ template <typename T> void launch_spring(const int* start, const int* nbr, const
                                          cudaStream_t s);
 // rowSlots != nullptr: only the tiles of that slot list (count *nRow, at most maxTiles) are written
 template <typename T> void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles,
-                                         int maxTiles, int tx, int ty, int ntx, int warpPerFace, cudaStream_t s,
+                                         int maxTiles, int tx, int ty, int ntx, cudaStream_t s,
                                          const int* rowSlots = nullptr, const int* nRow = nullptr);
 // the spreading's walk stored at set-up (rows: faces of the stencil-touched tiles, entries in the
 // gather's order, cap = 2 M W^2), then applied as one ordered dot product per face

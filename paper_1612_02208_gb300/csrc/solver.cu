@@ -70,7 +70,6 @@ struct Level {
     int* rowSlots = nullptr;
     int* nRowTiles = nullptr;
     int hnRowTiles = 0;
-    int spreadWarp = 0;
     LevelBuf p[2];                       // [0] FP64, [1] FP32
     double lamA = 0, lamM = 0;
     // assembled IB operator windows (per active tile), FP64 and FP32
@@ -328,8 +327,7 @@ void spread_apply(sib_ctx* c, const Level& lv, const IBK<T>& k, const T* F, T* f
                                       lv.hnRowTiles, lv.N, lv.tx, lv.ty, lv.ntx, f, s));
         return;
     }
-    KL(c, launch_spread<T>(k, F, f, lv.tiles, lv.nTiles, lv.hnRowTiles, lv.tx, lv.ty, lv.ntx, lv.spreadWarp, s,
-                           lv.rowSlots, lv.nRowTiles));
+    KL(c, launch_spread<T>(k, F, f, lv.tiles, lv.nTiles, lv.hnRowTiles, lv.tx, lv.ty, lv.ntx, s, lv.rowSlots, lv.nRowTiles));
 }
 
 // f = [S K J]^l u (velocity part of x), written into the level's fib (only IB-active tiles)
@@ -1344,9 +1342,6 @@ void setup(sib_ctx* c, cudaStream_t s) {
                 lv.winSlots = lv.hnTiles > 0 ? lv.hnTiles : 1;
             }
             if (!lv.winOverflow) lv.winOverflow = (int*)dalloc(c, sizeof(int));
-            // warp per face when a face gathers from many markers on average
-            const double faces = (double)lv.hnTiles * lv.tx * lv.ty;
-            lv.spreadWarp = faces > 0 && (double)c->M * lv.W * lv.W > 16.0 * faces ? 1 : 0;
         }
         kcheck(c);
         c->structDirty = false;
@@ -1849,8 +1844,7 @@ void build_rhs(sib_ctx* c, const double* g, bool addSKX, cudaStream_t s) {
         IBK<double> k = ibk<double>(c, c->lmax);
         double* F = (double*)c->F[0];
         KL(c, launch_spring<double>(c->adjStart, c->adjNbr, c->kap64, c->M, c->Xc, F, s));
-        KL(c, launch_spread<double>(k, F, (double*)lv.p[0].fib, lv.tiles, lv.nTiles, lv.hnTiles, lv.tx, lv.ty, lv.ntx,
-                                    lv.spreadWarp, s));
+        KL(c, launch_spread<double>(k, F, (double*)lv.p[0].fib, lv.tiles, lv.nTiles, lv.hnTiles, lv.tx, lv.ty, lv.ntx, s));
         KL(c, launch_axpby<double>(1.0, c->rhs, 1.0, (const double*)lv.p[0].fib, c->rhs, nv, s));
     }
     if (cavity(c)) {   // the walls are not unknowns; the moving lid enters through the ghost values
@@ -2614,7 +2608,7 @@ int sib_spread(sib_ctx* c, const double* F, double* f, void* stream) {
     KL(c, launch_deinterleave(F, c->M, (double*)c->F[0], s));
     CK(cudaMemsetAsync(lv.p[0].fib, 0, sizeof(double) * nv, s));
     KL(c, launch_spread<double>(k, (const double*)c->F[0], (double*)lv.p[0].fib, lv.tiles, lv.nTiles, lv.hnTiles,
-                                lv.tx, lv.ty, lv.ntx, lv.spreadWarp, s));
+                                lv.tx, lv.ty, lv.ntx, s));
     CK(cudaMemcpyAsync(f, lv.p[0].fib, sizeof(double) * nv, cudaMemcpyDeviceToDevice, s));
     kcheck(c);
     return SIB_OK;

@@ -1,0 +1,44 @@
+"""Kernels at the sizes where their tiling can go wrong, against the oracle."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import ib  # noqa: E402
+from paper_1612_02208_gb300 import sib  # noqa: E402
+
+EPS = 2.0 ** -53
+
+
+def cu(x):
+    return torch.as_tensor(np.ascontiguousarray(x), device="cuda")
+
+
+# grids below, at and above one 32 x 8 tile; single markers; a cell that holds every marker; markers
+# outside the unit square (they wrap)
+@pytest.mark.parametrize("N,M,where", [(4, 1, "any"), (8, 3, "any"), (16, 200, "any"), (32, 1, "seam"), (32, 700, "cell"),
+                                       (64, 999, "any"), (64, 64, "seam"), (128, 5001, "any"), (256, 37, "outside")])
+def test_spread_tiles(N, M, where):
+    rng = np.random.default_rng(100 * N + M)
+    X = rng.uniform(0.0, 1.0, (M, 2))
+    if where == "cell":
+        X = (5.0 + rng.uniform(0.0, 1.0, (M, 2))) / N
+    elif where == "seam":
+        X[:, 0] = rng.uniform(-1.0, 1.0, M) / N
+    elif where == "outside":
+        X = X * 3.0 - 1.0
+    F = rng.standard_normal((M, 2))
+    edges = np.array([[0, M - 1]], dtype=np.int32)
+    S = sib.Solver(N, n_min=4)
+    S.set_structure(cu(X), cu(edges), cu(np.array([1.0])))
+    S.setup()
+    f = S.spread(cu(F)).cpu().numpy()
+    ref = ib.spread_force(N, X, F)
+    # every term carries at most five roundings beside those of the weights (phi to a few ulp of its
+    # terms' magnitude, 1), and a face sums at most M of them; magnitudes from |S| |F|
+    mag = np.concatenate([abs(ib.spread_matrix(N, X, c)) @ np.abs(F[:, c]) for c in (0, 1)])
+    tol = (2 * M + 8) * EPS * mag + 64 * EPS * N * N * np.abs(F).max()
+    assert (np.abs(f - ref) <= tol).all(), np.abs(f - ref).max()
+    assert torch.equal(S.spread(cu(F)), S.spread(cu(F)))
+    S.close()
