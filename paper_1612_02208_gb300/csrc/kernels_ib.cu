@@ -484,7 +484,7 @@ void launch_spring(const int* start, const int* nbr, const T* kap, int M, const 
 // 4 x (1 + 4) FP64 operations, and the W bins are walked as one list (lanes differ by the bins' counts
 // only in total).  The bound is the FP64 pipe and the gathers' latency: a warp per face spent its lanes on
 // bins of four markers.  1024^2 disk and ellipse, 3e5 markers, FP64: interpolation, spreading and operator
-// together 722 us with the warp per face (598 us of it the spreading) -> 204 us.
+// together 722 us with the warp per face (598 us of it the spreading), 204 us so (66 us).
 constexpr int SP_MAXW = 4;
 template <typename T>
 struct alignas(16) Wgt4 {   // half of a marker's eight weights: 16 bytes (FP32) or 32 (FP64), aligned to them

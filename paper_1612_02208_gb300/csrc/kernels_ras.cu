@@ -9,12 +9,13 @@
 // (o <= ii, jj < o + b), nown = 3 b^2, ordered u, v, p and row-major.
 //
 // Set-up (FP64): the local operator L_k = R_k L R_k^T is assembled from the stencil (A, G, -D) and the
-// IB windows, inverted by Gauss-Jordan with partial pivoting, and the owned rows of the inverse are
-// stored (column-major, FP64 and FP32).  Boxes whose subdomain meets no IB window all have the same
-// operator (the grid is uniform and periodic): one shared inverse per level serves them.  Subdomains
-// up to RAS_EMAX_SMEM cells wide are eliminated in shared memory and corrected by a persistent
-// kernel; wider ones (the paper's 8 x 8 boxes with overlap 2 and up) are eliminated in a global
-// workspace and corrected by a batched product over tiles of boxes.
+// IB windows, inverted, and the owned rows of the inverse are stored (column-major, FP64 and FP32).
+// Boxes whose subdomain meets no IB window all have the same operator (the grid is uniform and
+// periodic): one shared inverse per level serves them.  Subdomains up to RAS_BE_EMAX cells wide are
+// inverted by block elimination in shared memory, wider ones (and those whose blocks are not positive
+// definite) by Gauss-Jordan with partial pivoting in a global workspace.  Subdomains up to RAS_EMAX_SMEM
+// cells wide are corrected by a persistent kernel, wider ones (the paper's 8 x 8 boxes with overlap 2
+// and up) by a batched product over tiles of boxes.
 #include <algorithm>
 
 #include "sib_internal.h"
@@ -101,145 +102,6 @@ __global__ void k_ras_classify(RasGeo G, RasIB ib, int* __restrict__ list, int* 
     }
     hit = __syncthreads_or(hit);
     if (hit && threadIdx.x == 0) list[atomicAdd(count, 1)] = k;
-}
-
-// Assembles L_k in shared memory (row-major, ne x ne), inverts it in place and stores the owned rows
-// of the inverse.  Block 0 builds the shared IB-free operator (box 0 without IB terms); block s > 0
-// builds box list[s - 1] with its IB terms.  info != 0 on a zero pivot.
-__global__ void __launch_bounds__(256) k_ras_setup(RasGeo G, RasIB ib, double a0, double c, double inv_h, double dt,
-                                                  const int* __restrict__ list, double* __restrict__ inv64,
-                                                  float* __restrict__ inv32, int* __restrict__ info) {
-    extern __shared__ double smem_ras[];
-    const int n = G.ne, tid = threadIdx.x, nt = blockDim.x;
-    double* A = smem_ras;                 // n x n
-    double* colk = A + n * n;             // n
-    double* redv = colk + n;              // 32
-    int* redi = reinterpret_cast<int*>(redv + 32);   // 32
-    int* perm = redi + 32;                // n
-    const bool withIB = blockIdx.x > 0;
-    const int k = withIB ? list[blockIdx.x - 1] : 0;
-    const int I = k % G.nbs, J = k / G.nbs, m = G.N - 1;
-    const int i0 = I * G.b - G.o, j0 = J * G.b - G.o;
-    const int per = ib.tx * ib.ty;
-    for (int t = tid; t < n * n; t += nt) A[t] = 0.0;
-    __syncthreads();
-    for (int q = tid; q < n; q += nt) {   // row q of L_k
-        int comp, ii, jj;
-        ras_dof(G, q, comp, ii, jj);
-        double* row = A + (size_t)q * n;
-        if (comp < 2) {
-            row[q] = a0;
-            // couplings to dofs of the subdomain, at local coordinates taken modulo N (on small grids a
-            // neighbour or window offset can wrap around onto the far side of the same subdomain; the
-            // subdomain itself never wraps onto itself, so the local index is unique)
-            const int nb[4][2] = {{ii + 1, jj}, {ii - 1, jj}, {ii, jj + 1}, {ii, jj - 1}};
-            for (int s2 = 0; s2 < 4; ++s2) {
-                const int col = ras_index(G, comp, nb[s2][0] & m, nb[s2][1] & m);
-                if (col >= 0) row[col] -= c;
-            }
-            // G p: u(i, j) -> (p(i, j) - p(i-1, j)) / h;  v(i, j) -> (p(i, j) - p(i, j-1)) / h
-            const int pc = ras_index(G, 2, ii, jj);
-            const int pm = comp == 0 ? ras_index(G, 2, ii - 1, jj) : ras_index(G, 2, ii, jj - 1);
-            if (pc >= 0) row[pc] += inv_h;
-            if (pm >= 0) row[pm] -= inv_h;
-            if (withIB) {   // -dt B(f, g) for g of the same component in the subdomain (window offsets)
-                const int gi = (i0 + ii) & m, gj = (j0 + jj) & m;
-                const int slot = face_slot(ib, gi, gj);
-                if (slot >= 0) {
-                    const double* w = ib.win + ((size_t)(slot * 2 + comp) * WIN_SIZE) * per;
-                    const int qt = (gj % ib.ty) * ib.tx + (gi % ib.tx);
-                    for (int dj = -WR; dj <= WR; ++dj)
-                        for (int di = -WR; di <= WR; ++di) {
-                            const int col = ras_index(G, comp, (ii + di) & m, (jj + dj) & m);
-                            if (col >= 0) row[col] -= dt * w[(size_t)((dj + WR) * WD + (di + WR)) * per + qt];
-                        }
-                }
-            }
-        } else {   // -D u: -(u(i+1, j) - u(i, j) + v(i, j+1) - v(i, j)) / h
-            row[ras_index(G, 0, ii + 1, jj)] -= inv_h;
-            row[ras_index(G, 0, ii, jj)] += inv_h;
-            row[ras_index(G, 1, ii, jj + 1)] -= inv_h;
-            row[ras_index(G, 1, ii, jj)] += inv_h;
-        }
-    }
-    __syncthreads();
-    // in-place Gauss-Jordan with partial (row) pivoting: A <- (P A)^{-1}
-    const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-    for (int kk = 0; kk < n; ++kk) {
-        double best = -1.0;
-        int bi = kk;
-        for (int i = kk + tid; i < n; i += nt) {
-            const double v = fabs(A[(size_t)i * n + kk]);
-            if (v > best) {
-                best = v;
-                bi = i;
-            }
-        }
-        for (int off = 16; off > 0; off >>= 1) {
-            const double ov = __shfl_xor_sync(0xffffffffu, best, off);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-            if (ov > best || (ov == best && oi < bi)) {
-                best = ov;
-                bi = oi;
-            }
-        }
-        if (lane == 0) {
-            redv[wid] = best;
-            redi[wid] = bi;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double bv = redv[0];
-            int bx = redi[0];
-            for (int w2 = 1; w2 < nw; ++w2)
-                if (redv[w2] > bv || (redv[w2] == bv && redi[w2] < bx)) {
-                    bv = redv[w2];
-                    bx = redi[w2];
-                }
-            perm[kk] = bx;
-            if (!(bv > 0.0)) atomicExch(info, 1);
-        }
-        __syncthreads();
-        const int p = perm[kk];
-        if (p != kk)
-            for (int j = tid; j < n; j += nt) {
-                const double t = A[(size_t)kk * n + j];
-                A[(size_t)kk * n + j] = A[(size_t)p * n + j];
-                A[(size_t)p * n + j] = t;
-            }
-        __syncthreads();
-        const double piv = A[(size_t)kk * n + kk];
-        const double pinv = piv != 0.0 ? 1.0 / piv : 0.0;
-        for (int i = tid; i < n; i += nt) colk[i] = A[(size_t)i * n + kk];
-        __syncthreads();
-        for (int j = tid; j < n; j += nt) A[(size_t)kk * n + j] = (j == kk ? 1.0 : A[(size_t)kk * n + j]) * pinv;
-        __syncthreads();
-        for (int t = tid; t < n * n; t += nt) {
-            const int i = t / n, j = t - i * n;
-            if (i == kk) continue;
-            A[t] = (j == kk ? 0.0 : A[t]) - colk[i] * A[(size_t)kk * n + j];
-        }
-        __syncthreads();
-    }
-    // (P A)^{-1} P = A^{-1}: swap columns back in reverse order of the row interchanges
-    for (int kk = n - 1; kk >= 0; --kk) {
-        const int p = perm[kk];
-        if (p != kk)
-            for (int i = tid; i < n; i += nt) {
-                const double t = A[(size_t)i * n + kk];
-                A[(size_t)i * n + kk] = A[(size_t)i * n + p];
-                A[(size_t)i * n + p] = t;
-            }
-        __syncthreads();
-    }
-    // owned rows, column-major: out[q * nown + r] = A^{-1}(owned(r), q)
-    const size_t base = (size_t)blockIdx.x * n * G.nown;
-    for (int t = tid; t < n * G.nown; t += nt) {
-        const int q = t / G.nown, r = t - q * G.nown;
-        const double v = A[(size_t)ras_owned(G, r) * n + q];
-        inv64[base + t] = v;
-        inv32[base + t] = (float)v;
-    }
 }
 
 // One RAS correction: xo(owned) = x(owned) + omega (Inv_k r_k)(owned) for every box k, with r the
@@ -395,15 +257,17 @@ __global__ void k_box_slots(const int* __restrict__ list, const int* __restrict_
     if (s < *count) slotOfBox[list[s]] = s;
 }
 
-// ---- subdomains wider than RAS_EMAX_SMEM cells (e <= RAS_EMAX, ne <= 800) ----------------------
-// The local operator (up to 5 MB in FP64) no longer fits shared memory.  Each set-up block assembles
-// its matrix in a global workspace and eliminates there, with the pivot column and the scaled pivot
-// row in shared memory.  The shared-inverse correction becomes one batched product per level,
+// ---- set-up with pivoting, and subdomains wider than RAS_EMAX_SMEM cells (e <= RAS_EMAX, ne <= 800) ----
+// The local operator takes up to 5 MB in FP64.  Each set-up block assembles its matrix in a global
+// workspace and eliminates there, with the pivot column and the scaled pivot row in shared memory.  For
+// the wide subdomains the shared-inverse correction becomes one batched product per level,
 // C (nown x boxes) = Inv (nown x ne) R (ne x boxes), over tiles of boxes; the IB boxes keep one block
 // each.
 
-// Row q of L_k for the subdomain with corner cell (i0, j0), added into `row` (zeroed by the caller):
-// the same stencil and window entries as the shared-memory set-up above.
+// Row q of L_k for the subdomain with corner cell (i0, j0), added into `row` (zeroed by the caller).
+// Couplings go to dofs of the subdomain at local coordinates taken modulo N: on small grids a neighbour or
+// window offset can wrap around onto the far side of the same subdomain; the subdomain itself never wraps
+// onto itself, so the local index is unique.
 __device__ void ras_assemble_row(const RasGeo& G, const RasIB& ib, double a0, double c, double inv_h, double dt,
                                  bool withIB, int i0, int j0, int q, double* row) {
     const int m = G.N - 1, per = ib.tx * ib.ty;
@@ -443,7 +307,7 @@ __device__ void ras_assemble_row(const RasGeo& G, const RasIB& ib, double a0, do
 
 // Block b of a launch inverts matrix first + b (0: the shared IB-free operator; s > 0: the operator
 // of box list[s - 1]) in work + b ne^2 by Gauss-Jordan with partial (row) pivoting, then stores the
-// owned rows of the inverse column-major at slot first + b, as the shared-memory set-up does.
+// owned rows of the inverse column-major at slot first + b.
 constexpr int RAS_BIG_SETUP_THREADS = 512;
 __global__ void __launch_bounds__(RAS_BIG_SETUP_THREADS)
     k_ras_setup_big(RasGeo G, RasIB ib, double a0, double c, double inv_h, double dt, const int* __restrict__ list,
@@ -546,6 +410,275 @@ __global__ void __launch_bounds__(RAS_BIG_SETUP_THREADS)
         const double v = A[(size_t)ras_owned(G, r) * n + q];
         inv64[base + t] = v;
         inv32[base + t] = (float)v;
+    }
+}
+
+// ---- set-up by block elimination (subdomains up to RAS_BE_EMAX cells wide) ------------------------
+// L_k = [A G; G^T 0] with A = diag(A_u, A_v): the IB windows couple a component only to itself, and
+// -D = G^T.  As kappa >= 0, both A blocks are symmetric positive definite, and so is S = G^T A^{-1} G (G
+// has full column rank on a subdomain with all its faces), so no pivoting is needed:
+//   L_k^{-1} = [A^{-1} - W S^{-1} W^T,  W S^{-1};  S^{-1} W^T,  -S^{-1}],   W = A^{-1} G,
+// where a column of G has two entries (+1/h on the cell's left or bottom face, -1/h on the other), so
+// that W and S are differences of entries of A^{-1}.  Only the owned rows are formed.  Against the
+// elimination of the whole ne x ne matrix with partial pivoting this takes 17 M instead of 95 M FP64
+// multiply-adds for 8 x 8 boxes with overlap 2, in shared memory instead of through L2, and its error on
+// the paper's stiffest boxes is no larger (relative to the entries' maximum, thin circle, mu = 0.01,
+// gamma = 500, 64^2: 1.6e-12 against 2.9e-12).  Every kernel is bound by the FP64 pipe (two multiply-adds
+// per clock and SM).  Whole set-up of the 128^2 annulus with 8 x 8 boxes: 142 ms with the pivoted
+// elimination (35 ms a level, whatever its number of boxes), 8.7 ms so.
+// A pivot that is not positive (a block so badly conditioned that rounding takes its definiteness, or a
+// value that is not finite) raises bit 1 of *info: the caller then takes k_ras_setup_big, which pivots.
+constexpr int BE_THREADS = 256, BE_WARPS = BE_THREADS / 32;
+constexpr int BE_ROWS = 32;        // owned rows per block, four per warp
+constexpr int BE_CPL = 5;          // columns per lane
+constexpr int BE_COLS = 32 * BE_CPL;
+constexpr int BE_KC = 16;          // pressures per shared-memory chunk
+__host__ __device__ inline int be_nu(int e) { return e * (e + 1); }
+__device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
+
+// A (lower triangle, packed rows, n x n) <- -A^{-1} by symmetric sweeps: at step k, with d = 1 / A_kk and
+// v = column k, A_ij -= v_i v_j d for i, j != k, A_ik = v_i d, A_kk = -d.  Rows i and n - 1 - i are swept as
+// one row of n + 1 entries, so that the warps' lanes stay full.
+__device__ void be_sweep(double* A, double* v, double* vd, int n, int* info) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, pairs = (n + 1) / 2;
+    for (int k = 0; k < n; ++k) {
+        const double akk = A[tri(k) + k];
+        const double d = 1.0 / akk;
+        for (int i = threadIdx.x; i < n; i += BE_THREADS) {
+            const double x = i >= k ? A[tri(i) + k] : A[tri(k) + i];
+            v[i] = x;
+            vd[i] = x * d;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && !(akk > 0.0)) atomicOr(info, 2);
+        for (int p = wid; p < pairs; p += BE_WARPS) {
+            const int i1 = p, i2 = n - 1 - p;             // i1 <= i2; equal in the middle of an odd n
+            const int len = i1 == i2 ? i1 + 1 : n + 1;
+            for (int t = lane; t < len; t += 32) {
+                const int i = t <= i1 ? i1 : i2, j = t <= i1 ? t : t - i1 - 1;
+                double* a = A + tri(i) + j;
+                double x = *a - v[i] * vd[j];
+                if (i == k || j == k) x = i == j ? -d : vd[i == k ? j : i];
+                *a = x;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// A_c^{-1} of matrix first + blockIdx.x (0: the shared IB-free operator; s > 0: box list[s - 1]) for component
+// c = blockIdx.y, into its workspace [A_u^{-1} | A_v^{-1} | S^{-1}]
+__global__ void __launch_bounds__(BE_THREADS) k_ras_be_velocity(RasGeo G, RasIB ib, double a0, double cc, double dt,
+                                                               const int* __restrict__ list, int first,
+                                                               double* __restrict__ work, int* __restrict__ info) {
+    extern __shared__ double be_sm[];
+    const int n = be_nu(G.e), np = G.e * G.e, comp = blockIdx.y, m = G.N - 1, per = ib.tx * ib.ty;
+    double* A = be_sm;
+    double* v = A + (size_t)n * (n + 1) / 2;
+    double* vd = v + n;
+    const int mi = first + blockIdx.x;
+    const bool withIB = mi > 0;
+    const int k = withIB ? list[mi - 1] : 0;
+    const int i0 = (k % G.nbs) * G.b - G.o, j0 = (k / G.nbs) * G.b - G.o;
+    for (int t = threadIdx.x; t < n * (n + 1) / 2; t += BE_THREADS) A[t] = 0.0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < n; q += BE_THREADS) {   // row q up to its diagonal; neighbours modulo N as in
+        double* row = A + tri(q);                         // ras_assemble_row
+        const int wd = comp == 0 ? G.e + 1 : G.e, jj = q / wd, ii = q - jj * wd;
+        row[q] = a0;
+        auto add = [&](int ci, int cj, double x) {
+            const int col = ras_index(G, comp, ci & m, cj & m) - comp * n;
+            if (col >= 0 && col <= q) row[col] += x;
+        };
+        add(ii + 1, jj, -cc);
+        add(ii - 1, jj, -cc);
+        add(ii, jj + 1, -cc);
+        add(ii, jj - 1, -cc);
+        if (!withIB) continue;
+        const int gi = (i0 + ii) & m, gj = (j0 + jj) & m;
+        const int slot = face_slot(ib, gi, gj);
+        if (slot < 0) continue;
+        const double* w = ib.win + ((size_t)(slot * 2 + comp) * WIN_SIZE) * per + (gj % ib.ty) * ib.tx + (gi % ib.tx);
+        for (int dj = -WR; dj <= WR; ++dj)
+            for (int di = -WR; di <= WR; ++di)
+                add(ii + di, jj + dj, -dt * w[(size_t)((dj + WR) * WD + (di + WR)) * per]);
+    }
+    __syncthreads();
+    be_sweep(A, v, vd, n, info);
+    double* out = work + (size_t)blockIdx.x * (2 * (size_t)n * n + (size_t)np * np) + (size_t)comp * n * n;
+    for (int t = threadIdx.x; t < n * n; t += BE_THREADS) {
+        const int i = t / n, j = t - i * n;
+        out[t] = -(i >= j ? A[tri(i) + j] : A[tri(j) + i]);
+    }
+}
+
+// faces of cell q of the subdomain in component c: the one with +1/h in G's column q, then the one with -1/h
+__device__ __forceinline__ void be_faces(int e, int c, int q, int& f1, int& f2) {
+    const int jj = q / e, ii = q - jj * e;
+    f1 = c == 0 ? jj * (e + 1) + ii : q;
+    f2 = c == 0 ? f1 + 1 : f1 + e;
+}
+
+// S^{-1} of matrix blockIdx.x from its A^{-1}
+__global__ void __launch_bounds__(BE_THREADS) k_ras_be_pressure(RasGeo G, double inv_h, double* __restrict__ work,
+                                                               int* __restrict__ info) {
+    extern __shared__ double be_sm[];
+    const int n = be_nu(G.e), np = G.e * G.e;
+    double* A = be_sm;
+    double* v = A + (size_t)np * (np + 1) / 2;
+    double* vd = v + np;
+    double* wk = work + (size_t)blockIdx.x * (2 * (size_t)n * n + (size_t)np * np);
+    const double ih2 = inv_h * inv_h;
+    for (int t = threadIdx.x; t < np * np; t += BE_THREADS) {
+        const int i = t / np, j = t - i * np;
+        if (j > i) continue;
+        double s = 0.0;
+        for (int c = 0; c < 2; ++c) {
+            int i1, i2, j1, j2;
+            be_faces(G.e, c, i, i1, i2);
+            be_faces(G.e, c, j, j1, j2);
+            const double* M = wk + (size_t)c * n * n;
+            s += (M[(size_t)i1 * n + j1] - M[(size_t)i1 * n + j2]) - (M[(size_t)i2 * n + j1] - M[(size_t)i2 * n + j2]);
+        }
+        A[tri(i) + j] = ih2 * s;
+    }
+    __syncthreads();
+    be_sweep(A, v, vd, np, info);
+    double* out = wk + 2 * (size_t)n * n;
+    for (int t = threadIdx.x; t < np * np; t += BE_THREADS) {
+        const int i = t / np, j = t - i * np;
+        out[t] = -(i >= j ? A[tri(i) + j] : A[tri(j) + i]);
+    }
+}
+
+// acc[a][k] = sum_c Q[row a][c] B[c][col k], c < np, for the warp's four rows (Q in shared memory, row-major) and
+// the columns lane + 32 k of a tile; B comes in chunks of BE_KC rows through `chunk`, filled by load(c, col)
+template <typename F>
+__device__ __forceinline__ void be_product(const double* Qw, int np, double* chunk, F load, double (&acc)[4][BE_CPL]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int k = 0; k < BE_CPL; ++k) acc[a][k] = 0.0;
+    for (int c0 = 0; c0 < np; c0 += BE_KC) {
+        const int kc = min(BE_KC, np - c0);
+        __syncthreads();   // the previous chunk is consumed
+        for (int t = threadIdx.x; t < kc * BE_COLS; t += BE_THREADS) chunk[t] = load(c0 + t / BE_COLS, t % BE_COLS);
+        __syncthreads();
+        for (int c = 0; c < kc; ++c) {
+            double b[BE_CPL];
+#pragma unroll
+            for (int k = 0; k < BE_CPL; ++k) b[k] = chunk[c * BE_COLS + lane + 32 * k];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const double q = Qw[(size_t)a * np + c0 + c];
+#pragma unroll
+                for (int k = 0; k < BE_CPL; ++k) acc[a][k] += q * b[k];
+            }
+        }
+    }
+}
+
+// BE_ROWS owned rows of L_k^{-1} (blockIdx.y: which) of matrix first + blockIdx.x.  For an owned velocity row
+// Q = W_own S^{-1}, for an owned pressure row Q = -S^{-1}_own; the row is [A^{-1}_own or 0] - Q W^T on the
+// velocities and Q on the pressures.  Stored column-major, as every set-up here does.
+__global__ void __launch_bounds__(BE_THREADS) k_ras_be_owned(RasGeo G, double inv_h, const double* __restrict__ work,
+                                                            int first, double* __restrict__ inv64,
+                                                            float* __restrict__ inv32) {
+    extern __shared__ double be_sm[];
+    const int n = be_nu(G.e), np = G.e * G.e, bb = G.b * G.b;
+    double* Wo = be_sm;                             // BE_ROWS x np
+    double* Q = Wo + (size_t)BE_ROWS * np;          // BE_ROWS x np
+    double* chunk = Q + (size_t)BE_ROWS * np;       // BE_KC x BE_COLS
+    const double* wk = work + (size_t)blockIdx.x * (2 * (size_t)n * n + (size_t)np * np);
+    const double* Si = wk + 2 * (size_t)n * n;
+    const int r0 = blockIdx.y * BE_ROWS, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // W_own of the velocity rows; -S^{-1}_own of the pressure rows goes straight into Q
+    for (int t = threadIdx.x; t < BE_ROWS * np; t += BE_THREADS) {
+        const int a = t / np, c = t - a * np, r = r0 + a;
+        double w = 0.0, q = 0.0;
+        if (r < G.nown) {
+            const int comp = r / bb, own = ras_owned(G, r);
+            if (comp < 2) {
+                int f1, f2;
+                be_faces(G.e, comp, c, f1, f2);
+                const double* M = wk + (size_t)comp * n * n + (own - comp * n);
+                w = inv_h * (M[(size_t)f1 * n] - M[(size_t)f2 * n]);
+            } else {
+                q = -Si[(size_t)(own - 2 * n) * np + c];
+            }
+        }
+        Wo[t] = w;
+        Q[t] = q;
+    }
+    double acc[4][BE_CPL];
+    if (r0 < 2 * bb) {   // some velocity row (uniform over the block)
+        for (int d0 = 0; d0 < np; d0 += BE_COLS) {
+            be_product(Wo + (size_t)(4 * wid) * np, np, chunk,
+                       [&](int c, int col) { return d0 + col < np ? Si[(size_t)c * np + d0 + col] : 0.0; }, acc);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                if (r0 + 4 * wid + a >= 2 * bb) continue;
+#pragma unroll
+                for (int k = 0; k < BE_CPL; ++k)
+                    if (d0 + lane + 32 * k < np) Q[(size_t)(4 * wid + a) * np + d0 + lane + 32 * k] = acc[a][k];
+            }
+        }
+    }
+    __syncthreads();
+    const int rw = r0 + 4 * wid;   // the warp's first owned row
+    const size_t base = (size_t)(first + blockIdx.x) * G.ne * G.nown;
+    auto store = [&](int q, const double (&val)[4]) {   // column q of the warp's rows
+        const size_t at = base + (size_t)q * G.nown + rw;
+        if ((G.nown & 3) == 0) {   // b > 1: 16-byte stores (base and rw are multiples of 4)
+            if (rw >= G.nown) return;
+            *reinterpret_cast<double2*>(inv64 + at) = make_double2(val[0], val[1]);
+            *reinterpret_cast<double2*>(inv64 + at + 2) = make_double2(val[2], val[3]);
+            *reinterpret_cast<float4*>(inv32 + at) =
+                make_float4((float)val[0], (float)val[1], (float)val[2], (float)val[3]);
+            return;
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            if (rw + a < G.nown) {
+                inv64[at + a] = val[a];
+                inv32[at + a] = (float)val[a];
+            }
+    };
+    for (int q0 = 0; q0 < 2 * n; q0 += BE_COLS) {   // velocity columns
+        be_product(Q + (size_t)(4 * wid) * np, np, chunk,
+                   [&](int c, int col) {
+                       const int q = q0 + col;
+                       if (q >= 2 * n) return 0.0;
+                       const int comp = q >= n ? 1 : 0;
+                       int f1, f2;
+                       be_faces(G.e, comp, c, f1, f2);
+                       const double* M = wk + (size_t)comp * n * n + (q - comp * n);
+                       return inv_h * (M[(size_t)f1 * n] - M[(size_t)f2 * n]);
+                   },
+                   acc);
+#pragma unroll
+        for (int k = 0; k < BE_CPL; ++k) {
+            const int q = q0 + lane + 32 * k;
+            if (q >= 2 * n) continue;
+            const int cq = q >= n ? 1 : 0;
+            double val[4];
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const int r = rw + a;
+                const double ai = (r < G.nown && r / bb == cq)
+                                      ? wk[(size_t)cq * n * n + (size_t)(ras_owned(G, r) - cq * n) * n + (q - cq * n)]
+                                      : 0.0;
+                val[a] = ai - acc[a][k];
+            }
+            store(q, val);
+        }
+    }
+    for (int q = lane; q < np; q += 32) {   // pressure columns: Q itself
+        double val[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) val[a] = Q[(size_t)(4 * wid + a) * np + q];
+        store(2 * n + q, val);
     }
 }
 
@@ -1590,10 +1723,6 @@ __global__ void k_ras_tc_pack_rows(RasGeo G, const double* __restrict__ inv0, in
 
 bool ras_big(int b, int o) { return b + 2 * o > RAS_EMAX_SMEM; }
 
-size_t ras_setup_smem(int b, int o) {
-    const RasGeo G = ras_geo(16, b, o);
-    return sizeof(double) * ((size_t)G.ne * G.ne + G.ne + 32) + sizeof(int) * (32 + G.ne);
-}
 int ras_ne(int b, int o) { return ras_geo(16, b, o).ne; }
 
 void launch_ras_classify(int N, int b, int o, const RasIB& ib, int* list, int* count, cudaStream_t s) {
@@ -1608,12 +1737,25 @@ void launch_box_slots(int nboxes, const int* list, const int* count, int* slotOf
     k_box_slots<<<(nboxes + 255) / 256, 256, 0, s>>>(list, count, slotOfBox);
 }
 
-void launch_ras_setup(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
-                      const int* list, int nIB, double* inv64, float* inv32, int* info, cudaStream_t s) {
+bool ras_block_elimination(int b, int o) { return b + 2 * o <= RAS_BE_EMAX; }
+size_t ras_be_work(int b, int o) {
+    const size_t nu = be_nu(ras_geo(16, b, o).e), np = (size_t)(b + 2 * o) * (b + 2 * o);
+    return 2 * nu * nu + np * np;
+}
+void launch_ras_setup_be(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
+                         const int* list, int first, int count, double* work, double* inv64, float* inv32, int* info,
+                         cudaStream_t s) {
     const RasGeo G = ras_geo(N, b, o);
-    const size_t smem = ras_setup_smem(b, o);
-    cudaFuncSetAttribute(k_ras_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_ras_setup<<<1 + nIB, 256, smem, s>>>(G, ib, a0, c, inv_h, dt, list, inv64, inv32, info);
+    const size_t nu = be_nu(G.e), np = (size_t)G.e * G.e;
+    const size_t sv = sizeof(double) * (nu * (nu + 1) / 2 + 2 * nu), sp = sizeof(double) * (np * (np + 1) / 2 + 2 * np);
+    const size_t so = sizeof(double) * (2 * BE_ROWS * np + (size_t)BE_KC * BE_COLS);
+    cudaFuncSetAttribute(k_ras_be_velocity, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv);
+    cudaFuncSetAttribute(k_ras_be_pressure, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp);
+    cudaFuncSetAttribute(k_ras_be_owned, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)so);
+    k_ras_be_velocity<<<dim3(count, 2), BE_THREADS, sv, s>>>(G, ib, a0, c, dt, list, first, work, info);
+    k_ras_be_pressure<<<count, BE_THREADS, sp, s>>>(G, inv_h, work, info);
+    k_ras_be_owned<<<dim3(count, (G.nown + BE_ROWS - 1) / BE_ROWS), BE_THREADS, so, s>>>(G, inv_h, work, first, inv64,
+                                                                                         inv32);
 }
 
 void launch_ras_setup_big(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,

@@ -1072,8 +1072,8 @@ void power_M_enqueue(sib_ctx* c, int l, int slot, double* part, cudaStream_t s) 
 
 // Box RAS set-up on levels 1..lmax (Sec. 3.3, Alg. 2 with boxes): classify the boxes by whether
 // their subdomain meets an IB window, then assemble and invert the shared IB-free subdomain operator
-// and one per IB box (FP64), keeping the owned rows of each inverse.  Wide subdomains are eliminated
-// in a temporary global workspace, at most RAS_WORK_BYTES of matrices per launch.
+// and one per IB box (FP64), keeping the owned rows of each inverse, in a temporary workspace of at most
+// RAS_WORK_BYTES.
 constexpr size_t RAS_WORK_BYTES = size_t(1) << 31;
 // The RAS reading on a level too small for the boxes (b does not divide N_l, or a subdomain's b + 2o + 1
 // face columns would wrap onto themselves): the box clipped to the periodic level is the whole level, and
@@ -1186,12 +1186,58 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     c->launches += 3;
 }
 
+// The owned rows of every box inverse of the levels that take boxes: by block elimination (be), the levels
+// side by side on the per-level streams (a level's boxes may be far fewer than the GPU's SMs), or with
+// pivoting, one level after another.  The matrices of a launch take at most RAS_WORK_BYTES of workspace
+// over all levels.  Returns the information word (0: done).
+int ras_invert(sib_ctx* c, const std::vector<int>& cnt, bool be, std::vector<void*>& tmp, cudaStream_t s) {
+    const int b = c->opts.box, o = c->opts.box_overlap;
+    const size_t matWords = be ? ras_be_work(b, o) : (size_t)ras_ne(b, o) * ras_ne(b, o);
+    const size_t most = std::max<size_t>(1, RAS_WORK_BYTES / (sizeof(double) * matWords) / (be ? c->lmax : 1));
+    size_t need = 0;   // matrices of workspace: every level its own (be), or the largest level's
+    for (int l = 1; l <= c->lmax; ++l) {
+        if (c->L[l].rasExact) continue;
+        const size_t n = std::min<size_t>(most, 1 + (size_t)cnt[l]);
+        need = be ? need + n : std::max(need, n);
+    }
+    double* work = (double*)dalloc(c, sizeof(double) * matWords * std::max<size_t>(1, need));
+    tmp.push_back(work);
+    CK(cudaMemsetAsync(c->rasInfo, 0, sizeof(int), s));
+    CK(cudaEventRecord(c->evFork, s));
+    double* wk = work;
+    for (int l = 1; l <= c->lmax; ++l) {
+        Level& lv = c->L[l];
+        if (lv.rasExact) continue;
+        const RasIB ib{c->haveIB ? lv.slotOf : nullptr, (const double*)lv.win[0], lv.tx, lv.ty, lv.ntx};
+        const double h = lv.h, a0 = c->rho / c->dt + 4.0 * c->mu / (h * h), cc = c->mu / (h * h);
+        const int total = 1 + cnt[l], batch = (int)std::min<size_t>(most, (size_t)total);
+        const bool own = be && l < sib_ctx::LVS && c->lvStream[l];
+        cudaStream_t ls = own ? c->lvStream[l] : s;
+        if (own) CK(cudaStreamWaitEvent(ls, c->evFork, 0));
+        for (int first = 0; first < total; first += batch) {
+            const int count = std::min(batch, total - first);
+            auto launch = be ? launch_ras_setup_be : launch_ras_setup_big;
+            launch(lv.N, b, o, ib, a0, cc, 1.0 / h, c->dt, lv.rasList, first, count, wk, (double*)lv.rasInv[0],
+                   (float*)lv.rasInv[1], c->rasInfo, ls);
+            c->launches += be ? 3 : 1;
+        }
+        if (own) {
+            CK(cudaEventRecord(c->lvDone[l], ls));
+            CK(cudaStreamWaitEvent(s, c->lvDone[l], 0));
+        }
+        if (be) wk += matWords * batch;
+    }
+    int info = 0;
+    CK(cudaMemcpyAsync(&info, c->rasInfo, sizeof(int), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemsetAsync(c->rasInfo, 0, sizeof(int), s));
+    CK(cudaStreamSynchronize(s));
+    return info;
+}
+
 void ras_setup_all(sib_ctx* c, cudaStream_t s) {
     const int b = c->opts.box, o = c->opts.box_overlap;
     const int ne = ras_ne(b, o), nown = 3 * b * b;
     const bool huge = ras_huge(b);
-    const bool big = !huge && ras_big(b, o);
-    const size_t matBytes = sizeof(double) * (size_t)ne * ne;
     std::vector<int> cnt(c->lmax + 1, 0);
     for (int l = 1; l <= c->lmax; ++l) {
         Level& lv = c->L[l];
@@ -1219,15 +1265,6 @@ void ras_setup_all(sib_ctx* c, cudaStream_t s) {
     int* ginfo = (int*)dalloc(c, sizeof(int));
     tmp.push_back(ginfo);
     CK(cudaMemsetAsync(ginfo, 0, sizeof(int), s));
-    int batch = 0;   // wide subdomains: matrices per set-up launch
-    double* work = nullptr;
-    if (big) {
-        int most = 1;
-        for (int l = 1; l <= c->lmax; ++l) most = std::max(most, 1 + cnt[l]);
-        batch = (int)std::max<size_t>(1, std::min<size_t>((size_t)most, RAS_WORK_BYTES / matBytes));
-        work = (double*)dalloc(c, matBytes * batch);
-        tmp.push_back(work);
-    }
     for (int l = 1; l <= c->lmax; ++l) {
         Level& lv = c->L[l];
         if (lv.rasExact) {
@@ -1249,38 +1286,34 @@ void ras_setup_all(sib_ctx* c, cudaStream_t s) {
             lv.rasInv[1] = dalloc(c, sizeof(float) * ent);
             lv.rasInvCap = ent;
         }
-        const RasIB ib{c->haveIB ? lv.slotOf : nullptr, (const double*)lv.win[0], lv.tx, lv.ty, lv.ntx};
         lv.rasNIB = cnt[l];
-        const double h = lv.h, a0 = c->rho / c->dt + 4.0 * c->mu / (h * h), cc = c->mu / (h * h);
-        if (big) {
-            for (int first = 0; first < 1 + cnt[l]; first += batch) {
-                launch_ras_setup_big(lv.N, b, o, ib, a0, cc, 1.0 / h, c->dt, lv.rasList, first,
-                                     std::min(batch, 1 + cnt[l] - first), work, (double*)lv.rasInv[0],
-                                     (float*)lv.rasInv[1], c->rasInfo, s);
-                ++c->launches;
+    }
+    int info = 0;
+    if (!huge) {
+        if (ras_block_elimination(b, o)) info = ras_invert(c, cnt, true, tmp, s);
+        // pivoting: wide subdomains, and (bit 1) blocks that lost their definiteness to rounding
+        if (!ras_block_elimination(b, o) || (info & 2)) info = ras_invert(c, cnt, false, tmp, s);
+        for (int l = 1; l <= c->lmax; ++l) {
+            Level& lv = c->L[l];
+            if (lv.rasExact) continue;
+            // the shared inverse (slot 0) packed for the tensor-core correction of FP32 levels
+            const size_t pf = ras_tc_pack_floats(b, o);
+            if (pf > lv.rasTCCap) {
+                dfree(c, lv.rasTC);
+                lv.rasTC = (float*)dalloc(c, sizeof(float) * pf);
+                lv.rasTCCap = pf;
             }
-        } else {
-            launch_ras_setup(lv.N, b, o, ib, a0, cc, 1.0 / h, c->dt, lv.rasList, cnt[l], (double*)lv.rasInv[0],
-                             (float*)lv.rasInv[1], c->rasInfo, s);
+            launch_ras_tc_pack(b, o, (const double*)lv.rasInv[0], lv.rasTC, s);
             ++c->launches;
         }
-        // the shared inverse (slot 0) packed for the tensor-core correction of FP32 levels
-        const size_t pf = ras_tc_pack_floats(b, o);
-        if (pf > lv.rasTCCap) {
-            dfree(c, lv.rasTC);
-            lv.rasTC = (float*)dalloc(c, sizeof(float) * pf);
-            lv.rasTCCap = pf;
-        }
-        launch_ras_tc_pack(b, o, (const double*)lv.rasInv[0], lv.rasTC, s);
-        ++c->launches;
     }
-    int info = 0, gj = 0;
-    CK(cudaMemcpyAsync(&info, c->rasInfo, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int gj = 0, wb = 0;
+    CK(cudaMemcpyAsync(&wb, c->rasInfo, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaMemcpyAsync(&gj, ginfo, sizeof(int), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     for (void* p : tmp) dfree(c, p);
     kcheck(c);
-    if (info != 0 || gj != 0) throw SibError(SIB_ERR_ARG, "a box subdomain operator is singular");
+    if (info != 0 || wb != 0 || gj != 0) throw SibError(SIB_ERR_ARG, "a box subdomain operator is singular");
 }
 
 void setup(sib_ctx* c, cudaStream_t s) {

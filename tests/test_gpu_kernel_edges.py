@@ -5,14 +5,13 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from oracle import ib  # noqa: E402
+from oracle import ib, multigrid  # noqa: E402
+from paper_1612_02208_gb300 import inputs as I  # noqa: E402
 from paper_1612_02208_gb300 import sib  # noqa: E402
 
+from tests.test_gpu_parity import TOL64, cu, host, rand, rel  # noqa: E402
+
 EPS = 2.0 ** -53
-
-
-def cu(x):
-    return torch.as_tensor(np.ascontiguousarray(x), device="cuda")
 
 
 # grids below, at and above one 32 x 8 tile; single markers; a cell that holds every marker; markers
@@ -31,7 +30,7 @@ def test_spread_tiles(N, M, where):
     F = rng.standard_normal((M, 2))
     edges = np.array([[0, M - 1]], dtype=np.int32)
     S = sib.Solver(N, n_min=4)
-    S.set_structure(cu(X), cu(edges), cu(np.array([1.0])))
+    S.set_structure(cu(X), torch.as_tensor(edges, device="cuda"), cu(np.array([1.0])))
     S.setup()
     f = S.spread(cu(F)).cpu().numpy()
     ref = ib.spread_force(N, X, F)
@@ -41,4 +40,23 @@ def test_spread_tiles(N, M, where):
     tol = (2 * M + 8) * EPS * mag + 64 * EPS * N * N * np.abs(F).max()
     assert (np.abs(f - ref) <= tol).all(), np.abs(f - ref).max()
     assert torch.equal(S.spread(cu(F)), S.spread(cu(F)))
+    S.close()
+
+
+# Box set-up by block elimination: one cell, one face row more than the box, ragged row tiles (12, 48 and
+# 192 owned rows in tiles of 32), the widest subdomain it takes (14 cells) and subdomains whose faces wrap
+# around a small level.  One FP64 sweep per level to the repository's FP64 bar.
+@pytest.mark.parametrize("b,o,N,kappa", [(1, 0, 32, 1e2), (1, 2, 32, 1e2), (2, 6, 32, 1e2), (4, 5, 32, 1e4), (8, 3, 32, 1e2),
+                                         (4, 1, 16, 1e4)])
+def test_box_inverses(b, o, N, kappa):
+    prob = I.thin_ellipse_stokes(N, kappa=kappa)
+    H = multigrid.Hierarchy(prob, smoother="ras", box=b, overlap=o)
+    S = sib.solver_for(prob, smoother=sib.SMOOTHER_RAS, box=b, box_overlap=o)
+    for l in range(1, len(H.levels)):
+        n3 = 3 * H.levels[l].n
+        x, rhs = rand(n3, 7000 + l), rand(n3, 7100 + l, 10.0)
+        y = cu(x.copy())
+        S.smooth(l, y, cu(rhs), 1)
+        ref = H.smooth(l, x, rhs, 1)
+        assert rel(host(y), ref) < TOL64, (l, rel(host(y), ref))
     S.close()
