@@ -107,7 +107,7 @@ __global__ void k_ras_classify(RasGeo G, RasIB ib, int* __restrict__ list, int* 
 // One RAS correction: xo(owned) = x(owned) + omega (Inv_k r_k)(owned) for every box k, with r the
 // residual (x == nullptr: zero initial guess, xo = omega Inv r).  The boxes without IB terms
 // (slotOfBox[k] < 0) share one inverse, staged once per block in shared memory (k_ras_apply); the
-// others, listed at set-up, use their own (k_ras_apply_ib, one block per box).
+// others, listed at set-up, use their own (k_ras_apply_split).
 // Every warp takes groups of RAS_GB consecutive boxes (grid-stride over the groups):
 // the group's residuals are gathered into shared memory as [q][box], and lane l accumulates owned
 // rows l and l + 32 for all boxes of the group, so one read of an inverse entry serves RAS_GB boxes.
@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(32 * RAS_WARPS) k_ras_apply(RasGeo G, const in
         T acc0[RAS_GB], acc1[RAS_GB];
 #pragma unroll
         for (int j = 0; j < RAS_GB; ++j) acc0[j] = acc1[j] = T(0);
-        {   // the shared inverse for the whole group (boxes with their own are stored by k_ras_apply_ib)
+        {   // the shared inverse for the whole group (boxes with their own are stored by k_ras_apply_split)
             const int c0 = r0 < G.nown ? r0 : 0, c1 = r1 < G.nown ? r1 : 0;   // rows past nown compute, unused
             const Quad<T>* rq = reinterpret_cast<const Quad<T>*>(rb);
 #pragma unroll 8
@@ -209,46 +209,6 @@ __global__ void __launch_bounds__(32 * RAS_WARPS) k_ras_apply(RasGeo G, const in
             }
         }
         __syncwarp();   // the group's residual buffer is reused by the next group
-    }
-}
-
-// One block per listed IB box: RAS_QS groups of threads each take a quarter of the q range for every
-// owned row, and the partial sums are added in shared memory in a fixed order.
-constexpr int RAS_QS = 4;
-template <typename T>
-__global__ void __launch_bounds__(64 * RAS_QS) k_ras_apply_ib(RasGeo G, const int* __restrict__ list,
-                                                             const T* __restrict__ inv, T omega,
-                                                             const T* __restrict__ r, const T* x, T* xo) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T* rb = reinterpret_cast<T*>(smem_raw);   // ne
-    T* part = rb + G.ne;                      // RAS_QS x 64
-    const int s = blockIdx.x, k = list[s];    // set-up data
-    pdl_entry();
-    const int I = k % G.nbs, J = k / G.nbs, N = G.N, n = N * N, m = N - 1, bb = G.b * G.b;
-    const int i0 = I * G.b - G.o, j0 = J * G.b - G.o;
-    for (int q = threadIdx.x; q < G.ne; q += blockDim.x) {
-        int comp, ii, jj;
-        ras_dof(G, q, comp, ii, jj);
-        rb[q] = r[(size_t)comp * n + ((j0 + jj) & m) * N + ((i0 + ii) & m)];
-    }
-    __syncthreads();
-    const T* M = inv + (size_t)(s + 1) * G.ne * G.nown;
-    const int rr = threadIdx.x & 63, part_id = threadIdx.x >> 6;
-    const int qchunk = (G.ne + RAS_QS - 1) / RAS_QS;
-    const int qa = part_id * qchunk, qb = min(G.ne, qa + qchunk);
-    T acc = T(0);
-    if (rr < G.nown) {
-#pragma unroll 6
-        for (int q = qa; q < qb; ++q) acc += M[(size_t)q * G.nown + rr] * rb[q];
-    }
-    part[part_id * 64 + rr] = acc;
-    __syncthreads();
-    if (part_id == 0 && rr < G.nown) {
-        T sum = part[rr];
-        for (int p2 = 1; p2 < RAS_QS; ++p2) sum += part[p2 * 64 + rr];
-        const int comp = rr / bb, rem = rr - comp * bb;
-        const size_t d = (size_t)comp * n + (J * G.b + rem / G.b) * N + I * G.b + rem % G.b;
-        xo[d] = (x ? x[d] : T(0)) + omega * sum;
     }
 }
 
@@ -682,7 +642,7 @@ __global__ void __launch_bounds__(BE_THREADS) k_ras_be_owned(RasGeo G, double in
     }
 }
 
-// Batched shared-inverse correction.  A block takes a tile of RAS_NBX consecutive boxes and all their
+// Batched shared-inverse correction (FP32 levels above 128^2 without the tensor cores).  A block takes a tile of RAS_NBX consecutive boxes and all their
 // owned rows; the subdomain dofs q are taken in chunks of RAS_KC: the chunk of the inverse (rows
 // [q][row], contiguous in memory) is copied to shared memory asynchronously while the chunk of the
 // tile's residual windows is gathered, then warp w accumulates the owned rows lane + 32 a (a < RA)
@@ -703,21 +663,12 @@ template <>
 struct Vec16<float> {
     using type = float4;
 };
-template <>
-struct Vec16<double> {
-    using type = double2;
-};
 template <typename T>
 __device__ __forceinline__ T vget(const typename Vec16<T>::type& v, int c);
 template <>
 __device__ __forceinline__ float vget<float>(const float4& v, int c) {
     return c == 0 ? v.x : c == 1 ? v.y : c == 2 ? v.z : v.w;
 }
-template <>
-__device__ __forceinline__ double vget<double>(const double2& v, int c) {
-    return c == 0 ? v.x : v.y;
-}
-
 template <typename T, int RA>
 __global__ void __launch_bounds__(32 * RAS_BW) k_ras_apply_big(RasGeo G, const int* __restrict__ slotOfBox,
                                                               const T* __restrict__ inv, T omega,
@@ -808,7 +759,7 @@ __global__ void __launch_bounds__(32 * RAS_BW) k_ras_apply_big(RasGeo G, const i
 #pragma unroll
     for (int c2 = 0; c2 < TL::BPT; ++c2) {
         const int kb = k0 + warp * TL::BPT + c2;
-        if (kb >= nboxes || (slotOfBox && slotOfBox[kb] >= 0)) continue;   // IB boxes: k_ras_apply_big_ib
+        if (kb >= nboxes || (slotOfBox && slotOfBox[kb] >= 0)) continue;   // IB boxes: k_ras_apply_split
         const int I = kb % G.nbs, J = kb / G.nbs;
 #pragma unroll
         for (int a = 0; a < RA; ++a) {
@@ -821,42 +772,132 @@ __global__ void __launch_bounds__(32 * RAS_BW) k_ras_apply_big(RasGeo G, const i
     }
 }
 
-// One block per listed IB box with a subdomain wider than RAS_EMAX_SMEM: four groups of 64 threads
-// each take a quarter of the q range for the owned rows lane64, lane64 + 64, ...; the partial sums
-// are added in shared memory in a fixed order.
-template <typename T>
-__global__ void __launch_bounds__(256) k_ras_apply_big_ib(RasGeo G, const int* __restrict__ list,
-                                                         const T* __restrict__ inv, T omega,
-                                                         const T* __restrict__ r, const T* x, T* xo) {
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    T* rb = reinterpret_cast<T*>(smem_raw);   // ne
-    T* part = rb + G.ne;                      // 4 x nown
-    const int s = blockIdx.x, k = list[s];    // set-up data
+// ---- the IB boxes, and on levels of few boxes every box, in one launch ----------------------------
+// A block takes RC owned rows of one IB box (its own inverse) or of NB consecutive boxes that share the
+// IB-free inverse; thread (row, ks) sums its row over the ks-th part of the subdomain dofs.  Such levels are
+// bound by latency: the tensor-core and tiled forms give a tile of 64 or 128 boxes to one SM, which then
+// walks all ne dofs (128^2, 8 x 8 boxes: two SMs, 31 us), and one block per IB box leaves the reads of its
+// inverse (350 KB) to a single SM.  Here both spread over (boxes, rows), and a thread's inverse entries,
+// which are set-up data, are requested RAS_SP_U at a time ahead of their use, the first before the
+// dependency wait (8 x 8 boxes at 128^2: 86 -> 11.6 us a correction; the choice of form is in
+// launch_ras_apply).  Sums are formed over RAS_SP_U terms, then over a thread's chunks, then over ks: the
+// blocked summation keeps the FP32 rounding of the cancelling terms low.
+constexpr int RAS_SP_T = 256, RAS_SP_U = 16, RAS_SP_NB = 8;
+struct RasSplit {
+    int threads, rc, ks, chunks, qlen;   // threads and rows a block, dof parts, blocks a box group, dofs a part
+};
+// Rows a block: every owned row of 1 x 1 and 2 x 2 boxes, 16 of a 4 x 4 box's 48, 32 of an 8 x 8 box's 192.  The
+// narrow IB boxes of a large level (on their own) are bound by the blocks' rate, not by one block's latency:
+// blocks of half the threads with every owned row (annulus at 512^2, 4 x 4 boxes, FP32: 50 -> 26 us).
+inline RasSplit ras_split(const RasGeo& G, bool own) {
+    RasSplit p;
+    p.rc = G.nown <= 12 ? G.nown : (G.nown <= 48 ? 16 : 32);
+    p.threads = RAS_SP_T;
+    if (G.nown <= 48 && own) {
+        p.rc = G.nown;
+        p.threads = RAS_SP_T / 2;
+    }
+    p.ks = p.threads / p.rc;
+    p.chunks = (G.nown + p.rc - 1) / p.rc;
+    p.qlen = (G.ne + p.ks - 1) / p.ks;
+    return p;
+}
+template <typename T, int NB>
+__device__ void ras_split_body(const RasGeo& G, const RasSplit& p, int ch, const int (&box)[NB],
+                               const T* __restrict__ M, T omega, const T* __restrict__ r, const T* x, T* xo,
+                               unsigned char* smem) {
+    T* rb = reinterpret_cast<T*>(smem);            // ne x NB
+    T* part = rb + (size_t)G.ne * NB;              // ks x rc x NB
+    const int N = G.N, n = N * N, m = N - 1, bb = G.b * G.b, tid = threadIdx.x;
+    const int ks = tid / p.rc, lr = tid - ks * p.rc, row = ch * p.rc + lr;
+    const int qa = min(G.ne, ks * p.qlen), qb = min(G.ne, qa + p.qlen);
+    const bool live = ks < p.ks && row < G.nown;
+    T mv[RAS_SP_U];
+    auto fetch = [&](int q0) {
+#pragma unroll
+        for (int u = 0; u < RAS_SP_U; ++u) mv[u] = (live && q0 + u < qb) ? M[(size_t)(q0 + u) * G.nown + row] : T(0);
+    };
+    fetch(qa);
     pdl_entry();
-    const int I = k % G.nbs, J = k / G.nbs, N = G.N, n = N * N, m = N - 1, bb = G.b * G.b, nown = G.nown;
-    const int i0 = I * G.b - G.o, j0 = J * G.b - G.o;
-    for (int q = threadIdx.x; q < G.ne; q += blockDim.x) {
+    int i0[NB], j0[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) {
+        const int k = max(box[j], 0);   // a box without this correction: any residuals, its sums are not stored
+        i0[j] = (k % G.nbs) * G.b - G.o;
+        j0[j] = (k / G.nbs) * G.b - G.o;
+    }
+    for (int q = tid; q < G.ne; q += p.threads) {
         int comp, ii, jj;
         ras_dof(G, q, comp, ii, jj);
-        rb[q] = r[(size_t)comp * n + (size_t)((j0 + jj) & m) * N + ((i0 + ii) & m)];
+        const T* rc = r + (size_t)comp * n;
+        T g[NB];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) g[j] = rc[(size_t)((j0[j] + jj) & m) * N + ((i0[j] + ii) & m)];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) rb[q * NB + j] = g[j];
     }
     __syncthreads();
-    const T* M = inv + (size_t)(s + 1) * G.ne * nown;
-    const int lr = threadIdx.x & 63, part_id = threadIdx.x >> 6;
-    const int qchunk = (G.ne + 3) / 4;
-    const int qa = part_id * qchunk, qb = min(G.ne, qa + qchunk);
-    for (int rr = lr; rr < nown; rr += 64) {
-        T acc = T(0);
-#pragma unroll 4
-        for (int q = qa; q < qb; ++q) acc += M[(size_t)q * nown + rr] * rb[q];
-        part[part_id * nown + rr] = acc;
+    T tot[NB];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) tot[j] = T(0);
+    for (int q0 = qa; q0 < qb; q0 += RAS_SP_U) {
+        T cur[RAS_SP_U];
+#pragma unroll
+        for (int u = 0; u < RAS_SP_U; ++u) cur[u] = mv[u];
+        fetch(q0 + RAS_SP_U);
+        T acc[NB];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) acc[j] = T(0);
+#pragma unroll
+        for (int u = 0; u < RAS_SP_U; ++u) {
+            if (q0 + u >= qb) break;
+#pragma unroll
+            for (int j = 0; j < NB; ++j) acc[j] += cur[u] * rb[(q0 + u) * NB + j];
+        }
+#pragma unroll
+        for (int j = 0; j < NB; ++j) tot[j] += acc[j];
     }
+    if (ks < p.ks)
+#pragma unroll
+        for (int j = 0; j < NB; ++j) part[(ks * p.rc + lr) * NB + j] = tot[j];
     __syncthreads();
-    for (int rr = threadIdx.x; rr < nown; rr += blockDim.x) {
-        const T sum = ((part[rr] + part[nown + rr]) + part[2 * nown + rr]) + part[3 * nown + rr];
+    for (int t = tid; t < p.rc * NB; t += p.threads) {   // thread: box t / rc, row t % rc (rows run along x)
+        const int j = t / p.rc, q = t - j * p.rc, rr = ch * p.rc + q;
+        const int kb = box[j];
+        if (kb < 0 || rr >= G.nown) continue;
+        T sum = part[q * NB + j];
+        for (int k = 1; k < p.ks; ++k) sum += part[(k * p.rc + q) * NB + j];
         const int comp = rr / bb, rem = rr - comp * bb;
-        const size_t d = (size_t)comp * n + (size_t)(J * G.b + rem / G.b) * N + I * G.b + rem % G.b;
+        const size_t d = (size_t)comp * n + (size_t)((kb / G.nbs) * G.b + rem / G.b) * N + (kb % G.nbs) * G.b + rem % G.b;
         xo[d] = (x ? x[d] : T(0)) + omega * sum;
+    }
+}
+// blocks: the IB boxes first (their inverses come from memory), then (GROUPS) the groups of IB-free boxes
+template <typename T, bool GROUPS>
+__global__ void __launch_bounds__(RAS_SP_T) k_ras_apply_split(RasGeo G, RasSplit p, const int* __restrict__ list, int nIB,
+                                                             const int* __restrict__ slotOfBox,
+                                                             const T* __restrict__ inv, T omega,
+                                                             const T* __restrict__ r, const T* x, T* xo) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int item = blockIdx.x / p.chunks, ch = blockIdx.x - item * p.chunks;
+    if (item < nIB) {
+        const int box[1] = {list[item]};
+        ras_split_body<T, 1>(G, p, ch, box, inv + (size_t)(item + 1) * G.ne * G.nown, omega, r, x, xo, smem_raw);
+        return;
+    }
+    if constexpr (GROUPS) {
+        int box[RAS_SP_NB];
+        bool any = false;
+#pragma unroll
+        for (int j = 0; j < RAS_SP_NB; ++j) {
+            const int k = (item - nIB) * RAS_SP_NB + j;
+            box[j] = k < G.nbs * G.nbs && !(slotOfBox && slotOfBox[k] >= 0) ? k : -1;
+            any |= box[j] >= 0;
+        }
+        if (any)
+            ras_split_body<T, RAS_SP_NB>(G, p, ch, box, inv, omega, r, x, xo, smem_raw);
+        else
+            pdl_entry();
     }
 }
 
@@ -2091,59 +2132,71 @@ bool launch_ras_apply_tc_groups(int N, int b, int o, const float* pack, int grou
 }
 
 template <typename T>
-void launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list, int nIB, const T* inv, T omega,
-                      const T* r, const T* x, T* xo, cudaStream_t s, const float* tcPack, int* err) {
+int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list, int nIB, const T* inv, T omega,
+                     const T* r, const T* x, T* xo, cudaStream_t s, const float* tcPack, int* err) {
     const RasGeo G = ras_geo(N, b, o);
+    auto split = [&](int ngroups) {
+        const RasSplit p = ras_split(G, ngroups == 0);
+        const int nb = ngroups > 0 ? RAS_SP_NB : 1;
+        const size_t smem = sizeof(T) * nb * ((size_t)G.ne + (size_t)p.ks * p.rc);
+        auto kern = ngroups > 0 ? k_ras_apply_split<T, true> : k_ras_apply_split<T, false>;
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        launch_pdl(kern, dim3((nIB + ngroups) * p.chunks), dim3(p.threads), smem, s, G, p, list, nIB,
+                   slotOfBox, inv, omega, r, x, xo);
+    };
+    // Which form (us per correction, thin circle, the other forms with one block per IB box / all boxes split):
+    //   FP32  4x4 o1: 64^2 14.5 / 4.8, 128^2 13.8 / 8.0, 256^2 14.8 / 17.1, 512^2 19.6 / 53.9
+    //         2x2 o2: 64^2 13.2 / 4.7, 128^2 14.9 / 8.9, 256^2 16.8 / 21.4, 512^2 41.2 / 67.2
+    //         8x8 o2: 64^2 77 / 7.8, 128^2 87 / 11.6, 256^2 79 / 27.8, 512^2 154 / 79, 1024^2 165 / 272
+    //   FP64  4x4 o1: 64^2 45 / 12, 128^2 45 / 24, 256^2 73 / 72, 512^2 262 / 252, 1024^2 858 / 987
+    //         2x2 o2: 256^2 258 / 88, 512^2 879 / 310;  8x8 o2: 256^2 825 / 219, 1024^2 2998 / 2692
+    // FP32 levels above 128^2 fill the GPU with tiles of boxes; FP64 is bound by the FP64 pipe in either form,
+    // and the persistent kernel's staged inverse pays only where its 64 lanes of owned rows are filled.
+    const bool all = sizeof(T) == 4 ? N <= 128 : !(G.e <= RAS_EMAX_SMEM && G.nown >= 32 && N > 256);
+    if (all) {
+        split((G.nbs * G.nbs + RAS_SP_NB - 1) / RAS_SP_NB);
+        return 1;
+    }
+    bool done = false;
     if constexpr (sizeof(T) == 4) {
-        // IB-free boxes on the tensor cores, IB boxes by their own inverses
-        if (tcPack && launch_ras_apply_tc(N, b, o, slotOfBox, tcPack, omega, r, x, xo, err, s)) {
-            if (nIB > 0) {
-                if (G.e > RAS_EMAX_SMEM)
-                    launch_pdl(k_ras_apply_big_ib<T>, dim3(nIB), dim3(256), sizeof(T) * ((size_t)G.ne + 4 * (size_t)G.nown),
-                               s, G, list, inv, omega, r, x, xo);
-                else
-                    launch_pdl(k_ras_apply_ib<T>, dim3(nIB), dim3(64 * RAS_QS), sizeof(T) * (G.ne + 64 * RAS_QS), s, G, list,
-                               inv, omega, r, x, xo);
-            }
-            return;
+        // IB-free boxes on the tensor cores, or as tiles of boxes on the CUDA cores
+        done = tcPack && launch_ras_apply_tc(N, b, o, slotOfBox, tcPack, omega, r, x, xo, err, s);
+        if (!done && G.e > RAS_EMAX_SMEM) {   // rows per lane: nown <= 32 RA
+            if (G.nown <= 32)
+                launch_ras_apply_big<T, 1>(G, slotOfBox, inv, omega, r, x, xo, s);
+            else if (G.nown <= 64)
+                launch_ras_apply_big<T, 2>(G, slotOfBox, inv, omega, r, x, xo, s);
+            else
+                launch_ras_apply_big<T, 6>(G, slotOfBox, inv, omega, r, x, xo, s);
+            done = true;
         }
     }
-    if (G.e > RAS_EMAX_SMEM) {   // rows per lane: nown <= 32 RA
-        if (G.nown <= 32)
-            launch_ras_apply_big<T, 1>(G, slotOfBox, inv, omega, r, x, xo, s);
-        else if (G.nown <= 64)
-            launch_ras_apply_big<T, 2>(G, slotOfBox, inv, omega, r, x, xo, s);
-        else
-            launch_ras_apply_big<T, 6>(G, slotOfBox, inv, omega, r, x, xo, s);
-        if (nIB > 0)
-            launch_pdl(k_ras_apply_big_ib<T>, dim3(nIB), dim3(256), sizeof(T) * ((size_t)G.ne + 4 * (size_t)G.nown), s,
-                       G, list, inv, omega, r, x, xo);
-        return;
+    if (!done) {
+        const size_t smem = sizeof(T) * (((size_t)G.ne * G.nown + 3) / 4 * 4 + (size_t)RAS_WARPS * G.ne * RAS_GB) +
+                            sizeof(int) * G.ne;
+        static thread_local size_t cachedSmem = 0;   // persistent grid: the blocks resident at once, per size
+        static thread_local int resident = 1;
+        if (smem != cachedSmem) {
+            cudaFuncSetAttribute(k_ras_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            int dev = 0, sms = 0, per = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply<T>, 32 * RAS_WARPS, smem);
+            resident = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+            cachedSmem = smem;
+        }
+        const int ngroups = G.nbs * G.nbs / RAS_GB;
+        const int want = (ngroups + RAS_WARPS - 1) / RAS_WARPS;
+        const int blocks = want < resident ? want : resident;
+        launch_pdl(k_ras_apply<T>, dim3(blocks), dim3(32 * RAS_WARPS), smem, s, G, slotOfBox, inv, omega, r, x, xo);
     }
-    const size_t smem = sizeof(T) * (((size_t)G.ne * G.nown + 3) / 4 * 4 + (size_t)RAS_WARPS * G.ne * RAS_GB) +
-                        sizeof(int) * G.ne;
-    static thread_local size_t cachedSmem = 0;   // persistent grid: the blocks resident at once, per size
-    static thread_local int resident = 1;
-    if (smem != cachedSmem) {
-        cudaFuncSetAttribute(k_ras_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int dev = 0, sms = 0, per = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_ras_apply<T>, 32 * RAS_WARPS, smem);
-        resident = (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
-        cachedSmem = smem;
-    }
-    const int ngroups = G.nbs * G.nbs / RAS_GB;
-    const int want = (ngroups + RAS_WARPS - 1) / RAS_WARPS;
-    const int blocks = want < resident ? want : resident;
-    launch_pdl(k_ras_apply<T>, dim3(blocks), dim3(32 * RAS_WARPS), smem, s, G, slotOfBox, inv, omega, r, x, xo);
-    if (nIB > 0)
-        launch_pdl(k_ras_apply_ib<T>, dim3(nIB), dim3(64 * RAS_QS), sizeof(T) * (G.ne + 64 * RAS_QS), s, G, list, inv,
-                   omega, r, x, xo);
+    if (nIB == 0) return 1;
+    split(0);   // the IB boxes
+    return 2;
 }
-template void launch_ras_apply<float>(int, int, int, const int*, const int*, int, const float*, float, const float*,
+template int launch_ras_apply<float>(int, int, int, const int*, const int*, int, const float*, float, const float*,
                                       const float*, float*, cudaStream_t, const float*, int*);
-template void launch_ras_apply<double>(int, int, int, const int*, const int*, int, const double*, double,
+template int launch_ras_apply<double>(int, int, int, const int*, const int*, int, const double*, double,
                                        const double*, const double*, double*, cudaStream_t, const float*, int*);
 
 }  // namespace sib

@@ -138,11 +138,12 @@ void launch_ras_setup_be(int N, int b, int o, const RasIB& ib, double a0, double
 void launch_ras_setup_big(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
                           const int* list, int first, int count, double* work, double* inv64, float* inv32, int* info,
                           cudaStream_t s);
-// the shared-inverse kernel, then (nIB > 0) one block per listed IB box
+// one launch for every box (levels of few boxes, FP64), or the shared-inverse kernel and then (nIB > 0) the IB
+// boxes; returns the number of launches
 // tcPack != nullptr (FP32): the IB-free boxes' correction runs on the tensor cores from the packed
 // shared inverse (launch_ras_tc_pack); err receives SIB_DEV_ERR_TMA_WAIT if one of its waits gives up
 template <typename T>
-void launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list, int nIB, const T* inv, T omega,
+int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list, int nIB, const T* inv, T omega,
                       const T* r, const T* x, T* xo, cudaStream_t s, const float* tcPack = nullptr,
                       int* err = nullptr);
 // the shared inverse (slot 0 of the FP64 inverses) packed for the tensor-core correction: hi and lo

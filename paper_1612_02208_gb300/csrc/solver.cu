@@ -588,9 +588,8 @@ void ras_apply(sib_ctx* c, int l, const T* r, const T* x, T* xo, double omega, c
         return;
     }
     const float* tc = ras_tc_pack_for<T>(c, lv);
-    KL(c, launch_ras_apply<T>(lv.N, c->opts.box, c->opts.box_overlap, lv.rasSlot, lv.rasList, lv.rasNIB,
-                              (const T*)lv.rasInv[pi], (T)omega, r, x, xo, s, tc, c->herr));
-    if (lv.rasNIB > 0) ++c->launches;
+    c->launches += launch_ras_apply<T>(lv.N, c->opts.box, c->opts.box_overlap, lv.rasSlot, lv.rasList, lv.rasNIB,
+                                       (const T*)lv.rasInv[pi], (T)omega, r, x, xo, s, tc, c->herr);
 }
 
 // one smoothing sweep xo <- smooth(x, b)

@@ -9,7 +9,7 @@ from oracle import ib, multigrid  # noqa: E402
 from paper_1612_02208_gb300 import inputs as I  # noqa: E402
 from paper_1612_02208_gb300 import sib  # noqa: E402
 
-from tests.test_gpu_parity import TOL64, cu, host, rand, rel  # noqa: E402
+from tests.test_gpu_parity import TOL32, TOL64, cu, host, rand, rel  # noqa: E402
 
 EPS = 2.0 ** -53
 
@@ -59,4 +59,27 @@ def test_box_inverses(b, o, N, kappa):
         S.smooth(l, y, cu(rhs), 1)
         ref = H.smooth(l, x, rhs, 1)
         assert rel(host(y), ref) < TOL64, (l, rel(host(y), ref))
+    S.close()
+
+
+# The tensor-core tiles of narrow boxes on a level above 128^2 (levels up to 128^2 take the split form), 64
+# and 128 boxes a row; one FP32 sweep to the repository's FP32 bar, with the CUDA-core form beside it.
+@pytest.mark.parametrize("make,b,o", [(lambda: I.thin_ellipse_re(256, kappa=1e4), 4, 1),
+                                      (lambda: I.no_structure(256, rho=1.0, seed=4), 2, 1)], ids=["4x4", "2x2"])
+def test_narrow_boxes_on_tensor_cores(make, b, o):
+    prob = make()
+    H = multigrid.Hierarchy(prob, smoother="ras", box=b, overlap=o)
+    S = sib.solver_for(prob, smoother=sib.SMOOTHER_RAS, box=b, box_overlap=o)
+    l = len(H.levels) - 1
+    x = rand(3 * H.levels[l].n, 7200 + b).astype(np.float32).astype(np.float64)
+    rhs = rand(3 * H.levels[l].n, 7300 + b, 10.0).astype(np.float32).astype(np.float64)
+    ref = H.smooth(l, x, rhs, 1)
+    for tc in (1, 0):
+        S.set_options(ras_tc=tc)
+        y = cu(x, torch.float32)
+        S.smooth(l, y, cu(rhs, torch.float32), 1)
+        assert rel(host(y), ref) < TOL32, (tc, rel(host(y), ref))
+    y = cu(x)
+    S.smooth(l, y, cu(rhs), 1)
+    assert rel(host(y), ref) < TOL64, rel(host(y), ref)
     S.close()
