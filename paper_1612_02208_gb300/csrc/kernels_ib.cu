@@ -885,9 +885,9 @@ __global__ void __launch_bounds__(256) k_window_fine(IBK<double> k, const double
     const int t = tiles[slot];
     const int N = k.N, mk = N - 1;
     const int i = (t % ntx) * tx + threadIdx.x, j = (t / ntx) * ty + threadIdx.y;
-    const int* bs = k.binStart[c];
-    const int* srt = k.sorted[c];
-    const double* wg = k.wgt[c];
+    const int* bs = c ? k.binStart[1] : k.binStart[0];   // selects: indexing the parameter arrays by c would copy
+    const int* srt = c ? k.sorted[1] : k.sorted[0];      // them to local memory
+    const double* wg = c ? k.wgt[1] : k.wgt[0];
     const double* kj = KJ + (size_t)c * k.M * 36;
     double acc[WD];
 #pragma unroll
@@ -923,84 +923,112 @@ void launch_window_fine(const IBK<double>& k, const double* KJ, const int* tiles
 
 // Coarse levels: the Galerkin product of Sec. 3.1 applied window to window,
 //   B_c(F, G) = sum_f R_u(F, f) sum_g B_f(f, g) P_u(g, G),  R_u = P_u^T / 4,
-// one thread per (coarse face, window row OY).  For x-faces R_u takes 1/4 of the two coincident
-// fine faces and 1/8 of the four faces half a coarse cell away in x, and P_u is linear in x and
-// constant in y; for y-faces the roles of x and y swap.
+// one thread per (coarse face F, window row OY).  Along the face's own direction ("linear": x for u) R_u
+// takes 1/4 of the two coincident fine faces and 1/8 of the four half a coarse cell away, and P_u gives a
+// fine face between two coarse ones half to each; across it ("constant") fine index g belongs to g >> 1.
+// A fine column at offset o of the fine face 2 F + d lies at k = o + d, |k| <= WR + 1, from 2 F: the fine rows
+// that reach OY are added by k (a register each), and the columns then go to the coarse offset k / 2, or half
+// each to the two around it, at most RAP_R away.  The rows of one fine face are loaded together; the loop over
+// the faces is kept rolled (unrolled, the instruction cache's misses alone took 30 us on an 8 x 8 level).
+// 128^2 disk, the four products of a set-up: 358 us with run-time sums in local memory, 108 us so.
+constexpr int RAP_R = 3;
+constexpr int RAP_K = WR + 1;
+template <int C>
+__device__ __forceinline__ void rap_columns(const double* __restrict__ winF, const int* __restrict__ slotF, int Nf,
+                                            int lgx, int lgy, int ntxf, int I, int J, int OY,
+                                            double (&col)[2 * RAP_K + 1]) {
+    constexpr int ROWS = C == 0 ? 2 : 3;   // fine rows 2 (J + OY) + e, e = 0, 1 (constant) or -1, 0, 1 (linear)
+    const int mkf = Nf - 1, perf = 1 << (lgx + lgy);
+#pragma unroll 1
+    for (int r = 0; r < 6; ++r) {
+        const int lin = r < 2 ? 0 : (r < 4 ? 1 : -1), con = r & 1;
+        const int dx = C == 0 ? lin : con, dy = C == 0 ? con : lin;
+        const double wr = r < 2 ? 0.25 : 0.125;
+        const int wx = (2 * I + dx) & mkf, wy = (2 * J + dy) & mkf;
+        const int sf = slotF[(wy >> lgy) * ntxf + (wx >> lgx)];
+        if (sf < 0) continue;
+        const double* w = winF + (((size_t)(sf * 2 + C) * WIN_SIZE) << (lgx + lgy)) +
+                          ((wy & ((1 << lgy) - 1)) << lgx) + (wx & ((1 << lgx) - 1));
+        double v[ROWS][2 * RAP_K + 1];
+#pragma unroll
+        for (int e = 0; e < ROWS; ++e) {
+            const int oy = 2 * OY + (C == 0 ? e : e - 1) - dy;
+#pragma unroll
+            for (int k = -RAP_K; k <= RAP_K; ++k) {
+                const int ox = k - dx;
+                v[e][k + RAP_K] = oy >= -WR && oy <= WR && ox >= -WR && ox <= WR
+                                      ? w[(size_t)((oy + WR) * WD + ox + WR) * perf]
+                                      : 0.0;
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < ROWS; ++e) {
+            const double wt = C == 1 && e != 1 ? 0.5 * wr : wr;
+#pragma unroll
+            for (int k = 0; k <= 2 * RAP_K; ++k) col[k] += wt * v[e][k];
+        }
+    }
+}
+// grid (coarse tiles, 2 WD): component and window row; lgx, lgy: log2 of the fine tile's sides
 __global__ void __launch_bounds__(256) k_window_rap(const double* __restrict__ winF, const int* __restrict__ slotF,
-                                                    int Nf, int txf, int tyf, int ntxf, const int* __restrict__ tilesC,
+                                                    int Nf, int lgx, int lgy, int ntxf, const int* __restrict__ tilesC,
                                                     int nTilesC, int Nc, int txc, int tyc, int ntxc,
                                                     double* __restrict__ winC) {
     pdl_entry();
     const int slot = blockIdx.x;
     if (slot >= nTilesC) return;
     const int c = blockIdx.y / WD, OY = (int)(blockIdx.y % WD) - WR;
-    const int perc = txc * tyc, perf = txf * tyf, q = threadIdx.y * txc + threadIdx.x;
+    const int perc = txc * tyc, q = threadIdx.y * txc + threadIdx.x;
     const int t = tilesC[slot];
     const int I = (t % ntxc) * txc + threadIdx.x, J = (t / ntxc) * tyc + threadIdx.y;
-    const int mkf = Nf - 1;
-    double acc[WD];
-    for (int e = 0; e < WD; ++e) acc[e] = 0.0;
-    for (int r = 0; r < 6; ++r) {
-        int dx, dy;
-        double wr;
-        if (c == 0) {
-            dx = r < 2 ? 0 : (r < 4 ? 1 : -1);
-            dy = r & 1;
-            wr = r < 2 ? 0.25 : 0.125;
+    double col[2 * RAP_K + 1];
+#pragma unroll
+    for (int k = 0; k <= 2 * RAP_K; ++k) col[k] = 0.0;
+    // the unwrapped rows that the window stores as row OY: OY itself, and on a level of four cells its aliases
+#pragma unroll 1
+    for (int o = -RAP_R; o <= RAP_R; ++o) {
+        if (wrapdiff(o, Nc) != OY) continue;
+        if (c == 0)
+            rap_columns<0>(winF, slotF, Nf, lgx, lgy, ntxf, I, J, o, col);
+        else
+            rap_columns<1>(winF, slotF, Nf, lgx, lgy, ntxf, I, J, o, col);
+    }
+    double acc[2 * RAP_R + 1];
+#pragma unroll
+    for (int o = 0; o <= 2 * RAP_R; ++o) acc[o] = 0.0;
+#pragma unroll
+    for (int k = -RAP_K; k <= RAP_K; ++k) {
+        const int k2 = k + 2 * RAP_R;   // even shift: keeps the operands of >> and & positive
+        const double x = col[k + RAP_K];
+        if ((k2 & 1) == 0) {
+            acc[k2 / 2] += x;
+        } else if (c == 1) {
+            acc[(k2 - 1) / 2] += x;
         } else {
-            dy = r < 2 ? 0 : (r < 4 ? 1 : -1);
-            dx = r & 1;
-            wr = r < 2 ? 0.25 : 0.125;
-        }
-        const int fx = 2 * I + dx, fy = 2 * J + dy;                 // unwrapped fine face
-        const int wx = fx & mkf, wy = fy & mkf;
-        const int sf = slotF[(wy / tyf) * ntxf + wx / txf];
-        if (sf < 0) continue;
-        const int qf = (wy % tyf) * txf + (wx % txf);
-        const double* w = winF + ((size_t)(sf * 2 + c) * WIN_SIZE) * perf + qf;
-        for (int oy = -WR; oy <= WR; ++oy) {
-            const int gy = fy + oy;
-            // targets of gy in y: constant (c == 0) or linear (c == 1)
-            int Gy[2];
-            double wyv[2];
-            int ny;
-            if (c == 0 || (gy & 1) == 0) {
-                Gy[0] = gy >> 1;
-                wyv[0] = 1.0;
-                ny = 1;
-            } else {
-                Gy[0] = (gy - 1) >> 1;
-                Gy[1] = (gy + 1) >> 1;
-                wyv[0] = wyv[1] = 0.5;
-                ny = 2;
-            }
-            double wsum = 0.0;
-            for (int a = 0; a < ny; ++a)
-                if (wrapdiff(Gy[a] - J, Nc) == OY) wsum += wyv[a];
-            if (wsum == 0.0) continue;
-            for (int ox = -WR; ox <= WR; ++ox) {
-                const double b = w[(size_t)((oy + WR) * WD + ox + WR) * perf];
-                if (b == 0.0) continue;
-                const int gx = fx + ox;
-                const double v = wr * wsum * b;
-                if (c == 1 || (gx & 1) == 0) {
-                    const int OX = wrapdiff((gx >> 1) - I, Nc);
-                    acc[OX + WR] += v;
-                } else {
-                    acc[wrapdiff(((gx - 1) >> 1) - I, Nc) + WR] += 0.5 * v;
-                    acc[wrapdiff(((gx + 1) >> 1) - I, Nc) + WR] += 0.5 * v;
-                }
-            }
+            acc[(k2 - 1) / 2] += 0.5 * x;
+            acc[(k2 + 1) / 2] += 0.5 * x;
         }
     }
     double* wout = winC + ((size_t)(slot * 2 + c) * WIN_SIZE + (size_t)(OY + WR) * WD) * perc + q;
-    for (int e = 0; e < WD; ++e) wout[(size_t)e * perc] = acc[e];
+#pragma unroll
+    for (int OX = -WR; OX <= WR; ++OX) {   // the columns likewise
+        double v = 0.0;
+#pragma unroll
+        for (int o = -RAP_R; o <= RAP_R; ++o)
+            if (wrapdiff(o, Nc) == OX) v += acc[o + RAP_R];
+        wout[(size_t)(OX + WR) * perc] = v;
+    }
+}
+static int log2i(int v) {
+    int l = 0;
+    while ((1 << l) < v) ++l;
+    return l;
 }
 void launch_window_rap(const double* winF, const int* slotF, int Nf, int txf, int tyf, int ntxf, const int* tilesC,
                        int nTilesC, int Nc, int txc, int tyc, int ntxc, double* winC, cudaStream_t s) {
     if (nTilesC == 0) return;
-    launch_pdl(k_window_rap, dim3(nTilesC, 2 * WD), dim3(txc, tyc), 0, s, winF, slotF, Nf, txf, tyf, ntxf, tilesC, nTilesC, Nc,
-                                                                 txc, tyc, ntxc, winC);
+    launch_pdl(k_window_rap, dim3(nTilesC, 2 * WD), dim3(txc, tyc), 0, s, winF, slotF, Nf, log2i(txf), log2i(tyf), ntxf,
+               tilesC, nTilesC, Nc, txc, tyc, ntxc, winC);
 }
 
 // slot of every tile of a level (-1 when the tile is not IB-active)
