@@ -305,6 +305,20 @@ template <typename T> void launch_wscale(const T* w, const double* nrm2, T* v, i
 // launchers (kernels_ib.cu)
 void launch_stencils(const double* X, int M, int Nf, int lmax, int** base, double** w64, float** w32,
                      cudaStream_t s);
+// The markers' Morton order and the bins of every level by counting (kernels_ib.cu)
+constexpr int BIN_MAX = 64;          // markers of one fine bin that k_bin_order puts in order
+struct BinArgs {
+    int M, nbins, lmax;              // markers, fine bins (N^2), finest level
+    const int* base[2];              // packed fine stencil origins
+    int* start[2];                   // nbins + 1: fine bin starts (counts on the way)
+    int* coarse[SIB_MAX_LEVELS][2];  // bin starts of the levels below lmax
+    uint32_t* arrival[2];            // M
+    int* sorted[2];                  // M: the result
+    int* sums;                       // 2 bin_chunks(nbins)
+    int* most;                       // largest fine bin; above BIN_MAX, sorted[] must come from launch_bitonic
+};
+int bin_chunks(int nbins);
+int launch_bin_markers(const BinArgs& a, cudaStream_t s);   // returns the number of launches
 void launch_sort_keys(const int* baseFine, int M, int Mpad, uint64_t* keys, cudaStream_t s);
 void launch_bitonic(uint64_t* keys, int Mpad, cudaStream_t s);
 void launch_unpack_sorted(const uint64_t* keys, int M, int* sorted, uint32_t* mkey, cudaStream_t s);

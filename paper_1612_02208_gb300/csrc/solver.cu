@@ -145,7 +145,8 @@ struct sib_ctx {
     bool haveIB = false;
     // topology
     uint64_t* keys = nullptr;
-    int Mpad = 0;
+    int* binSums = nullptr;      // scratch of the marker binning
+    int* binMost = nullptr;      // most markers of one fine bin
     int* sorted[2] = {nullptr, nullptr};
     uint32_t* mkey[2] = {nullptr, nullptr};
     int* adjStart = nullptr;
@@ -1332,17 +1333,20 @@ void setup(sib_ctx* c, cudaStream_t s) {
                 }
             KL(c, launch_stencils(c->X, c->M, c->N, c->lmax, base.data(), w64.data(), w32.data(), s));
             KL(c, launch_deinterleave(c->X, c->M, c->Xc, s));
-            int Mpad = 1;
-            while (Mpad < c->M) Mpad <<= 1;
-            c->Mpad = Mpad;
+            BinArgs ba{};
+            ba.M = c->M;
+            ba.nbins = c->N * c->N;
+            ba.lmax = c->lmax;
+            ba.sums = c->binSums;
+            ba.most = c->binMost;
             for (int q = 0; q < 2; ++q) {
-                KL(c, launch_sort_keys(c->L[c->lmax].base[q], c->M, Mpad, c->keys, s));
-                launch_bitonic(c->keys, Mpad, s);
-                KL(c, launch_unpack_sorted(c->keys, c->M, c->sorted[q], c->mkey[q], s));
-                for (int l = 0; l <= c->lmax; ++l)
-                    KL(c, launch_bins(c->mkey[q], c->M, c->L[l].N * c->L[l].N, 2 * (c->lmax - l),
-                                      c->L[l].binStart[q], s));
+                ba.base[q] = c->L[c->lmax].base[q];
+                ba.start[q] = c->L[c->lmax].binStart[q];
+                for (int l = 0; l < c->lmax; ++l) ba.coarse[l][q] = c->L[l].binStart[q];
+                ba.arrival[q] = c->mkey[q];
+                ba.sorted[q] = c->sorted[q];
             }
+            c->launches += launch_bin_markers(ba, s);
         }
         for (int l = 0; l <= c->lmax; ++l) {
             Level& lv = c->L[l];
@@ -1356,11 +1360,22 @@ void setup(sib_ctx* c, cudaStream_t s) {
         }
         launch_adjacency(c->edges, c->E, c->M, c->deg, c->adjStart, c->adjNbr, c->adjEid, s);
         std::vector<int> cnt(2 * (c->lmax + 1));
+        int most = 0;
+        if (c->M > 0) CK(cudaMemcpyAsync(&most, c->binMost, sizeof(int), cudaMemcpyDeviceToHost, s));
         for (int l = 0; l <= c->lmax; ++l) {
             CK(cudaMemcpyAsync(&cnt[2 * l], c->L[l].nTiles, sizeof(int), cudaMemcpyDeviceToHost, s));
             CK(cudaMemcpyAsync(&cnt[2 * l + 1], c->L[l].nRowTiles, sizeof(int), cudaMemcpyDeviceToHost, s));
         }
         CK(cudaStreamSynchronize(s));
+        if (most > BIN_MAX) {   // a crowded cell: the order by the sorting network instead
+            int Mpad = 1;
+            while (Mpad < c->M) Mpad <<= 1;
+            for (int q = 0; q < 2; ++q) {
+                KL(c, launch_sort_keys(c->L[c->lmax].base[q], c->M, Mpad, c->keys, s));
+                launch_bitonic(c->keys, Mpad, s);
+                KL(c, launch_unpack_sorted(c->keys, c->M, c->sorted[q], c->mkey[q], s));
+            }
+        }
         for (int l = 0; l <= c->lmax; ++l) {
             Level& lv = c->L[l];
             lv.hnTiles = cnt[2 * l];
@@ -2182,6 +2197,8 @@ int sib_create(sib_ctx** out, int N, int n_min) {
         CK(cudaMallocHost(&c->herr, 64));
         std::memset(c->herr, 0, 64);
         alloc_markers(c);
+        c->binSums = (int*)dalloc(c, sizeof(int) * 2 * (size_t)bin_chunks(N * N));
+        c->binMost = (int*)dalloc(c, sizeof(int));
     } catch (const SibError& e) {
         std::fprintf(stderr, "sib_create: %s\n", e.what());
         sib_destroy(c);

@@ -14,10 +14,12 @@ from tests.test_gpu_parity import TOL32, TOL64, cu, host, rand, rel  # noqa: E40
 EPS = 2.0 ** -53
 
 
-# grids below, at and above one 32 x 8 tile; single markers; a cell that holds every marker; markers
-# outside the unit square (they wrap)
+# grids below, at and above one 32 x 8 tile; single markers; a cell that holds every marker, with as many as
+# the counting sort orders itself and one more; markers outside the unit square (they wrap); more chunks of
+# bins than a scan block has threads
 @pytest.mark.parametrize("N,M,where", [(4, 1, "any"), (8, 3, "any"), (16, 200, "any"), (32, 1, "seam"), (32, 700, "cell"),
-                                       (64, 999, "any"), (64, 64, "seam"), (128, 5001, "any"), (256, 37, "outside")])
+                                       (64, 999, "any"), (64, 64, "seam"), (128, 5001, "any"), (256, 37, "outside"),
+                                       (32, 64, "cell"), (32, 65, "cell"), (1024, 20000, "any")])
 def test_spread_tiles(N, M, where):
     rng = np.random.default_rng(100 * N + M)
     X = rng.uniform(0.0, 1.0, (M, 2))
@@ -82,4 +84,25 @@ def test_narrow_boxes_on_tensor_cores(make, b, o):
     y = cu(x)
     S.smooth(l, y, cu(rhs), 1)
     assert rel(host(y), ref) < TOL64, rel(host(y), ref)
+    S.close()
+
+
+# Galerkin windows of every level, down to 4 x 4 cells, where window offsets alias, and the coarsest
+# pseudo-inverse by block elimination (4 and 8 cells) and by Gauss-Jordan (16), with and without a density
+@pytest.mark.parametrize("n_min", [4, 8, 16])
+@pytest.mark.parametrize("make", [lambda: I.disk_stokes(32, kappa=1e4, seed=1), lambda: I.thin_ellipse_re(64, kappa=1e4)],
+                         ids=["stokes", "re"])
+def test_coarse_levels(make, n_min):
+    prob = make()
+    H = multigrid.Hierarchy(prob, n_min=n_min)
+    st = prob.structure
+    S = sib.Solver(prob.N, n_min=n_min)
+    S.set_fluid(prob.rho, prob.mu, prob.dt)
+    S.set_structure(cu(st.X), torch.as_tensor(st.edges, device="cuda"), cu(st.kappa))
+    S.setup()
+    for l, lev in enumerate(H.levels):
+        u = rand(2 * lev.n, 7400 + l)
+        assert rel(host(S.apply_ib(l, cu(u))), lev.B @ u) < TOL64, l
+    b = rand(3 * n_min * n_min, 7500)
+    assert rel(host(S.coarse_solve(cu(b))), H.coarse_pinv @ b) < TOL64
     S.close()
