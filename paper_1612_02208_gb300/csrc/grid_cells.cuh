@@ -101,26 +101,6 @@ __device__ __forceinline__ T res_v_act(const GridK<T>& g, bool act, const T* __r
     return b[n + c] - Av;
 }
 
-// Coarse right-hand side of coarse cell (I, J): R (b - L x) from the sixteen fine residuals that
-// R = diag(P_u^T / 4, P_v^T / 4, average) combines (Sec. 3.2, Alg. 1).
-template <typename T>
-__device__ __forceinline__ void residual_restrict_cell(const GridK<T>& g, const T* __restrict__ x,
-                                                       const T* __restrict__ b, T* __restrict__ bc, int I, int J) {
-    const int Nc = g.N / 2;
-    const int i = 2 * I, j = 2 * J;
-    const T su = (res_u(g, x, b, i, j) + res_u(g, x, b, i, j + 1)) +
-                 T(0.5) * ((res_u(g, x, b, i + 1, j) + res_u(g, x, b, i + 1, j + 1)) +
-                           (res_u(g, x, b, i - 1, j) + res_u(g, x, b, i - 1, j + 1)));
-    const T sv = (res_v(g, x, b, i, j) + res_v(g, x, b, i + 1, j)) +
-                 T(0.5) * ((res_v(g, x, b, i, j + 1) + res_v(g, x, b, i + 1, j + 1)) +
-                           (res_v(g, x, b, i, j - 1) + res_v(g, x, b, i + 1, j - 1)));
-    const T sp = (res_p(g, x, b, i, j) + res_p(g, x, b, i + 1, j)) + (res_p(g, x, b, i, j + 1) + res_p(g, x, b, i + 1, j + 1));
-    const int nc = Nc * Nc, c = J * Nc + I;
-    bc[c] = T(0.25) * su;
-    bc[nc + c] = T(0.25) * sv;
-    bc[2 * nc + c] = T(0.25) * sp;
-}
-
 // Coarse right-hand side of coarse cell (I, J) from a fine residual rf (Sec. 3.2): a coarse x-face
 // takes 1/4 of the two coincident fine faces plus 1/8 of the four fine faces half a coarse cell
 // away in x (R_u = P_u^T / 4); pressure: the average of the four fine cells.

@@ -738,27 +738,88 @@ void launch_vanka_zero(const GridK<T>& g, const T* b, T* xo, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Fine residual and its restriction in one pass (Sec. 3.2, Alg. 1): one thread per coarse cell.
+// Fine residual and its restriction in one pass (Sec. 3.2, Alg. 1), bc = R (b - L x) with R = diag(P_u^T / 4,
+// P_v^T / 4, average): a coarse x-face takes 1/4 of the two coincident fine faces and 1/8 of the four half a
+// coarse cell away in x, a y-face likewise in y, a pressure the average of its four cells.  One block per
+// 32 x 8 fine tile: every thread forms its cell's three residuals straight from global memory (all loads
+// independent), two more warps those of the faces left of and below the tile, and the tile's coarse values are
+// combined from shared memory.  Levels that fit the caches are bound by this one chain of latencies, FP64 levels
+// by the FP64 pipe (each residual formed once); staging a 64 x 16 tile first, as the FP32 form for large levels
+// below does, cost 11.3 us at 64^2 ... 256^2 against 1.7 here (FP64: 21.4 against 3.6; 4096^2 1,141 against 903).
+constexpr int RS_HALO = 64;   // two warps for the tile's neighbours
 template <typename T>
-__global__ void k_residual_restrict(GridK<T> g, const T* __restrict__ x, const T* __restrict__ b, T* __restrict__ bc) {
+__global__ void __launch_bounds__(TX * TY + RS_HALO) k_residual_restrict(GridK<T> g, const T* __restrict__ x,
+                                                                         const T* __restrict__ b,
+                                                                         T* __restrict__ bc) {
+    __shared__ T su[TY][TX + 1], sv[TY + 1][TX], sp[TY][TX];   // su: column 0 is the face left of the tile, sv: row
+    const int N = g.N, n = N * N, m = N - 1, tx = g.tx, ty = g.ty, per = tx * ty, tid = threadIdx.x;   // 0 below it
+    const bool act = g.tile != nullptr && g.tile[blockIdx.y * g.ntx + blockIdx.x];   // set-up data, before the wait
     pdl_entry();
-    const int Nc = g.N / 2;
-    const int I = blockIdx.x * blockDim.x + threadIdx.x;
-    const int J = blockIdx.y * blockDim.y + threadIdx.y;
-    if (I >= Nc || J >= Nc) return;
-    residual_restrict_cell(g, x, b, bc, I, J);
+    const int i0 = blockIdx.x * tx, j0 = blockIdx.y * ty;
+    const T* u = x;
+    const T* v = x + n;
+    const T* p = x + 2 * n;
+    // residual of the u (v) face of cell (i, j): the flag covers the faces beside the tile too
+    auto ru = [&](int i, int j) {
+        const int ip = (i + 1) & m, im = (i - 1) & m, jp = (j + 1) & m, jm = (j - 1) & m, c = j * N + i;
+        T Au = g.a0 * u[c] - g.c * ((u[j * N + ip] + u[j * N + im]) + (u[jp * N + i] + u[jm * N + i])) +
+               (p[c] - p[j * N + im]) * g.inv_h;
+        Au -= g.dt * ibf_act(g, act, 0, i, j);
+        return b[c] - Au;
+    };
+    auto rv = [&](int i, int j) {
+        const int ip = (i + 1) & m, im = (i - 1) & m, jp = (j + 1) & m, jm = (j - 1) & m, c = j * N + i;
+        T Av = g.a0 * v[c] - g.c * ((v[j * N + ip] + v[j * N + im]) + (v[jp * N + i] + v[jm * N + i])) +
+               (p[c] - p[jm * N + i]) * g.inv_h;
+        Av -= g.dt * ibf_act(g, act, 1, i, j);
+        return b[n + c] - Av;
+    };
+    if (tid < per) {
+        const int lx = tid & (tx - 1), ly = tid >> g.lgtx, i = i0 + lx, j = j0 + ly, c = j * N + i;
+        su[ly][lx + 1] = ru(i, j);
+        sv[ly + 1][lx] = rv(i, j);
+        sp[ly][lx] = b[2 * n + c] + ((u[j * N + ((i + 1) & m)] - u[c]) + (v[((j + 1) & m) * N + i] - v[c])) * g.inv_h;
+    } else if (tid >= TX * TY) {
+        const int q = tid & 31;
+        if (tid < TX * TY + 32) {
+            if (q < ty) su[q][0] = ru((i0 - 1) & m, j0 + q);
+        } else {
+            if (q < tx) sv[0][q] = rv(i0 + q, (j0 - 1) & m);
+        }
+    }
+    __syncthreads();
+    // one thread per coarse cell and component
+    const int cx = tx >> 1, cper = per >> 2;
+    for (int t = tid; t < 3 * cper; t += TX * TY + RS_HALO) {
+        const int comp = t >= 2 * cper ? 2 : (t >= cper ? 1 : 0), q = t - comp * cper;
+        const int X = q & (cx - 1), Y = q >> (g.lgtx - 1), f = 2 * X, h = 2 * Y;
+        T s;
+        if (comp == 0)
+            s = (su[h][f + 1] + su[h + 1][f + 1]) +
+                T(0.5) * ((su[h][f + 2] + su[h + 1][f + 2]) + (su[h][f] + su[h + 1][f]));
+        else if (comp == 1)
+            s = (sv[h + 1][f] + sv[h + 1][f + 1]) +
+                T(0.5) * ((sv[h + 2][f] + sv[h + 2][f + 1]) + (sv[h][f] + sv[h][f + 1]));
+        else
+            s = (sp[h][f] + sp[h][f + 1]) + (sp[h + 1][f] + sp[h + 1][f + 1]);
+        const int Nc = N / 2;
+        bc[(size_t)comp * Nc * Nc + (j0 / 2 + Y) * Nc + i0 / 2 + X] = T(0.25) * s;
+    }
 }
-// The same residual and restriction for N >= 64, tiled: one block per 32 x 8 coarse cells (64 x 16
+
+// The same residual and restriction on large FP32 levels, tiled: one block per 32 x 8 coarse cells (64 x 16
 // fine cells).  The block stages x (three components, fine rows fj0-2 .. fj0+17), b and the IB force
 // (rows fj0-1 .. fj0+16), all over columns fi0-4 .. fi0+67, in shared memory.  Blocks whose staged
-// rows and columns lie inside the grid load 16-byte vectors, every load issued before the first
-// shared store; the others (the periodic wrap) gather element by element.  Each thread then forms, in
-// registers, the fine residuals its coarse cell's restriction needs (u faces of columns 2I-1 .. 2I+1,
-// v faces of rows 2J-1 .. 2J+1, p of its four cells; the faces it shares with a neighbour are formed
-// by both) with the arithmetic of res_u / res_v / res_p, reading the staged rows as column pairs, and
-// restricts them as residual_restrict_cell does.  The IB force is read where one of the tile's four
-// fine tiles is IB-active: their flags are dilated by one tile and cover the one-cell halo, and the
-// force is zero on inactive tiles.
+// rows and columns lie inside the grid take three TMA box copies; the others (the periodic wrap) gather
+// element by element, RR_BATCH loads of a thread in flight.  Each thread then forms, in registers, the fine
+// residuals its coarse cell's restriction needs (u faces of columns 2I-1 .. 2I+1, v faces of rows
+// 2J-1 .. 2J+1, p of its four cells; the faces it shares with a neighbour are formed by both), reading the
+// staged rows as column pairs.  The IB force is read where one of the tile's four fine tiles is IB-active:
+// their flags are dilated by one tile and cover the one-cell halo, and the force is zero on inactive tiles.
+// From RR_MIN on the staged reads pay: 1024^2 15.8 us against 9.4 by the kernel above, 2048^2 29.4 against
+// 44.4, 4096^2 91 against 169 (103 with the wrap tiles' loads one at a time).
+constexpr int RR_MIN = 2048;
+constexpr int RR_BATCH = 8;
 constexpr int RR_CX = 32, RR_CY = 8;                 // coarse cells per block
 constexpr int RR_FX = 2 * RR_CX, RR_FY = 2 * RR_CY;  // fine cells per block
 constexpr int RR_W = RR_FX + 8;                      // staged row width (columns fi0-4 .. fi0+67)
@@ -767,26 +828,14 @@ constexpr int RR_XH = RR_FY + 4, RR_BH = RR_FY + 2;  // staged rows of x (fj0-2 
 constexpr int RR_FOFF = ((3 * RR_XH + 3 * RR_BH) * RR_W + 31) / 32 * 32;
 constexpr int RR_WORDS = RR_FOFF + 2 * RR_BH * RR_W;
 static_assert((3 * RR_XH * RR_W) % 32 == 0, "the staged b starts on a 128-byte boundary");
-template <typename T>
-struct RRVec;
-template <>
-struct RRVec<float> {
-    using type = float4;
-    using pair = float2;
-};
-template <>
-struct RRVec<double> {
-    using type = double2;
-    using pair = double2;
-};
-template <typename T>
-__global__ void __launch_bounds__(RR_CX * RR_CY) k_residual_restrict_tiled(GridK<T> g,
+__global__ void __launch_bounds__(RR_CX * RR_CY) k_residual_restrict_tiled(GridK<float> g,
                                                                            const __grid_constant__ CUtensorMap mx,
                                                                            const __grid_constant__ CUtensorMap mb,
                                                                            const __grid_constant__ CUtensorMap mf,
-                                                                           int tma, const T* __restrict__ x,
-                                                                           const T* __restrict__ b,
-                                                                           T* __restrict__ bc) {
+                                                                           int tma, const float* __restrict__ x,
+                                                                           const float* __restrict__ b,
+                                                                           float* __restrict__ bc) {
+    using T = float;
     constexpr int NXB = 3 * RR_XH + 3 * RR_BH;                 // staged rows of x and b
     constexpr int NROWS = NXB + 2 * RR_BH;                     // and of the IB force
     constexpr int NT = RR_CX * RR_CY;
@@ -838,33 +887,40 @@ __global__ void __launch_bounds__(RR_CX * RR_CY) k_residual_restrict_tiled(GridK
             return;
         }
     } else {
-        const int rows = act ? NROWS : NXB;
-        for (int q = tid; q < rows * RR_W; q += NT) {
-            const int r = q / RR_W, cc = q - r * RR_W;
-            const T* base;
-            int gj;
-            T* dst;
-            if (r < 3 * RR_XH) {
-                const int comp = r / RR_XH;
-                base = x + (size_t)comp * n;
-                gj = fj0 - 2 + (r - comp * RR_XH);
-                dst = sx + r * RR_W;
-            } else if (r < NXB) {
-                const int rr = r - 3 * RR_XH, comp = rr / RR_BH;
-                base = b + (size_t)comp * n;
-                gj = fj0 - 1 + (rr - comp * RR_BH);
-                dst = sb + rr * RR_W;
-            } else {
-                const int rr = r - NXB, comp = rr / RR_BH;
-                base = g.fib + (size_t)comp * n;
-                gj = fj0 - 1 + (rr - comp * RR_BH);
-                dst = sf + rr * RR_W;
+        const int total = (act ? NROWS : NXB) * RR_W;
+        for (int q0 = tid; q0 < total; q0 += RR_BATCH * NT) {
+            T v[RR_BATCH];
+#pragma unroll
+            for (int k = 0; k < RR_BATCH; ++k) {   // staged row r: x rows, b rows, IB force rows, one after another
+                const int q = q0 + k * NT;
+                if (q >= total) break;
+                const int r = q / RR_W, cc = q - r * RR_W;
+                const T* base;
+                int gj;
+                if (r < 3 * RR_XH) {
+                    const int comp = r / RR_XH;
+                    base = x + (size_t)comp * n;
+                    gj = fj0 - 2 + (r - comp * RR_XH);
+                } else if (r < NXB) {
+                    const int rr = r - 3 * RR_XH, comp = rr / RR_BH;
+                    base = b + (size_t)comp * n;
+                    gj = fj0 - 1 + (rr - comp * RR_BH);
+                } else {
+                    const int rr = r - NXB, comp = rr / RR_BH;
+                    base = g.fib + (size_t)comp * n;
+                    gj = fj0 - 1 + (rr - comp * RR_BH);
+                }
+                v[k] = base[(size_t)(gj & m) * N + ((fi0 - 4 + cc) & m)];
             }
-            dst[cc] = base[(size_t)(gj & m) * N + ((fi0 - 4 + cc) & m)];
+#pragma unroll
+            for (int k = 0; k < RR_BATCH; ++k) {
+                const int q = q0 + k * NT;
+                if (q < total) (q < NXB * RR_W ? sx[q] : sf[q - NXB * RR_W]) = v[k];   // sb follows sx
+            }
         }
         __syncthreads();
     }
-    using P2 = typename RRVec<T>::pair;
+    using P2 = float2;
     const T* U = sx;
     const T* V = sx + RR_XH * RR_W;
     const T* P = sx + 2 * RR_XH * RR_W;
@@ -963,31 +1019,29 @@ __global__ void __launch_bounds__(RR_CX * RR_CY) k_residual_restrict_tiled(GridK
 
 template <typename T>
 void launch_residual_restrict(const GridK<T>& g, const T* x, const T* b, T* bc, cudaStream_t s) {
-    const int Nc = g.N / 2;
-    if (Nc >= RR_CX && g.tx == TX && g.ty == TY) {   // fine tiles of 32 x 8: two by two per block
-        const size_t smem = sizeof(T) * (size_t)RR_WORDS + 128;   // 128: room to align the staged tile
-        static thread_local bool enabled = false;
-        if (!enabled) {
-            cudaFuncSetAttribute(k_residual_restrict_tiled<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            enabled = true;
+    if constexpr (sizeof(T) == 4) {
+        if (g.N >= RR_MIN) {
+            const int Nc = g.N / 2;
+            const size_t smem = sizeof(T) * (size_t)RR_WORDS + 128;   // 128: room to align the staged tile
+            static thread_local bool enabled = false;
+            if (!enabled) {
+                cudaFuncSetAttribute(k_residual_restrict_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                enabled = true;
+            }
+            CUtensorMap mx, mb, mf;
+            std::memset(&mx, 0, sizeof(mx));
+            std::memset(&mb, 0, sizeof(mb));
+            std::memset(&mf, 0, sizeof(mf));
+            // the maps are only read by the interior tiles, the IB force's only where a tile is IB-active
+            const int es = (int)sizeof(T);
+            const int tma = field_map(&mx, x, g.N, es, RR_XH, RR_W, 3) && field_map(&mb, b, g.N, es, RR_BH, RR_W, 3) &&
+                            (!g.tile || !g.fib || field_map(&mf, g.fib, g.N, es, RR_BH, RR_W, 2));
+            launch_pdl(k_residual_restrict_tiled, dim3(Nc / RR_CX, Nc / RR_CY), dim3(RR_CX, RR_CY), smem, s, g, mx, mb,
+                       mf, tma, x, b, bc);
+            return;
         }
-        CUtensorMap mx, mb, mf;
-        std::memset(&mx, 0, sizeof(mx));
-        std::memset(&mb, 0, sizeof(mb));
-        std::memset(&mf, 0, sizeof(mf));
-        // interior tiles exist from N = 4 RR_FX on (a tile's staged columns reach 4 beyond it on each side);
-        // the maps are only read by those tiles, the IB force's only where a tile is IB-active
-        const int es = (int)sizeof(T);
-        const int tma = g.N >= 4 * RR_FX && field_map(&mx, x, g.N, es, RR_XH, RR_W, 3) &&
-                        field_map(&mb, b, g.N, es, RR_BH, RR_W, 3) &&
-                        (!g.tile || !g.fib || field_map(&mf, g.fib, g.N, es, RR_BH, RR_W, 2));
-        launch_pdl(k_residual_restrict_tiled<T>, dim3(Nc / RR_CX, Nc / RR_CY), dim3(RR_CX, RR_CY), smem, s, g, mx, mb,
-                   mf, tma, x, b, bc);
-        return;
     }
-    dim3 blk(Nc < 32 ? Nc : 32, Nc < 8 ? Nc : 8);
-    dim3 grd((Nc + blk.x - 1) / blk.x, (Nc + blk.y - 1) / blk.y);
-    launch_pdl(k_residual_restrict<T>, grd, blk, 0, s, g, x, b, bc);
+    launch_pdl(k_residual_restrict<T>, dim3(g.N / g.tx, g.N / g.ty), dim3(TX * TY + RS_HALO), 0, s, g, x, b, bc);
 }
 
 // ------------------------------------------------------------------------------------------
