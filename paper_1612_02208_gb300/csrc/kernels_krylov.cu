@@ -7,7 +7,6 @@
 #include <cmath>
 
 #include "sib_internal.h"
-#include "spd_sweep.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -408,112 +407,6 @@ __global__ void k_extract_pinv(const double* __restrict__ Aug, const int* __rest
 }
 void launch_extract_pinv(const double* Aug, const int* piv, int n, int N0, double rho, double* Pinv, cudaStream_t s) {
     launch_pdl(k_extract_pinv, dim3((n + 127) / 128, n), 128, 0, s, Aug, piv, n, N0, rho, Pinv);
-}
-
-// The coarsest pseudo-inverse of the periodic box by block elimination.  L0 = [A G; G^T 0] with
-// A = diag(A_u, A_v) (the IB block couples a component only to itself) and, with z the normalised constant of
-// n0 cells, A' = A + z z^T per component when rho = 0: A' and S = G^T A'^{-1} G + z z^T are positive definite,
-// so no pivoting is needed, and as G z = 0
-//   L0^+ = [A'^{-1} - W S^{-1} W^T - (rho = 0: z z^T),  W S^{-1};  S^{-1} W^T,  z z^T - S^{-1}],  W = A'^{-1} G.
-// Three launches: both velocity blocks in a block each, S in one block, then one block per row.  8 x 8 cells:
-// 575 us by the blocked Gauss-Jordan of the whole matrix (36 launches, its one-block panels 42 us each), 330 us so,
-// on the set-up's critical path for the Vanka smoother; 64 dependent steps of about 2.2 us in one SM bound it.  A pivot that is not positive sets bit 1 of *info and
-// voids the result; the caller then takes the Gauss-Jordan.  Levels of up to PI_MAXN cells a side.
-constexpr int PI_MAXN = 8;
-constexpr int PI_THREADS = 256;
-constexpr int PI_E = (PI_MAXN * PI_MAXN * (PI_MAXN * PI_MAXN + 1) / 2 + PI_THREADS - 1) / PI_THREADS;
-__global__ void __launch_bounds__(PI_THREADS) k_pinv_velocity(int N, double rho, double mu, double dt,
-                                                             const double* __restrict__ B, double* __restrict__ work,
-                                                             int* __restrict__ info) {
-    pdl_entry();
-    __shared__ double col[2 * PI_MAXN * PI_MAXN];
-    const int n = N * N, mk = N - 1, c = blockIdx.x;
-    const double a0 = rho / dt + 4.0 * mu * N * N, cc = mu * N * N, zz = rho == 0.0 ? 1.0 / n : 0.0;
-    double* out = work + (size_t)c * n * n;
-    spd_sweep_regs<PI_E>(
-        n, col, info,
-        [&](int q, int f) {
-            const int i = q % N, j = q / N;
-            double x = zz - dt * B[(size_t)c * n * n + q * n + f];
-            if (f == q) x += a0;
-            if (f == j * N + ((i + 1) & mk)) x -= cc;
-            if (f == j * N + ((i - 1) & mk)) x -= cc;
-            if (f == ((j + 1) & mk) * N + i) x -= cc;
-            if (f == ((j - 1) & mk) * N + i) x -= cc;
-            return x;
-        },
-        [&](int i, int j, double x) { out[i * n + j] = out[j * n + i] = x; });
-}
-// the face of cell q (component c) with -1/h in G's column q; the one with +1/h is q itself
-__device__ __forceinline__ int pinv_face(int N, int c, int q) {
-    const int i = q % N, j = q / N;
-    return c == 0 ? j * N + ((i + 1) & (N - 1)) : ((j + 1) & (N - 1)) * N + i;
-}
-__global__ void __launch_bounds__(PI_THREADS) k_pinv_pressure(int N, double* __restrict__ work, int* __restrict__ info) {
-    pdl_entry();
-    __shared__ double col[2 * PI_MAXN * PI_MAXN];
-    const int n = N * N;
-    const double ih2 = (double)N * N;
-    double* out = work + 2 * (size_t)n * n;
-    spd_sweep_regs<PI_E>(
-        n, col, info,
-        [&](int i, int j) {
-            double s = 0.0;
-            for (int c = 0; c < 2; ++c) {
-                const double* M = work + (size_t)c * n * n;
-                const int i2 = pinv_face(N, c, i), j2 = pinv_face(N, c, j);
-                s += (M[i * n + j] - M[i * n + j2]) - (M[i2 * n + j] - M[i2 * n + j2]);
-            }
-            return ih2 * s + 1.0 / n;
-        },
-        [&](int i, int j, double x) { out[i * n + j] = out[j * n + i] = x; });
-}
-// row r of the pseudo-inverse: q = the row of S^{-1}, or W_r S^{-1}; thread: one column (3 n <= PI_THREADS)
-__global__ void __launch_bounds__(PI_THREADS) k_pinv_rows(int N, double rho, const double* __restrict__ work,
-                                                         double* __restrict__ P) {
-    pdl_entry();
-    __shared__ double wr[PI_MAXN * PI_MAXN], q[PI_MAXN * PI_MAXN];
-    const int n = N * N, r = blockIdx.x, br = r / n, lr = r - br * n, t = threadIdx.x;
-    const double ih = (double)N, zz = 1.0 / n;
-    const double* Si = work + 2 * (size_t)n * n;
-    if (t < n) {
-        if (br < 2) {
-            const double* M = work + (size_t)br * n * n + lr;
-            wr[t] = ih * (M[(size_t)t * n] - M[(size_t)pinv_face(N, br, t) * n]);
-        } else {
-            q[t] = Si[(size_t)lr * n + t];
-        }
-    }
-    __syncthreads();
-    if (t < n && br < 2) {
-        double s = 0.0;
-#pragma unroll 8
-        for (int c = 0; c < n; ++c) s += wr[c] * Si[(size_t)c * n + t];
-        q[t] = s;
-    }
-    __syncthreads();
-    if (t >= 3 * n) return;
-    const int bc = t / n, lc = t - bc * n;
-    double v;
-    if (bc < 2) {
-        const double* M = work + (size_t)bc * n * n + lc;
-        double s = 0.0;
-#pragma unroll 8
-        for (int c = 0; c < n; ++c) s += q[c] * (ih * (M[(size_t)c * n] - M[(size_t)pinv_face(N, bc, c) * n]));
-        v = br == 2 ? s : (br == bc ? M[(size_t)lr * n] - (rho == 0.0 ? zz : 0.0) : 0.0) - s;
-    } else {
-        v = br == 2 ? zz - q[lc] : q[lc];
-    }
-    P[(size_t)r * 3 * n + t] = v;
-}
-bool launch_pinv_blocks(int N, double rho, double mu, double dt, const double* B, double* work, double* P, int* info,
-                        cudaStream_t s) {
-    if (N > PI_MAXN) return false;
-    const int n = N * N;
-    launch_pdl(k_pinv_velocity, 2, PI_THREADS, 0, s, N, rho, mu, dt, B, work, info);
-    launch_pdl(k_pinv_pressure, 1, PI_THREADS, 0, s, N, work, info);
-    launch_pdl(k_pinv_rows, 3 * n, PI_THREADS, 0, s, N, rho, (const double*)work, P);
-    return true;
 }
 
 // x = Pinv b, one warp per row, FP64 accumulation for both precisions

@@ -19,7 +19,6 @@
 #include <algorithm>
 
 #include "sib_internal.h"
-#include "spd_sweep.cuh"
 #include "tcgen05.cuh"
 #include "tma.cuh"
 
@@ -389,12 +388,43 @@ __global__ void __launch_bounds__(RAS_BIG_SETUP_THREADS)
 // elimination (35 ms a level, whatever its number of boxes), 8.7 ms so.
 // A pivot that is not positive (a block so badly conditioned that rounding takes its definiteness, or a
 // value that is not finite) raises bit 1 of *info: the caller then takes k_ras_setup_big, which pivots.
-constexpr int BE_THREADS = 256;
+constexpr int BE_THREADS = 256, BE_WARPS = BE_THREADS / 32;
 constexpr int BE_ROWS = 32;        // owned rows per block, four per warp
 constexpr int BE_CPL = 5;          // columns per lane
 constexpr int BE_COLS = 32 * BE_CPL;
 constexpr int BE_KC = 16;          // pressures per shared-memory chunk
 __host__ __device__ inline int be_nu(int e) { return e * (e + 1); }
+__device__ __forceinline__ int tri(int i) { return i * (i + 1) / 2; }
+
+// A (lower triangle, packed rows, n x n) <- -A^{-1} by symmetric sweeps: at step k, with d = 1 / A_kk and
+// v = column k, A_ij -= v_i v_j d for i, j != k, A_ik = v_i d, A_kk = -d.  Rows i and n - 1 - i are swept as
+// one row of n + 1 entries, so that the warps' lanes stay full.
+__device__ void be_sweep(double* A, double* v, double* vd, int n, int* info) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, pairs = (n + 1) / 2;
+    for (int k = 0; k < n; ++k) {
+        const double akk = A[tri(k) + k];
+        const double d = 1.0 / akk;
+        for (int i = threadIdx.x; i < n; i += BE_THREADS) {
+            const double x = i >= k ? A[tri(i) + k] : A[tri(k) + i];
+            v[i] = x;
+            vd[i] = x * d;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0 && !(akk > 0.0)) atomicOr(info, 2);
+        for (int p = wid; p < pairs; p += BE_WARPS) {
+            const int i1 = p, i2 = n - 1 - p;             // i1 <= i2; equal in the middle of an odd n
+            const int len = i1 == i2 ? i1 + 1 : n + 1;
+            for (int t = lane; t < len; t += 32) {
+                const int i = t <= i1 ? i1 : i2, j = t <= i1 ? t : t - i1 - 1;
+                double* a = A + tri(i) + j;
+                double x = *a - v[i] * vd[j];
+                if (i == k || j == k) x = i == j ? -d : vd[i == k ? j : i];
+                *a = x;
+            }
+        }
+        __syncthreads();
+    }
+}
 
 // A_c^{-1} of matrix first + blockIdx.x (0: the shared IB-free operator; s > 0: box list[s - 1]) for component
 // c = blockIdx.y, into its workspace [A_u^{-1} | A_v^{-1} | S^{-1}]
@@ -434,7 +464,7 @@ __global__ void __launch_bounds__(BE_THREADS) k_ras_be_velocity(RasGeo G, RasIB 
                 add(ii + di, jj + dj, -dt * w[(size_t)((dj + WR) * WD + (di + WR)) * per]);
     }
     __syncthreads();
-    spd_sweep(A, v, vd, n, info);
+    be_sweep(A, v, vd, n, info);
     double* out = work + (size_t)blockIdx.x * (2 * (size_t)n * n + (size_t)np * np) + (size_t)comp * n * n;
     for (int t = threadIdx.x; t < n * n; t += BE_THREADS) {
         const int i = t / n, j = t - i * n;
@@ -473,7 +503,7 @@ __global__ void __launch_bounds__(BE_THREADS) k_ras_be_pressure(RasGeo G, double
         A[tri(i) + j] = ih2 * s;
     }
     __syncthreads();
-    spd_sweep(A, v, vd, np, info);
+    be_sweep(A, v, vd, np, info);
     double* out = wk + 2 * (size_t)n * n;
     for (int t = threadIdx.x; t < np * np; t += BE_THREADS) {
         const int i = t / np, j = t - i * np;

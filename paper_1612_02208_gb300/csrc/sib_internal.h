@@ -405,10 +405,6 @@ void launch_assemble_L0(int N0, double rho, double mu, double dt, const double* 
 size_t gauss_jordan_work_bytes(int n);
 void launch_gauss_jordan(double* Aug, int n, int* info, int* piv, void* work, cudaStream_t s);
 void launch_extract_pinv(const double* Aug, const int* piv, int n, int N0, double rho, double* Pinv, cudaStream_t s);
-// the periodic coarsest pseudo-inverse by block elimination (work: 3 N^4 doubles); *info: bit 1 set where a pivot
-// is not positive (the result is void); false (nothing launched) where the level is too large for it
-bool launch_pinv_blocks(int N, double rho, double mu, double dt, const double* B, double* work, double* P, int* info,
-                        cudaStream_t s);
 template <typename T> void launch_coarse_apply(const double* Pinv, int n, const T* b, T* x, cudaStream_t s);
 // xo = x + omega P r (x == nullptr: 0), P dense n x n FP64: the exact level solve of a level too small
 // for the RAS boxes

@@ -1492,29 +1492,22 @@ void setup(sib_ctx* c, cudaStream_t s) {
         c->kappaDirty = false;
         c->fluidDirty = true;
     }
-    // coarsest pseudo-inverse (depends on rho, mu, dt and kappa), on the auxiliary stream beside the SC
-    // eigenvalue estimates and the box inverses below (which do not use it); the main stream joins it at the
-    // end.  Block elimination where it applies, else the blocked Gauss-Jordan.
-    auto gauss_jordan_pinv = [&](cudaStream_t q) {
+    // coarsest pseudo-inverse (depends on rho, mu, dt and kappa).  The Gauss-Jordan inversion holds
+    // one 16-block cluster for about a millisecond; it runs on the auxiliary stream, beside the SC
+    // eigenvalue estimates below (which do not use it), and the main stream joins it at the end.
+    {
         const int n = c->n0;
         if (cavity(c))
-            KL(c, launch_cavity_assemble_L0(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, q));
+            KL(c, launch_cavity_assemble_L0(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, s));
         else
-            KL(c, launch_assemble_L0(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, q));
-        KL(c, launch_gauss_jordan(c->Aug, n, c->info, c->piv, c->gjWork, q));
+            KL(c, launch_assemble_L0(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, s));
+        CK(cudaEventRecord(c->evFork, s));
+        CK(cudaStreamWaitEvent(c->aux, c->evFork, 0));
+        KL(c, launch_gauss_jordan(c->Aug, n, c->info, c->piv, c->gjWork, c->aux));
         // the gauge's Z Z^T comes off the pressure block alone in the cavity (passed as rho != 0)
-        KL(c, launch_extract_pinv(c->Aug, c->piv, n, c->L[0].N, cavity(c) ? 1.0 : c->rho, c->Pinv, q));
-    };
-    CK(cudaMemsetAsync(c->info, 0, sizeof(int), s));
-    CK(cudaEventRecord(c->evFork, s));
-    CK(cudaStreamWaitEvent(c->aux, c->evFork, 0));
-    const bool pinvBlocks = !cavity(c) && launch_pinv_blocks(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, c->Pinv,
-                                                             c->info, c->aux);
-    if (pinvBlocks)
-        c->launches += 3;
-    else
-        gauss_jordan_pinv(c->aux);
-    CK(cudaEventRecord(c->evJoin, c->aux));
+        KL(c, launch_extract_pinv(c->Aug, c->piv, n, c->L[0].N, cavity(c) ? 1.0 : c->rho, c->Pinv, c->aux));
+        CK(cudaEventRecord(c->evJoin, c->aux));
+    }
     // Vanka patch factors (they depend on the fluid parameters and the patch entries)
     for (int l = 1; l <= c->lmax; ++l) {
         Level& lv = c->L[l];
@@ -1575,11 +1568,6 @@ void setup(sib_ctx* c, cudaStream_t s) {
         int info = 0;
         CK(cudaMemcpyAsync(&info, c->info, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        if (pinvBlocks && info != 0) {   // definiteness lost to rounding: with pivoting
-            gauss_jordan_pinv(s);
-            CK(cudaMemcpyAsync(&info, c->info, sizeof(int), cudaMemcpyDeviceToHost, s));
-            CK(cudaStreamSynchronize(s));
-        }
         if (info != 0) throw SibError(SIB_ERR_ARG, "coarsest operator is singular beyond its gauge kernel");
         c->fluidDirty = false;
     }
@@ -2197,8 +2185,6 @@ int sib_create(sib_ctx** out, int N, int n_min) {
         c->piv = (int*)dalloc(c, sizeof(int) * c->n0);
         c->gjWork = dalloc(c, gauss_jordan_work_bytes(c->n0));
         c->flag = (int*)dalloc(c, sizeof(int));
-        c->binSums = (int*)dalloc(c, sizeof(int) * 2 * (size_t)bin_chunks(N * N));
-        c->binMost = (int*)dalloc(c, sizeof(int));
         const size_t n3 = 3 * (size_t)N * N;
         c->rhs = (double*)dalloc(c, sizeof(double) * n3);
         c->zcur = (double*)dalloc(c, sizeof(double) * n3);
@@ -2211,6 +2197,8 @@ int sib_create(sib_ctx** out, int N, int n_min) {
         CK(cudaMallocHost(&c->herr, 64));
         std::memset(c->herr, 0, 64);
         alloc_markers(c);
+        c->binSums = (int*)dalloc(c, sizeof(int) * 2 * (size_t)bin_chunks(N * N));
+        c->binMost = (int*)dalloc(c, sizeof(int));
     } catch (const SibError& e) {
         std::fprintf(stderr, "sib_create: %s\n", e.what());
         sib_destroy(c);
