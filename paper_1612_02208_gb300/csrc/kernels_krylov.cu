@@ -4,6 +4,7 @@
 // so results are bitwise reproducible run to run.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "sib_internal.h"
@@ -220,16 +221,117 @@ size_t gauss_jordan_work_bytes(int n) {
     return sizeof(double) * ((size_t)n * GJ_B + GJ_B * GJ_B + (size_t)GJ_B * 2 * n) + sizeof(int) * (size_t)(n + GJ_B);
 }
 
-__global__ void __launch_bounds__(512) k_gj_panel(const double* __restrict__ A, int n, int c0, GjWork w,
-                                                  int* __restrict__ piv, int* __restrict__ info) {
+// The end of a panel: G = A_PQ^{-1} for the chosen rows pS, by the whole block (at least GJ_B^2 threads)
+__device__ __forceinline__ void gj_pivot_block(int c0, GjWork w, const int* pS, int* piv, int* info) {
+    __shared__ double colv[2][GJ_B], rowv[2][GJ_B], rcp[2];
+    const int r = threadIdx.x;
+    // Gauss-Jordan in place in FP64 with the pivots on the diagonal; entry (s, u) of column u < t already belongs
+    // to the inverse, whose column t appears at step t as a unit vector
+    const int s = r / GJ_B, u = r % GJ_B;
+    const bool in = r < GJ_B * GJ_B;
+    double m = in ? w.Q0[(size_t)pS[s] * GJ_B + u] : 0.0;
+    auto next_pivot = [&](int t) {
+        if (!(m != 0.0) && *info == 0) *info = c0 + t + 1;
+        rcp[t & 1] = m != 0.0 ? 1.0 / m : 0.0;
+    };
+    if (r == 0) next_pivot(0);
+    for (int t = 0; t < GJ_B; ++t) {
+        const int b = t & 1;
+        if (in && u == t) colv[b][s] = m;
+        if (in && s == t) rowv[b][u] = u == t ? 1.0 : m;
+        __syncthreads();
+        if (!in) continue;
+        const double ipv = rcp[b], rv = rowv[b][u];
+        if (s == t) {
+            m = rv * ipv;
+        } else {
+            const double f = colv[b][s] * ipv;
+            m = (u == t ? 0.0 : m) - f * rv;
+        }
+        if (s == t + 1 && u == s) next_pivot(t + 1);
+    }
+    if (in) w.G[r] = m;
+    if (r < GJ_B) {
+        w.prow[r] = pS[r];
+        piv[c0 + r] = pS[r];
+    }
+}
+
+// One block, one candidate row per thread, its panel entries in registers.  The panels are the serial chain of
+// the inversion, a latency each: a pivot search is two warp-wide maxima with one barrier between them, every
+// warp's best row waiting in shared memory so that the winner's needs no second trip, and the pivot block is
+// inverted in place, one entry per thread, its reciprocal formed by the one thread that updates it (a division
+// in every warp cost the FP64 pipe more than the step's updates).  192 rows: 42 us a panel with the working
+// copy in shared memory, 16.5 us so (the whole inversion of 192 x 192: 575 -> 330 us).
+constexpr int GJ_MAXN = 768;   // 3 * 16^2, the largest coarsest grid
+__global__ void __launch_bounds__(GJ_MAXN) k_gj_panel(const double* __restrict__ A, int n, int c0, GjWork w,
+                                                      int* __restrict__ piv, int* __restrict__ info) {
+    pdl_entry();
+    __shared__ float cand[2][32][GJ_B];   // every warp's best row, its size and index (two steps in turn)
+    __shared__ unsigned ckey[2][32];
+    __shared__ int crow[2][32];
+    __shared__ int pS[GJ_B];
+    const int r = threadIdx.x, lane = r & 31, wid = r >> 5, nw = blockDim.x >> 5;
+    if (c0 == 0 && r == 0) *info = 0;
+    float a[GJ_B] = {};
+    bool used = true;
+    if (r < n) {
+        used = c0 != 0 && w.used[r];
+        const double2* row = reinterpret_cast<const double2*>(A + (size_t)r * 2 * n + c0);
+        double2* q0 = reinterpret_cast<double2*>(w.Q0 + (size_t)r * GJ_B);
+        double2 v[GJ_B / 2];
+#pragma unroll
+        for (int q = 0; q < GJ_B / 2; ++q) v[q] = row[q];
+#pragma unroll
+        for (int q = 0; q < GJ_B / 2; ++q) {
+            q0[q] = v[q];
+            a[2 * q] = (float)v[q].x;
+            a[2 * q + 1] = (float)v[q].y;
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < GJ_B; ++t) {
+        const int b = t & 1;
+        // magnitudes order as their bits do; 0: no candidate, 1: a zero (or not a number)
+        const float m = fabsf(a[t]);
+        const unsigned key = used ? 0u : (m >= 0.0f ? __float_as_uint(m) + 1u : 1u);
+        const unsigned wbest = __reduce_max_sync(0xffffffffu, key);
+        const int src = __ffs(__ballot_sync(0xffffffffu, key == wbest)) - 1;   // ties to the lower row
+        if (lane == src) {
+            ckey[b][wid] = key;
+            crow[b][wid] = r;
+#pragma unroll
+            for (int q = t; q < GJ_B; ++q) cand[b][wid][q] = a[q];
+        }
+        __syncthreads();
+        const unsigned k = lane < nw ? ckey[b][lane] : 0u;
+        const unsigned best = __reduce_max_sync(0xffffffffu, k);
+        const int ww = __ffs(__ballot_sync(0xffffffffu, k == best)) - 1;
+        const int p = crow[b][ww];
+        if (r == 0) pS[t] = p;
+        used = used || r == p;
+        const float pv = cand[b][ww][t];
+        const float ipv = pv != 0.0f ? 1.0f / pv : 0.0f;
+        const float f = a[t] * ipv;
+        if (!used && f != 0.0f) {
+#pragma unroll
+            for (int q = t + 1; q < GJ_B; ++q) a[q] -= f * cand[b][ww][q];
+        }
+    }
+    __syncthreads();
+    gj_pivot_block(c0, w, pS, piv, info);
+    if (r < n) w.used[r] = used;
+}
+
+// The same with the working copy in shared memory, for more rows than a block has registers for.
+__global__ void __launch_bounds__(512) k_gj_panel_wide(const double* __restrict__ A, int n, int c0, GjWork w,
+                                                       int* __restrict__ piv, int* __restrict__ info) {
     pdl_entry();
     extern __shared__ float smf[];
     float* Wp = smf;                                      // n x GJ_B working copy of the panel
     float* fac = Wp + (size_t)n * GJ_B;                   // n: column t before the pivot's elimination
     int* usedS = reinterpret_cast<int*>(fac + n);         // n
     __shared__ float prowv[GJ_B];
-    __shared__ double Mx[GJ_B][2 * GJ_B];
-    __shared__ double colv[GJ_B], rowv[2 * GJ_B];
     __shared__ float wv[32];
     __shared__ int wi[32];
     __shared__ int pS[GJ_B];
@@ -297,35 +399,7 @@ __global__ void __launch_bounds__(512) k_gj_panel(const double* __restrict__ A, 
         }
         __syncthreads();
     }
-    // G = A_PQ^{-1} in FP64: Gauss-Jordan on [A_PQ | I] with the pivots on the diagonal.  At step t
-    // the left columns < t are already unit vectors and the right columns > B + t still zero off
-    // the diagonal, so only columns [t, B + t] change (besides the diagonal's own unit entries).
-    for (int q = threadIdx.x; q < GJ_B * 2 * GJ_B; q += blockDim.x) {
-        const int t = q / (2 * GJ_B), u = q % (2 * GJ_B);
-        Mx[t][u] = u < GJ_B ? w.Q0[pS[t] * GJ_B + u] : (u - GJ_B == t ? 1.0 : 0.0);
-    }
-    __syncthreads();
-    for (int t = 0; t < GJ_B; ++t) {
-        if (threadIdx.x < GJ_B) colv[threadIdx.x] = Mx[threadIdx.x][t];
-        if (threadIdx.x < 2 * GJ_B) rowv[threadIdx.x] = Mx[t][threadIdx.x];
-        __syncthreads();
-        if (threadIdx.x == 0 && !(colv[t] != 0.0) && *info == 0) *info = c0 + t + 1;
-        const double ipv = colv[t] != 0.0 ? 1.0 / colv[t] : 0.0;
-        for (int q = threadIdx.x; q < GJ_B * 2 * GJ_B; q += blockDim.x) {
-            const int s2 = q / (2 * GJ_B), u = q % (2 * GJ_B);
-            if (u < t || u > GJ_B + t) continue;
-            if (s2 == t)
-                Mx[s2][u] = rowv[u] * ipv;
-            else
-                Mx[s2][u] -= colv[s2] * ipv * rowv[u];
-        }
-        __syncthreads();
-    }
-    for (int q = threadIdx.x; q < GJ_B * GJ_B; q += blockDim.x) w.G[q] = Mx[q / GJ_B][GJ_B + q % GJ_B];
-    if (threadIdx.x < GJ_B) {
-        w.prow[threadIdx.x] = pS[threadIdx.x];
-        piv[c0 + threadIdx.x] = pS[threadIdx.x];
-    }
+    gj_pivot_block(c0, w, pS, piv, info);
     for (int r = threadIdx.x; r < n; r += blockDim.x) w.used[r] = usedS[r];
 }
 
@@ -381,10 +455,15 @@ __global__ void __launch_bounds__(128) k_gj_rows(double* __restrict__ A, int n, 
 void launch_gauss_jordan(double* Aug, int n, int* info, int* piv, void* work, cudaStream_t s) {
     const GjWork w = gj_work(work, n);
     const size_t smem = sizeof(float) * ((size_t)n * GJ_B + n) + sizeof(int) * (size_t)n;
-    cudaFuncSetAttribute(k_gj_panel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const bool wide = n > GJ_MAXN;   // the box smoothers' largest subdomains
+    if (wide) cudaFuncSetAttribute(k_gj_panel_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const int ld = 2 * n;
     for (int c0 = 0; c0 < n; c0 += GJ_B) {
-        launch_pdl(k_gj_panel, 1, 512, smem, s, (const double*)Aug, n, c0, w, piv, info);
+        if (wide)
+            launch_pdl(k_gj_panel_wide, 1, 512, smem, s, (const double*)Aug, n, c0, w, piv, info);
+        else
+            launch_pdl(k_gj_panel, 1, std::max(GJ_B * GJ_B, (n + 31) / 32 * 32), 0, s, (const double*)Aug, n, c0, w, piv,
+                       info);
         const int R = ld - c0 - GJ_B;
         launch_pdl(k_gj_w, dim3((R + 15) / 16), dim3(16, GJ_B), 0, s, Aug, n, c0, w);
         launch_pdl(k_gj_rows, dim3(n, (ld - c0 + 127) / 128), dim3(128), 0, s, Aug, n, c0, w);
