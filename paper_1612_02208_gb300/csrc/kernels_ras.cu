@@ -17,6 +17,7 @@
 // cells wide are corrected by a persistent kernel, wider ones (the paper's 8 x 8 boxes with overlap 2
 // and up) by a batched product over tiles of boxes.
 #include <algorithm>
+#include <type_traits>
 
 #include "sib_internal.h"
 #include "tcgen05.cuh"
@@ -1547,21 +1548,25 @@ __global__ void __launch_bounds__(RAS_WB_THREADS)
 // gathers their windows into shared memory, and each warp walks owned rows: row own(r) of the shared
 // inverse, read once per block, against the RH_BX windows.  xo(owned) = x(owned) + omega c
 // (x == nullptr: 0).  Blocks along y split the owned rows (rows blockIdx.y, blockIdx.y + gridDim.y, ...
-// of the warps' walk), so that a level with few boxes still fills the GPU.
+// of the warps' walk), so that a level with few boxes still fills the GPU.  boxes != nullptr: only those `count`
+// boxes (FP32 levels, whose IB boxes are written whole afterwards: 40 us a sweep without it on the 128^2 circle's
+// levels, where most boxes are IB boxes).
 constexpr int RH_BX = 8, RH_THREADS = 256;
 template <typename T>
 __global__ void __launch_bounds__(RH_THREADS)
-    k_ras_huge_apply(RasGeo G, const T* __restrict__ inv, T omega, const T* __restrict__ r, const T* x, T* xo) {
+    k_ras_huge_apply(RasGeo G, const T* __restrict__ inv, T omega, const T* __restrict__ r, const T* x, T* xo,
+                     const int* __restrict__ boxes, int count) {
     extern __shared__ unsigned char smem_rh[];
     T* win = reinterpret_cast<T*>(smem_rh);   // RH_BX x ne
     const int N = G.N, n = N * N, m = N - 1, ne = G.ne;
-    const int nboxes = G.nbs * G.nbs, k0 = blockIdx.x * RH_BX;
+    const int k0 = blockIdx.x * RH_BX;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     pdl_entry();
     for (int t = threadIdx.x; t < RH_BX * ne; t += blockDim.x) {
-        const int j = t / ne, q = t - j * ne, kb = k0 + j;
+        const int j = t / ne, q = t - j * ne;
         T v = T(0);
-        if (kb < nboxes) {
+        if (k0 + j < count) {
+            const int kb = boxes ? boxes[k0 + j] : k0 + j;
             int comp, ii, jj;
             ras_dof(G, q, comp, ii, jj);
             const int gi = ((kb % G.nbs) * G.b - G.o + ii) & m, gj = ((kb / G.nbs) * G.b - G.o + jj) & m;
@@ -1583,12 +1588,12 @@ __global__ void __launch_bounds__(RH_THREADS)
 #pragma unroll
         for (int j = 0; j < RH_BX; ++j)
             for (int off = 16; off > 0; off >>= 1) acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], off);
-        if (lane < RH_BX && k0 + lane < nboxes) {
+        if (lane < RH_BX && k0 + lane < count) {
             T a = acc[0];
 #pragma unroll
             for (int j = 1; j < RH_BX; ++j)
                 if (lane == j) a = acc[j];
-            const int kb = k0 + lane, bb = G.b * G.b;
+            const int kb = boxes ? boxes[k0 + lane] : k0 + lane, bb = G.b * G.b;
             const int comp = rr / bb, rem = rr - comp * bb;
             const size_t d = (size_t)comp * n + (size_t)((kb / G.nbs) * G.b + rem / G.b) * N + (kb % G.nbs) * G.b +
                              rem % G.b;
@@ -1640,15 +1645,12 @@ __device__ double ras_row_dot(const RasGeo& G, const RasIB& ib, double a0, doubl
 // FP64 levels: delta_0 = M r_k is refined once against the local operator itself, delta = delta_0 +
 // M (r_k - L_k delta_0): with a stiff structure W is large and the two terms of M nearly cancel, and the
 // refinement recovers the digits they lose; then xo(owned) += omega (delta - L_0^{-1} r_k)(owned).
-// FP32 levels: the low-rank term alone, xo(owned) -= omega (L_0^{-1})_{own,T} W (L_0^{-1})_{T,:} r_k (what
-// the cancellation costs stays below FP32 rounding; m (ne + nown) flops instead of 2 ne^2).
 // L_0^{-1} is symmetric (L_0 is), so its columns T are read as rows.
-template <typename T>
 __global__ void __launch_bounds__(256)
     k_ras_wb_apply(RasGeo G, RasIB ib, double a0, double c, double inv_h, double dt, const int* __restrict__ list,
                    const int* __restrict__ offT, const int* __restrict__ Tl, const long long* __restrict__ offW,
-                   const double* __restrict__ Wd, const double* __restrict__ inv0, T omega, const T* __restrict__ r,
-                   T* xo) {
+                   const double* __restrict__ Wd, const double* __restrict__ inv0, double omega,
+                   const double* __restrict__ r, double* xo) {
     extern __shared__ double smem_wa[];
     const int N = G.N, n = N * N, mk = N - 1, ne = G.ne;
     const int k = list[blockIdx.x];
@@ -1695,33 +1697,6 @@ __global__ void __launch_bounds__(256)
         __syncthreads();
     };
     const int bb = G.b * G.b;
-    if constexpr (sizeof(T) == 4) {
-        for (int a = warp; a < m; a += nw) {   // y_T = (L_0^{-1})_{T,:} r_k
-            const double* row = inv0 + (size_t)Ts[a] * ne;
-            double acc = 0.0;
-            for (int t = lane; t < ne; t += 32) acc += row[t] * rk[t];
-            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (lane == 0) y0[a] = acc;
-        }
-        __syncthreads();
-        for (int a = warp; a < m; a += nw) {   // z = W y_T
-            const double* row = Wb + (size_t)a * m;
-            double acc = 0.0;
-            for (int t = lane; t < m; t += 32) acc += row[t] * y0[t];
-            for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-            if (lane == 0) z[a] = acc;
-        }
-        __syncthreads();
-        for (int rr = threadIdx.x; rr < G.nown; rr += blockDim.x) {
-            const double* row = inv0 + (size_t)ras_owned(G, rr) * ne;
-            double acc = 0.0;
-            for (int a = 0; a < m; ++a) acc += row[Ts[a]] * z[a];
-            const int comp = rr / bb, rem = rr - comp * bb;
-            const size_t d = (size_t)comp * n + (size_t)(J * G.b + rem / G.b) * N + I * G.b + rem % G.b;
-            xo[d] = (T)((double)xo[d] - (double)omega * acc);
-        }
-        return;
-    }
     woodbury(rk, y0, d0);
     for (int q = threadIdx.x; q < ne; q += blockDim.x)   // the residual of delta_0 in the local problem
         y1[q] = rk[q] - ras_row_dot(G, ib, a0, c, inv_h, dt, i0, j0, q, d0);
@@ -1733,7 +1708,7 @@ __global__ void __launch_bounds__(256)
         const int q = ras_owned(G, rr);
         const int comp = rr / bb, rem = rr - comp * bb;
         const size_t d = (size_t)comp * n + (size_t)(J * G.b + rem / G.b) * N + I * G.b + rem % G.b;
-        xo[d] = (T)((double)xo[d] + (double)omega * (d0[q] + rk[q] - y0[q]));
+        xo[d] = xo[d] + omega * (d0[q] + rk[q] - y0[q]);
     }
 }
 
@@ -1776,6 +1751,32 @@ void launch_ras_classify(int N, int b, int o, const RasIB& ib, int* list, int* c
 void launch_box_slots(int nboxes, const int* list, const int* count, int* slotOfBox, cudaStream_t s) {
     cudaMemsetAsync(slotOfBox, 0xff, sizeof(int) * (size_t)nboxes, s);
     k_box_slots<<<(nboxes + 255) / 256, 256, 0, s>>>(list, count, slotOfBox);
+}
+
+// the boxes without a slot, ascending; one block
+__global__ void __launch_bounds__(1024) k_ras_free_boxes(const int* __restrict__ slotOfBox, int nboxes,
+                                                         int* __restrict__ boxes) {
+    __shared__ int sums[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int base = 0;
+    for (int k0 = 0; k0 < nboxes; k0 += 1024) {
+        const int k = k0 + threadIdx.x;
+        const bool f = k < nboxes && slotOfBox[k] < 0;
+        const unsigned bal = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) sums[warp] = __popc(bal);
+        __syncthreads();
+        int before = 0, all = 0;
+        for (int w = 0; w < 32; ++w) {
+            before += w < warp ? sums[w] : 0;
+            all += sums[w];
+        }
+        if (f) boxes[base + before + __popc(bal & ((1u << lane) - 1))] = k;
+        base += all;
+        __syncthreads();
+    }
+}
+void launch_ras_free_boxes(const int* slotOfBox, int nboxes, int* boxes, cudaStream_t s) {
+    k_ras_free_boxes<<<1, 1024, 0, s>>>(slotOfBox, nboxes, boxes);
 }
 
 bool ras_block_elimination(int b, int o) { return b + 2 * o <= RAS_BE_EMAX; }
@@ -1957,7 +1958,9 @@ void launch_ras_wb_big(const double* Mx, int m, double* Aug, int* piv, void* wor
     k_ras_wb_take<<<dim3((m + 255) / 256, m), 256, 0, s>>>(Aug, piv, m, m16, Wb);
 }
 template <typename T>
-void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* r, const T* x, T* xo, cudaStream_t s) {
+void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* r, const T* x, T* xo, const int* boxes,
+                           int count, cudaStream_t s) {
+    if (count <= 0) return;
     const RasGeo G = ras_geo(N, b, o);
     const size_t smem = sizeof(T) * RH_BX * (size_t)G.ne;
     static thread_local size_t allowed = 48 * 1024;
@@ -1966,153 +1969,241 @@ void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* 
         allowed = smem;
     }
     // row splits: about two blocks per SM in all, at most one warp's row per split and warp
-    const int boxBlocks = (G.nbs * G.nbs + RH_BX - 1) / RH_BX, nw = RH_THREADS / 32;
+    const int boxBlocks = (count + RH_BX - 1) / RH_BX, nw = RH_THREADS / 32;
     const int splits = std::max(1, std::min((2 * 152 + boxBlocks - 1) / boxBlocks, (G.nown + nw - 1) / nw));
-    launch_pdl(k_ras_huge_apply<T>, dim3(boxBlocks, splits), dim3(RH_THREADS), smem, s, G, inv, omega, r, x, xo);
+    launch_pdl(k_ras_huge_apply<T>, dim3(boxBlocks, splits), dim3(RH_THREADS), smem, s, G, inv, omega, r, x, xo, boxes,
+               count);
 }
 template void launch_ras_huge_apply<float>(int, int, int, const float*, float, const float*, const float*, float*,
-                                           cudaStream_t);
+                                           const int*, int, cudaStream_t);
 template void launch_ras_huge_apply<double>(int, int, int, const double*, double, const double*, const double*,
-                                            double*, cudaStream_t);
-// FP32 levels, spread over the GPU: every IB box's local solve in three launches over (box, chunk), so
-// that the FP64 products run on every SM instead of one SM per IB box.
-//   1. y = L_0^{-1} r_k on the rows T and on the owned rows, a warp per row;
-//   2. z = W y_T, a warp per row;
-//   3. xo(owned) = x(owned) + omega (y_own - (L_0^{-1})_{own,T} z), 32 owned rows per block and eight
-//      partial sums per row, reading (L_0^{-1})_{T,own} (L_0 is symmetric) so that a warp's reads of one
-//      row of the inverse are consecutive.
-// The owned values of an IB box are written whole, from FP64 sums.  With a stiff structure the shared
-// term y_own and the low-rank term nearly cancel, and the FP32 shared correction of those rows (already
-// written by the kernel for all boxes) would carry its rounding, scaled by that cancellation, into the
-// result.
-constexpr int WB_ROWS = 32;   // rows per block in the first two launches
-template <typename T>
-__global__ void __launch_bounds__(256) k_ras_wb_y(RasGeo G, const int* __restrict__ list, const int* __restrict__ offT,
-                                                  const int* __restrict__ Tl, const double* __restrict__ inv0,
-                                                  const T* __restrict__ r, double* __restrict__ yT,
-                                                  double* __restrict__ yOwn) {
-    extern __shared__ double wb_rk[];   // ne: r_k
-    pdl_entry();   // every block waits (a block with no rows too), so completion orders the three launches
+                                            double*, const int*, int, cudaStream_t);
+// FP32 levels: every IB box's local solve M r = Q (r - P W P^T Q r), Q = L_0^{-1}, spread over the GPU in four
+// launches:
+//   0. every box's r_k in a row of its own;      1. y_T = Q_{T,:} r_k;      2. v_T = r_T - W y_T;
+//   3. xo(owned) = x(owned) + omega Q_{own,:} v, v = r_k outside T.
+// With a stiff structure the shared and the low-rank parts nearly cancel, so the sums need more than FP32.  They
+// were in FP64 (y on T and the owned rows, W y, Q_{own,T} z), bound by the FP64 pipe: 2 multiply-adds per SM and clock,
+// against 128 in FP32.  Here every value is a sum of two floats (Q and W split at set-up to 48 bits, r exact in one)
+// and every product and sum keeps its rounding error (two-product by FMA and Knuth's two-sum: Ogita, Rump and
+// Oishi's Dot2), twelve FP32 operations for one in FP64.  The rounding left is 2^-46 or so of the terms, and the
+// result is rounded to FP32 as before: one sweep's error against FP64 levels is the same to five digits from
+// gamma = 5 to 500 on 32^2 to 128^2, circle and annulus (2e-8 to 7e-8).
+// A block holds the vectors of WB_BX boxes in shared memory, and a warp takes a row of Q for those of them that need
+// it, so that Q, 25 MB in all, is read from L2 once per group and not once per box; eight elements a lane at a time,
+// whose sums overlap.
+// 128^2 circle, 16 x 16 boxes with overlap 4, with the IB-free boxes listed (k_ras_huge_apply): solve 25.9 -> 11.1 ms.
+struct TwoFloat {
+    float s, c;
+};
+// (s, c) += p + e, exact in s; c collects the errors
+__device__ __forceinline__ void tf_add(TwoFloat& a, float p, float e) {
+    const float t = __fadd_rn(a.s, p), z = __fsub_rn(t, a.s);
+    const float d = __fadd_rn(__fsub_rn(a.s, __fsub_rn(t, z)), __fsub_rn(p, z));
+    a.s = t;
+    a.c = __fadd_rn(a.c, __fadd_rn(d, e));
+}
+// a += (q.x + q.y) v and a += (q.x + q.y) (v.x + v.y)
+__device__ __forceinline__ void tf_fma(TwoFloat& a, float2 q, float v) {
+    const float p = __fmul_rn(q.x, v);
+    tf_add(a, p, __fmaf_rn(q.x, v, -p));
+    a.c = __fmaf_rn(q.y, v, a.c);
+}
+__device__ __forceinline__ void tf_fma(TwoFloat& a, float2 q, float2 v) {
+    const float p = __fmul_rn(q.x, v.x);
+    tf_add(a, p, __fmaf_rn(q.x, v.x, -p));
+    a.c = __fmaf_rn(q.y, v.x, __fmaf_rn(q.x, v.y, a.c));
+}
+__device__ __forceinline__ void tf_warp_sum(TwoFloat& a) {
+    for (int off = 16; off > 0; off >>= 1) {
+        const float os = __shfl_xor_sync(0xffffffffu, a.s, off), oc = __shfl_xor_sync(0xffffffffu, a.c, off);
+        tf_add(a, os, oc);
+    }
+}
+__device__ __forceinline__ float2 tf_normal(TwoFloat a) {   // the nearest float, and the rest
+    const float h = __fadd_rn(a.s, a.c);
+    return make_float2(h, __fsub_rn(a.c, __fsub_rn(h, a.s)));
+}
+// rows of `len` values as pairs of floats, a row `stride` pairs apart, the rest of it zero
+__global__ void k_ras_split(const double* __restrict__ in, size_t rows, int len, int stride, float2* __restrict__ out) {
+    for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < rows * stride; t += (size_t)gridDim.x * blockDim.x) {
+        const size_t r = t / stride;
+        const int q = (int)(t - r * stride);
+        const double v = q < len ? in[r * len + q] : 0.0;
+        const float h = (float)v;
+        out[t] = make_float2(h, (float)(v - (double)h));
+    }
+}
+// pos[box][q]: place of subdomain dof q among the box's T (the caller sets all to -1: not in T)
+__global__ void k_ras_wb_pos(const int* __restrict__ offT, const int* __restrict__ Tl, int ne, int* __restrict__ pos) {
     const int t0 = offT[blockIdx.x], m = offT[blockIdx.x + 1] - t0;
-    const int a0 = blockIdx.y * WB_ROWS;   // rows a < m: T; a >= m: owned row a - m
-    if (a0 >= m + G.nown) return;
-    const int N = G.N, n = N * N, mk = N - 1, ne = G.ne;
+    for (int a = threadIdx.x; a < m; a += blockDim.x) pos[(size_t)blockIdx.x * ne + Tl[t0 + a]] = a;
+}
+
+constexpr int WB_ROWS = 32;      // rows per block in launch 2
+constexpr int WB_BX = 8;         // boxes per block in launches 1 and 3
+constexpr int WB_THREADS = 512;
+constexpr int WB_U = 8;          // elements per lane and step
+__host__ __device__ inline int wb_stride(int ne) { return (ne + 32 * WB_U - 1) / (32 * WB_U) * (32 * WB_U); }
+// Launch 0: block (box, 256 dofs); rk and v hold wb_stride values per box, zero past ne
+__global__ void __launch_bounds__(256) k_ras_wb_gather(RasGeo G, const int* __restrict__ list, const float* __restrict__ r,
+                                                       float* __restrict__ rk, float2* __restrict__ v) {
+    const int N = G.N, n = N * N, mk = N - 1, st = wb_stride(G.ne), q = blockIdx.y * 256 + threadIdx.x;
     const int k = list[blockIdx.x];
-    const int I = k % G.nbs, J = k / G.nbs, i0 = I * G.b - G.o, j0 = J * G.b - G.o;
-    const int* Ts = Tl + t0;
+    int comp = 0, ii = 0, jj = 0;
+    if (q < G.ne) ras_dof(G, q, comp, ii, jj);
+    pdl_entry();
+    float x = 0.0f;
+    if (q < G.ne)
+        x = r[(size_t)comp * n + (size_t)(((k / G.nbs) * G.b - G.o + jj) & mk) * N + (((k % G.nbs) * G.b - G.o + ii) & mk)];
+    rk[(size_t)blockIdx.x * st + q] = x;
+    v[(size_t)blockIdx.x * st + q] = make_float2(x, 0.0f);
+}
+// Launches 1 (OWN = false: rows of T, vectors rk) and 3 (OWN = true: owned rows, vectors v); block (group of
+// WB_BX boxes, `rows` rows of Q)
+template <bool OWN>
+__global__ void __launch_bounds__(WB_THREADS) k_ras_wb_rows(RasGeo G, const int* __restrict__ list, int nIB, int rows,
+                                                           const int* __restrict__ offT, const int* __restrict__ pos,
+                                                           const float2* __restrict__ Q, const void* __restrict__ vec,
+                                                           float2* __restrict__ yT, float omega, const float* x,
+                                                           float* xo) {
+    using V = typename std::conditional<OWN, float2, float>::type;
+    extern __shared__ float4 wb_smem[];
+    const V* v = reinterpret_cast<const V*>(wb_smem);   // WB_BX x st
+    const int N = G.N, n = N * N, ne = G.ne, st = wb_stride(ne), k0 = blockIdx.x * WB_BX;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int q = threadIdx.x; q < ne; q += blockDim.x) {
-        int comp, ii, jj;
-        ras_dof(G, q, comp, ii, jj);
-        wb_rk[q] = (double)r[(size_t)comp * n + (size_t)((j0 + jj) & mk) * N + ((i0 + ii) & mk)];
+    const int total = OWN ? G.nown : 2 * G.e * (G.e + 1);   // T holds velocity dofs only
+    const int a0 = blockIdx.y * rows, a1 = min(total, a0 + rows);
+    pdl_entry();
+    {
+        const float4* src = reinterpret_cast<const float4*>(static_cast<const V*>(vec) + (size_t)k0 * st);
+        const int per = st * (int)sizeof(V) / 16, have = min(WB_BX, nIB - k0) * per;
+#pragma unroll 7
+        for (int t = threadIdx.x; t < WB_BX * per; t += WB_THREADS)
+            wb_smem[t] = t < have ? src[t] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     __syncthreads();
-    const int a1 = min(m + G.nown, a0 + WB_ROWS);
     for (int a = a0 + warp; a < a1; a += nw) {
-        const double* row = inv0 + (size_t)(a < m ? Ts[a] : ras_owned(G, a - m)) * ne;
-        double acc = 0.0;
-        for (int t = lane; t < ne; t += 32) acc += row[t] * wb_rk[t];
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) {
-            if (a < m)
-                yT[t0 + a] = acc;
-            else
-                yOwn[(size_t)blockIdx.x * G.nown + (a - m)] = acc;
+        const int q = OWN ? ras_owned(G, a) : a;
+        // the boxes that need this row, and the row's place in them (lane j: box j)
+        int p = -1;
+        if (lane < WB_BX && k0 + lane < nIB) p = OWN ? 0 : pos[(size_t)(k0 + lane) * ne + q];
+        const unsigned need = __ballot_sync(0xffffffffu, p >= 0);
+        if (need == 0) continue;
+        const float2* row = Q + (size_t)q * st;
+        TwoFloat acc[WB_BX] = {};
+        for (int t0 = lane; t0 < st; t0 += 32 * WB_U) {
+            float2 e[WB_U];
+#pragma unroll
+            for (int u = 0; u < WB_U; ++u) e[u] = row[t0 + 32 * u];
+#pragma unroll
+            for (int j = 0; j < WB_BX; ++j)
+                if (need >> j & 1) {
+#pragma unroll
+                    for (int u = 0; u < WB_U; ++u) tf_fma(acc[j], e[u], v[j * st + t0 + 32 * u]);
+                }
+        }
+        TwoFloat mine{};
+#pragma unroll
+        for (int j = 0; j < WB_BX; ++j)
+            if (need >> j & 1) {
+                tf_warp_sum(acc[j]);
+                if (lane == j) mine = acc[j];
+            }
+        if (p < 0) continue;
+        if constexpr (OWN) {
+            const int k = list[k0 + lane], bb = G.b * G.b, comp = a / bb, rem = a - comp * bb;
+            const size_t d = (size_t)comp * n + (size_t)((k / G.nbs) * G.b + rem / G.b) * N + (k % G.nbs) * G.b + rem % G.b;
+            const double delta = (double)mine.s + (double)mine.c;
+            xo[d] = (float)((x ? (double)x[d] : 0.0) + (double)omega * delta);
+        } else {
+            yT[offT[k0 + lane] + p] = tf_normal(mine);
         }
     }
 }
-__global__ void __launch_bounds__(256) k_ras_wb_z(const int* __restrict__ offT, const long long* __restrict__ offW,
-                                                  const double* __restrict__ Wd, const double* __restrict__ yT,
-                                                  double* __restrict__ z) {
+// Launch 2: block (box, WB_ROWS rows of W), a warp per row; v_T = r_T - W y_T into the box's row of v
+__global__ void __launch_bounds__(256) k_ras_wb_z(int st, const int* __restrict__ offT, const int* __restrict__ Tl,
+                                                  const long long* __restrict__ offW, const float2* __restrict__ W,
+                                                  const float* __restrict__ rk, const float2* __restrict__ yT,
+                                                  float2* __restrict__ v) {
     pdl_entry();
     const int t0 = offT[blockIdx.x], m = offT[blockIdx.x + 1] - t0;
     const int a0 = blockIdx.y * WB_ROWS;
     if (a0 >= m) return;
-    const double* Wb = Wd + offW[blockIdx.x];
+    const float2* Wb = W + offW[blockIdx.x];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int a1 = min(m, a0 + WB_ROWS);
     for (int a = a0 + warp; a < a1; a += nw) {
-        const double* row = Wb + (size_t)a * m;
-        double acc = 0.0;
-        for (int t = lane; t < m; t += 32) acc += row[t] * yT[t0 + t];
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) z[t0 + a] = acc;
+        const float2* row = Wb + (size_t)a * m;
+        TwoFloat acc{};
+#pragma unroll 8
+        for (int t = lane; t < m; t += 32) tf_fma(acc, row[t], yT[t0 + t]);
+        tf_warp_sum(acc);
+        if (lane == 0) {
+            const size_t d = (size_t)blockIdx.x * st + Tl[t0 + a];
+            TwoFloat s{rk[d], 0.0f};
+            tf_add(s, -acc.s, -acc.c);
+            v[d] = tf_normal(s);
+        }
     }
 }
-template <typename T>
-__global__ void __launch_bounds__(256) k_ras_wb_out(RasGeo G, const int* __restrict__ list, const int* __restrict__ offT,
-                                                    const int* __restrict__ Tl, const double* __restrict__ inv0,
-                                                    const double* __restrict__ z, const double* __restrict__ yOwn,
-                                                    T omega, const T* x, T* xo) {
-    // 32 owned rows per block; warp w sums the terms a = w, w + 8, ... of each row (lane = row), and
-    // the eight partial sums are added in warp order
-    __shared__ double part[8][32];
-    pdl_entry();
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int rr = blockIdx.y * 32 + lane;
-    const bool live = rr < G.nown;
-    const int N = G.N, n = N * N, ne = G.ne, bb = G.b * G.b;
-    const int t0 = offT[blockIdx.x], m = offT[blockIdx.x + 1] - t0;
-    const int* Ts = Tl + t0;
-    const int q = live ? ras_owned(G, rr) : 0;
-    double acc = 0.0;
-    if (live)
-        for (int a = w; a < m; a += 8) acc += inv0[(size_t)Ts[a] * ne + q] * z[t0 + a];
-    part[w][lane] = acc;
-    __syncthreads();
-    if (w != 0 || !live) return;
-    double sum = part[0][lane];
-#pragma unroll
-    for (int v = 1; v < 8; ++v) sum += part[v][lane];
-    const int k = list[blockIdx.x];
-    const int I = k % G.nbs, J = k / G.nbs;
-    const int comp = rr / bb, rem = rr - comp * bb;
-    const size_t d = (size_t)comp * n + (size_t)(J * G.b + rem / G.b) * N + I * G.b + rem % G.b;
-    const double delta = yOwn[(size_t)blockIdx.x * G.nown + rr] - sum;
-    xo[d] = (T)((x ? (double)x[d] : 0.0) + (double)omega * delta);
+size_t ras_wb_row(int b, int o) { return wb_stride(ras_ne(b, o)); }
+void launch_ras_wb_split(int b, int o, const double* inv0, void* Qs, const double* W, size_t nW, void* Ws, int nIB,
+                         const int* offT, const int* Tl, int* pos, cudaStream_t s) {
+    const int ne = ras_ne(b, o);
+    k_ras_split<<<304, 256, 0, s>>>(inv0, ne, ne, wb_stride(ne), static_cast<float2*>(Qs));
+    k_ras_split<<<304, 256, 0, s>>>(W, nW, 1, 1, static_cast<float2*>(Ws));
+    cudaMemsetAsync(pos, 0xff, sizeof(int) * ne * (size_t)nIB, s);
+    k_ras_wb_pos<<<nIB, 256, 0, s>>>(offT, Tl, ne, pos);
 }
-
-template <typename T>
-void launch_ras_wb_apply(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
-                         const int* list, int nIB, const int* offT, const int* Tl, const long long* offW,
-                         const double* W, const double* inv0, int mmax, T omega, const T* r, T* xo, cudaStream_t s,
-                         double* scratch, const T* x) {
+void launch_ras_wb_apply32(int N, int b, int o, const int* list, int nIB, const int* offT, const int* Tl,
+                           const long long* offW, const void* Ws, const void* Qs, const int* pos, int mmax, float omega,
+                           const float* r, const float* x, float* xo, double* scratch, cudaStream_t s) {
     if (nIB <= 0) return;
     const RasGeo G = ras_geo(N, b, o);
-    if (sizeof(T) == 4 && scratch) {   // FP32: the IB boxes' local solves over the whole GPU
-        // the caller's scratch holds (2 mmax + nown) nIB values
-        double* yT = scratch;
-        double* z = scratch + (size_t)mmax * nIB;
-        double* yOwn = z + (size_t)mmax * nIB;
-        const int chunks = (mmax + WB_ROWS - 1) / WB_ROWS, chunksY = (mmax + G.nown + WB_ROWS - 1) / WB_ROWS;
-        const size_t smem = sizeof(double) * (size_t)G.ne;
-        static thread_local size_t allowedY = 48 * 1024;
-        if (smem > allowedY) {
-            cudaFuncSetAttribute(k_ras_wb_y<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            allowedY = smem;
-        }
-        launch_pdl(k_ras_wb_y<T>, dim3(nIB, chunksY), dim3(256), smem, s, G, list, offT, Tl, inv0, r, yT, yOwn);
-        launch_pdl(k_ras_wb_z, dim3(nIB, chunks), dim3(256), 0, s, offT, offW, W, (const double*)yT, z);
-        launch_pdl(k_ras_wb_out<T>, dim3(nIB, (G.nown + 31) / 32), dim3(256), 0, s, G, list, offT, Tl, inv0,
-                   (const double*)z, (const double*)yOwn, omega, x, xo);
-        return;
+    const int st = wb_stride(G.ne);
+    const float2* Q = static_cast<const float2*>(Qs);
+    float2* v = reinterpret_cast<float2*>(scratch);
+    float* rk = reinterpret_cast<float*>(v + (size_t)st * nIB);
+    float2* yT = reinterpret_cast<float2*>(rk + (size_t)st * nIB);
+    const int groups = (nIB + WB_BX - 1) / WB_BX, nw = WB_THREADS / 32;
+    const size_t smem1 = sizeof(float) * WB_BX * (size_t)st, smem3 = 2 * smem1;
+    static thread_local size_t allowed = 0;
+    if (smem3 > allowed) {
+        cudaFuncSetAttribute(k_ras_wb_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
+        cudaFuncSetAttribute(k_ras_wb_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem3);
+        allowed = smem3;
     }
+    // rows per block: one wave of the blocks that shared memory lets an SM hold, a row per warp at least
+    auto rows_for = [&](int total, int perSM) {
+        const int blocks = std::max(1, perSM * 152 / groups);
+        return ((total + blocks - 1) / blocks + nw - 1) / nw * nw;
+    };
+    const int nv = 2 * G.e * (G.e + 1), r1 = rows_for(nv, 2), r3 = rows_for(G.nown, 1);
+    launch_pdl(k_ras_wb_gather, dim3(nIB, st / 256), dim3(256), 0, s, G, list, r, rk, v);
+    launch_pdl(k_ras_wb_rows<false>, dim3(groups, (nv + r1 - 1) / r1), dim3(WB_THREADS), smem1, s, G, list, nIB, r1,
+               offT, pos, Q, (const void*)rk, yT, omega, x, xo);
+    launch_pdl(k_ras_wb_z, dim3(nIB, (mmax + WB_ROWS - 1) / WB_ROWS), dim3(256), 0, s, st, offT, Tl, offW,
+               static_cast<const float2*>(Ws), (const float*)rk, (const float2*)yT, v);
+    launch_pdl(k_ras_wb_rows<true>, dim3(groups, (G.nown + r3 - 1) / r3), dim3(WB_THREADS), smem3, s, G, list, nIB, r3,
+               offT, pos, Q, (const void*)v, yT, omega, x, xo);
+}
+
+void launch_ras_wb_apply64(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
+                           const int* list, int nIB, const int* offT, const int* Tl, const long long* offW,
+                           const double* W, const double* inv0, int mmax, double omega, const double* r, double* xo,
+                           cudaStream_t s) {
+    if (nIB <= 0) return;
+    const RasGeo G = ras_geo(N, b, o);
     const size_t smem = sizeof(double) * (4 * (size_t)G.ne + (size_t)mmax);
     static thread_local size_t allowed = 48 * 1024;
     if (smem > allowed) {
-        cudaFuncSetAttribute(k_ras_wb_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(k_ras_wb_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         allowed = smem;
     }
-    launch_pdl(k_ras_wb_apply<T>, dim3(nIB), dim3(256), smem, s, G, ib, a0, c, inv_h, dt, list, offT, Tl, offW, W,
+    launch_pdl(k_ras_wb_apply, dim3(nIB), dim3(256), smem, s, G, ib, a0, c, inv_h, dt, list, offT, Tl, offW, W,
                inv0, omega, r, xo);
 }
-template void launch_ras_wb_apply<float>(int, int, int, const RasIB&, double, double, double, double, const int*, int,
-                                         const int*, const int*, const long long*, const double*, const double*, int,
-                                         float, const float*, float*, cudaStream_t, double*, const float*);
-template void launch_ras_wb_apply<double>(int, int, int, const RasIB&, double, double, double, double, const int*,
-                                          int, const int*, const int*, const long long*, const double*,
-                                          const double*, int, double, const double*, double*, cudaStream_t, double*,
-                                          const double*);
 size_t ras_tc_group_floats(int b, int o) {
     const RasGeo G = ras_geo(16, b, o);
     const int nch = (G.ne + RT_KC - 1) / RT_KC;

@@ -178,14 +178,23 @@ constexpr int RAS_WB_ONE_MAX = 256;
 void launch_ras_wb_big(const double* Mx, int m, double* Aug, int* piv, void* work, int* info, double* Wb,
                        cudaStream_t s);
 template <typename T>
-void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* r, const T* x, T* xo, cudaStream_t s);
-template <typename T>
-void launch_ras_wb_apply(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
-                         const int* list, int nIB, const int* offT, const int* Tl, const long long* offW,
-                         const double* W, const double* inv0, int mmax, T omega, const T* r, T* xo, cudaStream_t s,
-                         double* scratch = nullptr, const T* x = nullptr);
-// (FP32 with scratch, (2 mmax + 3 b^2) nIB values: three launches, which write the IB boxes' owned values
-// whole from x, distinct from xo; x == nullptr: zero)
+void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* r, const T* x, T* xo, const int* boxes,
+                           int count, cudaStream_t s);
+void launch_ras_free_boxes(const int* slotOfBox, int nboxes, int* boxes, cudaStream_t s);
+// FP64 levels: the IB boxes' update of the shared correction in xo
+void launch_ras_wb_apply64(int N, int b, int o, const RasIB& ib, double a0, double c, double inv_h, double dt,
+                           const int* list, int nIB, const int* offT, const int* Tl, const long long* offW,
+                           const double* W, const double* inv0, int mmax, double omega, const double* r, double* xo,
+                           cudaStream_t s);
+// FP32 levels: the shared inverse and W as pairs of floats (Qs: ne rows of ras_wb_row pairs, Ws: nW pairs) and the
+// place of every subdomain dof among a box's T (pos: nIB x ne), from which four launches write the IB boxes' owned
+// values of xo whole (scratch: (2 ras_wb_row + mmax) nIB values; x == nullptr: zero)
+size_t ras_wb_row(int b, int o);
+void launch_ras_wb_split(int b, int o, const double* inv0, void* Qs, const double* W, size_t nW, void* Ws, int nIB,
+                         const int* offT, const int* Tl, int* pos, cudaStream_t s);
+void launch_ras_wb_apply32(int N, int b, int o, const int* list, int nIB, const int* offT, const int* Tl,
+                           const long long* offW, const void* Ws, const void* Qs, const int* pos, int mmax, float omega,
+                           const float* r, const float* x, float* xo, double* scratch, cudaStream_t s);
 size_t ras_tc_group_floats(int b, int o);
 void launch_ras_tc_pack_rows(int b, int o, const double* inv0, int g, float* out, cudaStream_t s);
 // the 16 x 16 boxes' shared correction on the tensor cores, all `groups` row groups of RAS_TC_GROUP owned

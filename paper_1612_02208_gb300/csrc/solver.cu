@@ -100,6 +100,7 @@ struct Level {
     void* rasInv[2] = {nullptr, nullptr};
     size_t rasInvCap = 0;                // entries
     int rasNIB = 0;                      // boxes with their own inverse
+    int* rasFree = nullptr;              // 16 x 16 boxes: the others
     float* rasTC = nullptr;              // the shared inverse packed for the tensor-core correction
     size_t rasTCCap = 0;                 // floats
     // a level too small for the boxes: the exact level solve (gauge-fixed pseudo-inverse, FP64)
@@ -111,7 +112,10 @@ struct Level {
     int* wbT = nullptr;                  // the IB-touched local dofs of every IB box, ascending
     long long* wbOffW = nullptr;         // nIB offsets into wbW
     double* wbW = nullptr;               // W = (I + E Q)^-1 E per IB box
-    double* wbScratch = nullptr;         // (2 mmax + 3 b^2) nIB: y_T, z and y_own of the FP32 levels' IB boxes
+    void* hugeSplit = nullptr;           // the shared inverse and W as pairs of floats, for the FP32 levels
+    void* wbWs = nullptr;
+    int* wbPos = nullptr;                // nIB x ne: place of every subdomain dof among the box's T, or -1
+    double* wbScratch = nullptr;         // vectors of the FP32 levels' IB boxes
     int wbMmax = 0;                      // largest |T|
 };
 
@@ -577,14 +581,23 @@ void ras_apply(sib_ctx* c, int l, const T* r, const T* x, T* xo, double omega, c
                                               (const float*)r, (const float*)x, (float*)xo, c->herr, s);
             if (done) ++c->launches;
         }
-        if (!done) KL(c, launch_ras_huge_apply<T>(lv.N, b, o, (const T*)lv.hugeInv[pi], (T)omega, r, x, xo, s));
+        const int nboxes = (lv.N / b) * (lv.N / b);
+        const bool some = Prec<T>::id == 1 && lv.rasNIB > 0;   // the FP32 update below writes the IB boxes whole
+        if (!done && !(some && lv.rasNIB == nboxes))
+            KL(c, launch_ras_huge_apply<T>(lv.N, b, o, (const T*)lv.hugeInv[pi], (T)omega, r, x, xo,
+                                           some ? lv.rasFree : nullptr, some ? nboxes - lv.rasNIB : nboxes, s));
         if (lv.rasNIB > 0) {
-            const RasIB ib{lv.slotOf, (const double*)lv.win[0], lv.tx, lv.ty, lv.ntx};
-            const double h = lv.h, a0 = c->rho / c->dt + 4.0 * c->mu / (h * h), cc = c->mu / (h * h);
-            KL(c, launch_ras_wb_apply<T>(lv.N, b, o, ib, a0, cc, 1.0 / h, c->dt, lv.rasList, lv.rasNIB, lv.wbOffT,
-                                         lv.wbT, lv.wbOffW, lv.wbW, (const double*)lv.hugeInv[0], lv.wbMmax,
-                                         (T)omega, r, xo, s, lv.wbScratch, x));
-            if (Prec<T>::id == 1) c->launches += 2;   // the FP32 form is three launches
+            if constexpr (Prec<T>::id == 1) {
+                launch_ras_wb_apply32(lv.N, b, o, lv.rasList, lv.rasNIB, lv.wbOffT, lv.wbT, lv.wbOffW, lv.wbWs,
+                                      lv.hugeSplit, lv.wbPos, lv.wbMmax, omega, r, x, xo, lv.wbScratch, s);
+                c->launches += 4;
+            } else {
+                const RasIB ib{lv.slotOf, (const double*)lv.win[0], lv.tx, lv.ty, lv.ntx};
+                const double h = lv.h, a0 = c->rho / c->dt + 4.0 * c->mu / (h * h), cc = c->mu / (h * h);
+                KL(c, launch_ras_wb_apply64(lv.N, b, o, ib, a0, cc, 1.0 / h, c->dt, lv.rasList, lv.rasNIB, lv.wbOffT,
+                                            lv.wbT, lv.wbOffW, lv.wbW, (const double*)lv.hugeInv[0], lv.wbMmax, omega,
+                                            r, xo, s));
+            }
         }
         return;
     }
@@ -1131,7 +1144,12 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     dfree(c, lv.wbOffW);
     dfree(c, lv.wbW);
     dfree(c, lv.wbScratch);
+    dfree(c, lv.hugeSplit);
+    dfree(c, lv.wbWs);
+    dfree(c, lv.wbPos);
     lv.wbScratch = nullptr;
+    lv.hugeSplit = lv.wbWs = nullptr;
+    lv.wbPos = nullptr;
     lv.wbOffT = nullptr;
     lv.wbT = nullptr;
     lv.wbOffW = nullptr;
@@ -1157,7 +1175,10 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     lv.wbOffW = (long long*)dalloc(c, sizeof(long long) * (size_t)nIB);
     lv.wbT = (int*)dalloc(c, sizeof(int) * (size_t)std::max(1, offT[nIB]));
     lv.wbW = (double*)dalloc(c, sizeof(double) * (size_t)std::max(1LL, wTot));
-    lv.wbScratch = (double*)dalloc(c, sizeof(double) * (2 * (size_t)std::max(1, lv.wbMmax) + 3 * (size_t)b * b) * nIB);
+    lv.wbScratch = (double*)dalloc(c, sizeof(double) * (2 * ras_wb_row(b, o) + (size_t)lv.wbMmax) * nIB);
+    lv.hugeSplit = dalloc(c, 2 * sizeof(float) * (size_t)ne * ras_wb_row(b, o));
+    lv.wbWs = dalloc(c, 2 * sizeof(float) * (size_t)std::max(1LL, wTot));
+    lv.wbPos = (int*)dalloc(c, sizeof(int) * (size_t)ne * nIB);
     double* wwork = (double*)dalloc(c, sizeof(double) * (size_t)std::max(1LL, 2 * wTot));
     tmp.push_back(wwork);
     CK(cudaMemcpyAsync(lv.wbOffT, offT.data(), sizeof(int) * (size_t)(nIB + 1), cudaMemcpyHostToDevice, s));
@@ -1182,8 +1203,10 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
                 c->launches += 2 + 3 * ((cnt[k] + 15) / 16);
             }
     }
+    launch_ras_wb_split(b, o, (const double*)lv.hugeInv[0], lv.hugeSplit, lv.wbW, (size_t)wTot, lv.wbWs, nIB, lv.wbOffT,
+                        lv.wbT, lv.wbPos, s);
     CK(cudaStreamSynchronize(s));   // the host vectors above are the copies' sources
-    c->launches += 3;
+    c->launches += 6;
 }
 
 // The owned rows of every box inverse of the levels that take boxes: by block elimination (be), the levels
@@ -1249,6 +1272,8 @@ void ras_setup_all(sib_ctx* c, cudaStream_t s) {
         if (nboxes > lv.rasBoxCap) {
             dfree(c, lv.rasList);
             dfree(c, lv.rasSlot);
+            dfree(c, lv.rasFree);
+            lv.rasFree = (int*)dalloc(c, sizeof(int) * nboxes);
             lv.rasList = (int*)dalloc(c, sizeof(int) * nboxes);
             lv.rasSlot = (int*)dalloc(c, sizeof(int) * nboxes);
             lv.rasBoxCap = nboxes;
@@ -1275,6 +1300,7 @@ void ras_setup_all(sib_ctx* c, cudaStream_t s) {
         launch_box_slots(nboxes, lv.rasList, lv.rasCount, lv.rasSlot, s);
         ++c->launches;
         if (huge) {
+            KL(c, launch_ras_free_boxes(lv.rasSlot, nboxes, lv.rasFree, s));
             ras_huge_setup(c, l, cnt[l], tmp, ginfo, s);
             continue;
         }

@@ -106,3 +106,20 @@ def test_coarse_levels(make, n_min):
     b = rand(3 * n_min * n_min, 7500)
     assert rel(host(S.coarse_solve(cu(b))), H.coarse_pinv @ b) < TOL64
     S.close()
+
+
+# 16 x 16 boxes in FP32 on levels with a whole and with a partial group of eight IB boxes, and with boxes
+# that have none: the correction of a residual that FP32 holds exactly (a sweep from zero) against the FP64
+# level's, to the repository's FP32 bar
+@pytest.mark.parametrize("kind,N,gamma,o", [("circle", 64, 50.0, 4), ("circle", 128, 500.0, 4), ("annulus", 128, 5.0, 4),
+                                            ("circle", 128, 50.0, 2)])
+def test_wide_boxes_in_pairs_of_floats(kind, N, gamma, o):
+    S = sib.solver_for(I.paper_problem(kind, N, gamma), smoother=sib.SMOOTHER_RAS, box=16, box_overlap=o)
+    for l in range(1, S.num_levels):
+        n3 = 3 * (8 << l) ** 2
+        b = rand(n3, 7700 + l).astype(np.float32)
+        y32, y64 = cu(np.zeros(n3), torch.float32), cu(np.zeros(n3))
+        S.smooth(l, y32, cu(b, torch.float32), 1)
+        S.smooth(l, y64, cu(b.astype(np.float64)), 1)
+        assert rel(host(y32), host(y64)) < TOL32, l
+    S.close()
