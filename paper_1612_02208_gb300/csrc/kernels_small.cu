@@ -13,6 +13,8 @@
 // in the same order, on shared-memory copies of the same arrays.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "grid_cells.cuh"
 
 namespace cg = cooperative_groups;
@@ -350,7 +352,314 @@ __global__ void __launch_bounds__(NT, 1) k_vcycle_small(const __grid_constant__ 
     block_copy16(a.out, x, sizeof(T) * 3 * n);
 }
 
+// ------------------------------------------------------------------------------------------
+// The levels of up to 32 x 32 cells and the coarsest solve in one cluster of eight blocks (FP32, Vanka).
+//
+// As separate launches a 32 x 32 level is ten dependent kernels of 2 to 3 us, and k_vcycle_small runs 16 x 16
+// on one SM while seven wait: together 53 of the 133 us of a 128^2 solve's iteration.  Here every level is cut into
+// eight strips of rows, one per block, held in shared memory with the strip's patch factors and IB windows; a
+// neighbour's row is read from its block's shared memory, and a step ends with a cluster barrier (two a
+// sweep).  Bound by the latency of those steps and barriers, about 0.3 us each; eight blocks are the portable
+// cluster, and with them a block's share of a full 32 x 32 level's windows, 83 KB, fits beside the rest.
+// 32^2 ellipse: solve 1.51 -> 1.16 ms; 128^2 disk: 2.53 -> 2.33 ms (the windows still copied through registers; cp.async since).
+// The formulas are those of the per-level kernels in the same order.  FP64 levels keep the kernels above: eight
+// SMs' FP64 pipes are slower than the launches.
+constexpr int CV_T = 576, CV_WR8 = 2 * WR;   // 576: nine window rows of the 64 face vectors of a 32 x 32 strip
+__device__ __forceinline__ const float* cv_at(cg::cluster_group& cl, float* p, int rank) {
+    return cl.map_shared_rank(p, rank);
+}
+
+// 16 bytes to shared memory without a stop in a register (zero without `real`)
+__device__ __forceinline__ void cv_copy16(void* dst, const void* src, bool real) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(real ? 16 : 0)
+                 : "memory");
+}
+
+// r = b - L x on the block's strip
+__device__ __forceinline__ void cv_residual(cg::cluster_group& cl, const ClusterArgs& a, const ClusterLevel& L, float* sm,
+                                            int rank) {
+    const int N = L.N, m = N - 1, R = N / SMALL_CLUSTER, RN = R * N, lgR = L.lgN - 3, j0 = rank * R;
+    const float* part = sm + a.part;
+    if (L.ib) {   // u and v with a halo of WR, then the window rows of four faces a thread
+        const int W = N + CV_WR8, H = R + CV_WR8, nf = 2 * RN;
+        float* uh = sm + a.uh;
+        for (int t = threadIdx.x; t < 2 * H * W; t += CV_T) {
+            const int c = t >= H * W, q = t - c * H * W, jj = q / W, j = (j0 - WR + jj) & m, i = (q - jj * W - WR) & m;
+            uh[t] = *cv_at(cl, sm + L.x + c * RN + ((j & (R - 1)) << L.lgN) + i, j >> lgR);
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < WD * nf / 4; t += CV_T) {
+            const int oy = t / (nf / 4), f = (t - oy * (nf / 4)) * 4, c = f >= RN, q = f - c * RN;
+            const int lj = q >> L.lgN, i = q & m;
+            const float4* u4 = reinterpret_cast<const float4*>(uh + (c * H + lj + oy) * W + i);
+            float u[4 + CV_WR8];
+#pragma unroll
+            for (int v = 0; v < (4 + CV_WR8) / 4; ++v) {
+                const float4 x = u4[v];
+                u[4 * v] = x.x, u[4 * v + 1] = x.y, u[4 * v + 2] = x.z, u[4 * v + 3] = x.w;
+            }
+            const float* w = sm + L.wins + (size_t)oy * WD * nf + f;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int ox = 0; ox < WD; ++ox) {
+                const float4 k = *reinterpret_cast<const float4*>(w + ox * nf);
+                acc.x += k.x * u[ox], acc.y += k.y * u[ox + 1], acc.z += k.z * u[ox + 2], acc.w += k.w * u[ox + 3];
+            }
+            *reinterpret_cast<float4*>(sm + a.part + oy * nf + f) = acc;
+        }
+        __syncthreads();
+    }
+    const float* xl = sm + L.x;
+    const float* bl = sm + L.b;
+    for (int t = threadIdx.x; t < RN; t += CV_T) {
+        const int lj = t >> L.lgN, i = t & m, e = lj * N + ((i + 1) & m), w = lj * N + ((i - 1) & m);
+        const float* xn = lj + 1 < R ? xl + t + N : cv_at(cl, sm + L.x + i, (rank + 1) & (SMALL_CLUSTER - 1));
+        const float* xs = lj > 0 ? xl + t - N : cv_at(cl, sm + L.x + (R - 1) * N + i, (rank - 1) & (SMALL_CLUSTER - 1));
+        const float u = xl[t], v = xl[RN + t], p = xl[2 * RN + t], uE = xl[e], vN = xn[RN];
+        float Au = L.a0 * u - L.c * ((uE + xl[w]) + (xn[0] + xs[0])) + (p - xl[2 * RN + w]) * L.ih;
+        float Av = L.a0 * v - L.c * ((xl[RN + e] + xl[RN + w]) + (vN + xs[RN])) + (p - xs[2 * RN]) * L.ih;
+        if (L.ib) {
+            float fu = 0.f, fv = 0.f;
+#pragma unroll
+            for (int k = 0; k < WD; ++k) fu += part[k * 2 * RN + t], fv += part[k * 2 * RN + RN + t];
+            Au -= L.dt * fu;
+            Av -= L.dt * fv;
+        }
+        float* r = sm + L.r + t;
+        r[0] = bl[t] - Au;
+        r[RN] = bl[RN + t] - Av;
+        r[2 * RN] = bl[2 * RN + t] + ((uE - u) + (vN - v)) * L.ih;
+    }
+}
+
+// x += omega times the weighted patch corrections of the residual at rr (x = them: zero).  A cell takes the patches
+// of its own, its western and its southern cell.
+__device__ __forceinline__ void cv_update(cg::cluster_group& cl, const ClusterArgs& a, const ClusterLevel& L, float* sm,
+                                          int rank, int rr, bool zero) {
+    const int N = L.N, m = N - 1, R = N / SMALL_CLUSTER, RN = R * N;
+    const float* rl = sm + rr;
+    const float hw = 0.5f * a.omega;
+    for (int t = threadIdx.x; t < RN; t += CV_T) {
+        const int lj = t >> L.lgN, i = t & m, ie = (i + 1) & m, iw = (i - 1) & m;
+        const float* rc = rl + lj * N;
+        const float* rn = lj + 1 < R ? rc + N : cv_at(cl, sm + rr, (rank + 1) & (SMALL_CLUSTER - 1));
+        const float* rs = lj > 0 ? rc - N : cv_at(cl, sm + rr + (R - 1) * N, (rank - 1) & (SMALL_CLUSTER - 1));
+        float f[3][7];
+        const float* pf = sm + L.pfs + lj * N;   // row lj of the strip's factors is the row to the south
+#pragma unroll
+        for (int k = 0; k < 7; ++k) {
+            const float* pk = pf + k * (RN + N);
+            f[0][k] = pk[N + i], f[1][k] = pk[N + iw], f[2][k] = pk[i];
+        }
+        const float ru = rc[i], rv = rc[RN + i];
+        float d0, d1, d2, d3, dp, w0, w1, w2, w3, wp, s0, s1, s2, s3, sp;
+        patch_solve(f[0], L.ih, ru, rc[ie], rv, rn[RN + i], rc[2 * RN + i], d0, d1, d2, d3, dp);
+        patch_solve(f[1], L.ih, rc[iw], ru, rc[RN + iw], rn[RN + iw], rc[2 * RN + iw], w0, w1, w2, w3, wp);
+        patch_solve(f[2], L.ih, rs[i], rs[ie], rs[RN + i], rv, rs[2 * RN + i], s0, s1, s2, s3, sp);
+        const float du = hw * (d0 + w1), dv = hw * (d2 + s3), dq = a.omega * dp;
+        float* x = sm + L.x + t;
+        x[0] = zero ? du : x[0] + du;
+        x[RN] = zero ? dv : x[RN] + dv;
+        x[2 * RN] = zero ? dq : x[2 * RN] + dq;
+    }
+}
+
+// sum of the six (u, v) or four (p) residual terms that coarse cell (I, J) restricts; row(c, j) gives row j of component c
+template <typename Row>
+__device__ __forceinline__ float cv_restrict(int comp, int I, int J, int m, Row row) {
+    const int i = 2 * I, j = 2 * J, ip = i + 1, im = (i - 1) & m;
+    const float *q = row(comp, j), *qn = row(comp, j + 1);
+    if (comp == 0) return 0.25f * ((q[i] + qn[i]) + 0.5f * ((q[ip] + qn[ip]) + (q[im] + qn[im])));
+    if (comp == 2) return 0.25f * ((q[i] + q[ip]) + (qn[i] + qn[ip]));
+    const float* qs = row(comp, (j - 1) & m);
+    return 0.25f * ((q[i] + q[ip]) + 0.5f * ((qn[i] + qn[ip]) + (qs[i] + qs[ip])));
+}
+
+__global__ void __launch_bounds__(CV_T, 1) k_vcycle_cluster(const __grid_constant__ ClusterArgs a) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    cg::cluster_group cl = cg::this_cluster();
+    float* sm = reinterpret_cast<float*>(smraw);
+    const int rank = (int)cl.block_rank(), top = a.levels - 1;
+    // set-up data: not written by the kernel this one waits for
+    for (int l = 0; l <= top; ++l) {
+        const ClusterLevel& L = a.lv[l];
+        const int N = L.N, m = N - 1, R = N / SMALL_CLUSTER, RN = R * N, j0 = rank * R;
+        for (int t = threadIdx.x * 4; t < 7 * (RN + N); t += CV_T * 4) {
+            const int k = t / (RN + N), q = t - k * (RN + N);
+            cv_copy16(sm + L.pfs + t, L.pf + k * N * N + (((j0 - 1 + (q >> L.lgN)) & m) << L.lgN) + (q & m), true);
+        }
+        if (!L.ib) continue;
+        const int nv = 2 * RN / 4;   // 16-byte vectors of four faces (at most 64); CV_T / nv threads share one's entries
+        const int f = (threadIdx.x & (nv - 1)) * 4, c = f >= RN, q = f - c * RN, j = j0 + (q >> L.lgN), i = q & m;
+        const int slot = L.slotOf[((j >> L.lgty) << L.lgntx) + (i >> L.lgtx)];
+        const float* w = L.win + (((size_t)((slot < 0 ? 0 : slot) * 2 + c) * WIN_SIZE) << (L.lgtx + L.lgty)) +
+                         ((j & ((1 << L.lgty) - 1)) << L.lgtx) + (i & ((1 << L.lgtx) - 1));
+        for (int k = threadIdx.x / nv; k < WIN_SIZE; k += CV_T / nv)
+            cv_copy16(sm + L.wins + k * 2 * RN + f, w + ((size_t)k << (L.lgtx + L.lgty)), slot >= 0);
+    }
+    const int prows = a.n0 / SMALL_CLUSTER;   // rows of the pseudo-inverse per block
+    double* P = reinterpret_cast<double*>(sm + a.P);
+    for (int t = threadIdx.x * 2; t < prows * a.n0; t += CV_T * 2)
+        cv_copy16(P + t, a.Pinv + (size_t)rank * prows * a.n0 + t, true);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    pdl_entry();
+    {
+        const ClusterLevel& L = a.lv[top];
+        const int RN = L.N / SMALL_CLUSTER * L.N, n = L.N * L.N;
+        for (int t = threadIdx.x; t < 3 * RN; t += CV_T) {
+            const int c = t / RN;
+            sm[L.b + t] = a.b[c * n + rank * RN + t - c * RN];
+        }
+    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    cl.sync();
+    auto sweep = [&](const ClusterLevel& L) {
+        cv_residual(cl, a, L, sm, rank);
+        cl.sync();
+        cv_update(cl, a, L, sm, rank, L.r, false);
+    };
+    for (int l = top; l >= 0; --l) {
+        const ClusterLevel& L = a.lv[l];
+        const int N = L.N, R = N / SMALL_CLUSTER, RN = R * N, lgR = L.lgN - 3, m = N - 1, Nc = N / 2;
+        if (a.nu1 > 0) {
+            cv_update(cl, a, L, sm, rank, L.b, true);   // from zero the residual is b
+        } else {
+            for (int t = threadIdx.x; t < 3 * RN; t += CV_T) sm[L.x + t] = 0.f;
+        }
+        cl.sync();
+        for (int k = 1; k < a.nu1; ++k) {
+            sweep(L);
+            cl.sync();
+        }
+        cv_residual(cl, a, L, sm, rank);
+        cl.sync();
+        auto row = [&](int c, int j) { return cv_at(cl, sm + L.r + c * RN + ((j & (R - 1)) << L.lgN), j >> lgR); };
+        if (l > 0) {
+            const ClusterLevel& C = a.lv[l - 1];
+            const int Rc = R / 2, RNc = Rc * Nc;
+            for (int t = threadIdx.x; t < 3 * RNc; t += CV_T) {
+                const int c = t / RNc, q = t - c * RNc, lJ = q >> C.lgN;
+                sm[C.b + t] = cv_restrict(c, q & (Nc - 1), rank * Rc + lJ, m, row);
+            }
+            cl.sync();
+            continue;
+        }
+        // coarsest solve: the whole b0 in every block, a share of the rows each, the result to all
+        double* b0 = reinterpret_cast<double*>(sm + a.b0);
+        const int nc = Nc * Nc;
+        for (int t = threadIdx.x; t < a.n0; t += CV_T) {
+            const int c = t / nc, q = t - c * nc;
+            b0[t] = (double)cv_restrict(c, q & (Nc - 1), q / Nc, m, row);
+        }
+        __syncthreads();
+        const int sub = threadIdx.x & 7;   // eight lanes a row; every lane of a warp takes the same trips
+        for (int r0 = 0; r0 < prows; r0 += CV_T / 8) {
+            const int r = r0 + (int)(threadIdx.x >> 3);
+            double acc = 0.0;
+            if (r < prows)
+                for (int c = sub; c < a.n0; c += 8) acc += P[r * a.n0 + c] * b0[c];
+            for (int o = 1; o < 8; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (r < prows) *cl.map_shared_rank(sm + a.x0 + rank * prows + r, sub) = (float)acc;
+        }
+        cl.sync();
+    }
+    for (int l = 0; l <= top; ++l) {
+        const ClusterLevel& L = a.lv[l];
+        const ClusterLevel& C = a.lv[l > 0 ? l - 1 : 0];
+        const int N = L.N, m = N - 1, R = N / SMALL_CLUSTER, RN = R * N, Nc = N / 2, mc = Nc - 1;
+        const int Rc = l > 0 ? R / 2 : Nc, lgNc = L.lgN - 1, lgRc = l > 0 ? L.lgN - 4 : lgNc, RNc = Rc * Nc;
+        for (int t = threadIdx.x; t < RN; t += CV_T) {
+            const int i = t & m, j = rank * R + (t >> L.lgN), I = i >> 1, J = j >> 1;
+            const int I1 = (I + 1) & mc, I2 = (I + ((i & 1) ? 1 : -1)) & mc, J2 = (J + ((j & 1) ? 1 : -1)) & mc;
+            // coarse rows J and J2: x0 is whole in every block, a coarser level's strip in its own
+            const float* e = l > 0 ? cv_at(cl, sm + C.x + ((J & (Rc - 1)) << lgNc), J >> lgRc) : sm + a.x0 + J * Nc;
+            const float* e2 = l > 0 ? cv_at(cl, sm + C.x + ((J2 & (Rc - 1)) << lgNc), J2 >> lgRc) : sm + a.x0 + J2 * Nc;
+            const float pu = (i & 1) ? 0.5f * (e[I] + e[I1]) : e[I];
+            const float pv = (j & 1) ? 0.5f * (e[RNc + I] + e2[RNc + I]) : e[RNc + I];
+            const float pp = 9.0f / 16.0f * e[2 * RNc + I] + 3.0f / 16.0f * (e[2 * RNc + I2] + e2[2 * RNc + I]) +
+                             1.0f / 16.0f * e2[2 * RNc + I2];
+            float* x = sm + L.x + t;
+            x[0] += pu;
+            x[RN] += pv;
+            x[2 * RN] += pp;
+        }
+        for (int k = 0; k < a.nu2; ++k) {
+            cl.sync();
+            sweep(L);
+        }
+        if (l == top) {   // every thread writes the cells that it updated last
+            const int n = N * N;
+            for (int t = threadIdx.x; t < RN; t += CV_T)
+                for (int c = 0; c < 3; ++c) a.out[c * n + rank * RN + t] = sm[L.x + c * RN + t];
+        }
+        cl.sync();   // for the finer level's prolongation; no block leaves while another reads its shared memory
+    }
+}
+
 }  // namespace
+
+size_t cluster_layout(ClusterArgs& a) {
+    int off = 0, halo = 0, part = 0;
+    auto take = [&](int n) {
+        const int p = off;
+        off += (n + 3) & ~3;
+        return p;
+    };
+    for (int l = 0; l < a.levels; ++l) {
+        ClusterLevel& L = a.lv[l];
+        const int R = L.N / SMALL_CLUSTER, RN = R * L.N;
+        L.x = take(3 * RN);
+        L.b = take(3 * RN);
+        L.r = take(3 * RN);
+        L.pfs = take(7 * (RN + L.N));
+        L.wins = take(L.ib ? WIN_SIZE * 2 * RN : 0);
+        if (!L.ib) continue;
+        halo = std::max(halo, 2 * (R + CV_WR8) * (L.N + CV_WR8));
+        part = std::max(part, WD * 2 * RN);
+    }
+    a.uh = take(halo);
+    a.part = take(part);
+    a.x0 = take(a.n0);
+    a.b0 = take(2 * a.n0);
+    a.P = take(2 * (a.n0 / SMALL_CLUSTER) * a.n0);
+    return sizeof(float) * (size_t)off;
+}
+static cudaLaunchConfig_t cluster_config(size_t smem, cudaLaunchAttribute* attr) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(SMALL_CLUSTER);
+    cfg.blockDim = dim3(CV_T);
+    cfg.dynamicSmemBytes = smem;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = SMALL_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+bool vcycle_cluster_fits(size_t smem) {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(smem, attr);
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    if (cudaFuncSetAttribute(k_vcycle_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&clusters, k_vcycle_cluster, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return clusters > 0;
+}
+cudaError_t launch_vcycle_cluster(const ClusterArgs& a, size_t smem, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_vcycle_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = cluster_config(smem, attr);
+    cfg.stream = s;
+    return cudaLaunchKernelEx(&cfg, k_vcycle_cluster, a);
+}
 
 template <typename T>
 size_t vcycle_small_smem(int N1, int n0, int nTiles, int per, int ntiles) {

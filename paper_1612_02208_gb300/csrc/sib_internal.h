@@ -217,6 +217,27 @@ struct SmallArgs {
     const double* Pinv;         // coarsest pseudo-inverse, n0 x n0
 };
 
+// The levels of up to CV_MAXN cells a side in one cluster (FP32, Vanka; kernels_small.cu), lowest first
+constexpr int CV_LEVELS = 3, CV_MAXN = 32;
+struct ClusterLevel {
+    int N, lgN, ib;             // ib: the level's IB operator is applied (through its windows)
+    int lgtx, lgty, lgntx;
+    float a0, c, ih, dt;
+    const float* pf;            // patch factors
+    const float* win;           // IB windows of the active tiles
+    const int* slotOf;          // tile -> slot of its windows, -1 without
+    int x, b, r, pfs, wins;     // places in shared memory, in floats
+};
+struct ClusterArgs {
+    ClusterLevel lv[CV_LEVELS];
+    int levels, nu1, nu2, n0;
+    float omega;
+    const double* Pinv;         // coarsest pseudo-inverse, n0 x n0
+    const float* b;             // right-hand side and result of the highest of the levels
+    float* out;
+    int uh, part, x0, b0, P;
+};
+
 // ------------------------------------------------------------------------------------------
 // launchers (kernels_grid.cu)
 template <typename T> void launch_residual(const GridK<T>& g, const T* x, const T* b, T* r, cudaStream_t s);
@@ -283,6 +304,9 @@ template <typename T> void launch_power_Mfinish(const GridK<T>& g, const T* ya, 
 template <typename T> size_t vcycle_small_smem(int N1, int n0, int nTiles, int per, int ntiles);
 template <typename T> int vcycle_small_cluster(size_t smem);
 template <typename T> cudaError_t launch_vcycle_small(const SmallArgs<T>& a, size_t smem, cudaStream_t s);
+size_t cluster_layout(ClusterArgs& a);   // places of the levels' arrays; returns the bytes of one block
+bool vcycle_cluster_fits(size_t smem);
+cudaError_t launch_vcycle_cluster(const ClusterArgs& a, size_t smem, cudaStream_t s);
 
 // launchers (kernels_wrap.cu): the Krylov-wrapped smoothing step
 constexpr int WRAP_MAXK = 8;     // at most this many FGMRES iterations a smoothing stage

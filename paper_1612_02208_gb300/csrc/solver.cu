@@ -751,11 +751,63 @@ void wrapped_smooth(sib_ctx* c, int l, const T* x, const T* b, T* xo, int k, cud
     KL(c, launch_wmaxpy<T>(Z, n3, k, y, 1.0, x, xo, n3, s));
 }
 
+// The highest level of the cluster kernel (FP32, Vanka): levels of up to CV_MAXN cells a side whose IB operator
+// has windows; 0 where it does not apply.  Fills the kernel's arguments.
+template <typename T>
+int cluster_top(sib_ctx* c, ClusterArgs* a, size_t* smem) {
+    if (Prec<T>::id != 1 || !c->opts.fuse_small || cavity(c) || c->opts.smooth_krylov ||
+        c->opts.smoother != SIB_SMOOTHER_VANKA || c->n_min > 8)
+        return 0;
+    int top = 0;
+    for (int l = 1; l <= c->lmax && l <= CV_LEVELS && c->L[l].N <= CV_MAXN; ++l) {
+        const Level& lv = c->L[l];
+        const bool ib = c->haveIB && lv.hnTiles > 0;
+        if (ib && !lv.useWindow) break;
+        const GridK<float> g = gridk<float>(c, l);
+        ClusterLevel& k = a->lv[l - 1];
+        k = ClusterLevel{};
+        k.N = lv.N;
+        while ((1 << k.lgN) < lv.N) ++k.lgN;
+        while ((1 << k.lgntx) < lv.ntx) ++k.lgntx;
+        k.ib = ib;
+        k.lgtx = g.lgtx;
+        k.lgty = g.lgty;
+        k.a0 = g.a0;
+        k.c = g.c;
+        k.ih = g.inv_h;
+        k.dt = g.dt;
+        k.pf = g.pf;
+        k.win = (const float*)lv.win[1];
+        k.slotOf = lv.slotOf;
+        top = l;
+    }
+    if (top == 0) return 0;
+    a->levels = top;
+    a->nu1 = c->opts.nu1;
+    a->nu2 = c->opts.nu2;
+    a->n0 = c->n0;
+    a->omega = (float)c->opts.omega;
+    a->Pinv = c->Pinv;
+    a->b = (const float*)c->L[top].p[1].b;
+    a->out = (float*)c->L[top].p[1].x;
+    *smem = cluster_layout(*a);
+    return *smem <= (size_t)c->smemOptin && vcycle_cluster_fits(*smem) ? top : 0;
+}
+
 // Alg. 1 on level l with right-hand side in the level's b; returns the buffer holding w.
 template <typename T>
 T* vcycle_level(sib_ctx* c, int l, cudaStream_t s) {
     Level& lv = c->L[l];
     const int pi = Prec<T>::id;
+    if (l > 0 && lv.N <= CV_MAXN) {
+        ClusterArgs a{};
+        size_t smem = 0;
+        if (cluster_top<T>(c, &a, &smem) == l) {
+            CK(launch_vcycle_cluster(a, smem, s));
+            ++c->launches;
+            return (T*)lv.p[pi].x;
+        }
+    }
     if (l == 1 && !c->opts.smooth_krylov && small_ok<T>(c)) return vcycle_small<T>(c, s);
     if (l == 0) {
         KL(c, launch_coarse_apply<T>(c->Pinv, c->n0, (const T*)lv.p[pi].b, (T*)lv.p[pi].x, s));

@@ -123,3 +123,25 @@ def test_wide_boxes_in_pairs_of_floats(kind, N, gamma, o):
         S.smooth(l, y64, cu(b.astype(np.float64)), 1)
         assert rel(host(y32), host(y64)) < TOL32, l
     S.close()
+
+
+# The cluster kernel's levels: one, two and three of them, strips of one, two and four rows, as the whole
+# V-cycle or below a 64^2 level, with and without IB windows; to the repository's bar for an FP32 V-cycle
+@pytest.mark.parametrize("n_min,N", [(4, 8), (4, 16), (4, 32), (8, 16), (8, 32), (8, 64), (4, 64)])
+@pytest.mark.parametrize("make", [lambda N: I.disk_stokes(N, kappa=1e2, seed=1), lambda N: I.no_structure(N, rho=1.0, seed=4)],
+                         ids=["disk", "fluid"])
+def test_cluster_levels(make, n_min, N):
+    prob = make(N)
+    H = multigrid.Hierarchy(prob, n_min=n_min)
+    st = prob.structure
+    S = sib.Solver(N, n_min=n_min)
+    S.set_fluid(prob.rho, prob.mu, prob.dt)
+    if st.M > 0:
+        S.set_structure(cu(st.X), torch.as_tensor(st.edges, device="cuda"), cu(st.kappa))
+    S.setup()
+    b = rand(3 * N * N, 7600 + N).astype(np.float32).astype(np.float64)
+    b[2 * N * N:] -= b[2 * N * N:].mean()
+    z = S.vcycle(cu(b, torch.float32))
+    assert rel(host(z), H.vcycle(b)) < 1e-4
+    assert torch.equal(S.vcycle(cu(b, torch.float32)), z)
+    S.close()
