@@ -25,11 +25,19 @@ constexpr int WIN_SIZE = WD * WD;
 // memory, then lets its dependents be scheduled (they start waiting while this grid finishes), so
 // consecutive kernels of a stream or graph overlap their launch latency.  Dependents become
 // eligible only after every block of this grid has started, so early triggering cannot starve it.
-__device__ __forceinline__ void pdl_entry() {
+__device__ __forceinline__ void pdl_wait() {
 #if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
+#endif
+}
+__device__ __forceinline__ void pdl_launch() {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 900
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 #endif
+}
+__device__ __forceinline__ void pdl_entry() {
+    pdl_wait();
+    pdl_launch();
 }
 
 template <typename... KArgs, typename... Args>
@@ -451,14 +459,15 @@ template <typename T> void launch_fg_zstore(const T* src, double* Z, int64_t n, 
                                             cudaStream_t s);
 void launch_multidot_dev(const double* V, int64_t ld, const double* w, int64_t n, double* partials,
                          const FgDev* st, cudaStream_t s);
-void launch_reduce_partials_dev(const double* partials, int nblk, double* out, const FgDev* st, int count,
-                                cudaStream_t s);
-void launch_multi_axpy_dev(const double* V, int64_t ld, const double* coef, double sign, double* y, int64_t n,
-                           const FgDev* st, int useK, cudaStream_t s);
-// returns the number of partial sums written
-int launch_multi_axpy_norm_dev(const double* V, int64_t ld, const double* coef, double sign, double* y, int64_t n,
-                               const FgDev* st, double* partials, cudaStream_t s);
-void launch_fg_arnoldi(FgDev* st, const double* h1, const double* h2, const double* nrm,
+constexpr int MD_MAXPART = 5120;             // partials of launch_multidot_dev, at most
+// y -= sum_{i <= j} h_i V_i, h_i from those partials (dots) and left in h; partials != nullptr: the block
+// partials of ||y||^2, whose number is returned
+int launch_gs_update_dev(const double* V, int64_t ld, const double* dots, double* h, double* y, int64_t n,
+                         const FgDev* st, double* partials, cudaStream_t s);
+// y += sum_{i < k} coef[i] V_i, k = st->k
+void launch_multi_axpy_dev(const double* V, int64_t ld, const double* coef, double* y, int64_t n, const FgDev* st,
+                           cudaStream_t s);
+void launch_fg_arnoldi(FgDev* st, const double* h1, const double* h2, const double* nrm, int nb,
                        cudaGraphConditionalHandle handle, cudaStream_t s);
 void launch_fg_backsolve(FgDev* st, cudaStream_t s);
 

@@ -1840,14 +1840,11 @@ void build_fg_graph(sib_ctx* c) {
             KL(c, launch_fg_zstore<T>(out, c->Z, n, c->fg, c->zcur, s));
             matvec(c, c->zcur, c->res, s);
             KL(c, launch_multidot_dev(c->V, n, c->res, n, c->part, c->fg, s));
-            KL(c, launch_reduce_partials_dev(c->part, 0, c->scal, c->fg, 0, s));
-            KL(c, launch_multi_axpy_dev(c->V, n, c->scal, -1.0, c->res, n, c->fg, 0, s));
+            KL(c, launch_gs_update_dev(c->V, n, c->part, c->scal, c->res, n, c->fg, nullptr, s));
             KL(c, launch_multidot_dev(c->V, n, c->res, n, c->part, c->fg, s));
-            KL(c, launch_reduce_partials_dev(c->part, 0, c->scal + 128, c->fg, 0, s));
             int nb = 0;
-            KL(c, nb = launch_multi_axpy_norm_dev(c->V, n, c->scal + 128, -1.0, c->res, n, c->fg, c->part, s));
-            KL(c, launch_reduce_partials_dev(c->part, nb, c->scal + 256, c->fg, 1, s));
-            KL(c, launch_fg_arnoldi(c->fg, c->scal, c->scal + 128, c->scal + 256, h, s));
+            KL(c, nb = launch_gs_update_dev(c->V, n, c->part, c->scal + 128, c->res, n, c->fg, c->part + MD_MAXPART, s));
+            KL(c, launch_fg_arnoldi(c->fg, c->scal, c->scal + 128, c->part + MD_MAXPART, nb, h, s));
         } catch (...) {
             cudaGraph_t tmp;
             cudaStreamEndCapture(s, &tmp);
@@ -1859,7 +1856,7 @@ void build_fg_graph(sib_ctx* c) {
         CK(cudaStreamBeginCaptureToGraph(s, g, &wnode, nullptr, 1, cudaStreamCaptureModeThreadLocal));
         const double* y = reinterpret_cast<const double*>(reinterpret_cast<const char*>(c->fg) + offsetof(FgDev, y));
         KL(c, launch_fg_backsolve(c->fg, s));
-        KL(c, launch_multi_axpy_dev(c->Z, n, y, 1.0, c->sol, n, c->fg, 1, s));
+        KL(c, launch_multi_axpy_dev(c->Z, n, y, c->sol, n, c->fg, s));
         CK(cudaStreamEndCapture(s, &tmp));
         CK(cudaGraphInstantiate(&c->fgExec[pi], g, 0));
         c->fgBody[pi] = mid - before;

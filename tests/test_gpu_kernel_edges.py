@@ -145,3 +145,23 @@ def test_cluster_levels(make, n_min, N):
     assert rel(host(z), H.vcycle(b)) < 1e-4
     assert torch.equal(S.vcycle(cu(b, torch.float32)), z)
     S.close()
+
+
+# Arnoldi steps of one, two and three groups of eight vectors, on vectors shorter than a slice and longer; the
+# true residual, formed after the solve, is the stopping test's to rounding
+@pytest.mark.parametrize("N,n_min", [(8, 4), (32, 8), (128, 8)])
+@pytest.mark.parametrize("restart", [7, 8, 9, 17, 100])
+def test_arnoldi_lengths(N, n_min, restart):
+    prob = I.disk_stokes(N, kappa=1e2, seed=1)
+    st, its = prob.structure, []
+    for graphs in (1, 0):
+        S = sib.Solver(N, n_min=n_min)
+        S.set_fluid(prob.rho, prob.mu, prob.dt)
+        S.set_options(rtol=1e-10, restart=restart, max_it=200, use_graphs=graphs)
+        S.set_structure(cu(st.X), torch.as_tensor(st.edges, device="cuda"), cu(st.kappa))
+        S.setup()
+        S.solve(cu(prob.g))
+        assert S.stats.converged and S.stats.rel_residual < 2e-10, (graphs, S.stats.rel_residual)
+        its.append(S.stats.iterations)
+        S.close()
+    assert abs(its[0] - its[1]) <= 1, its
