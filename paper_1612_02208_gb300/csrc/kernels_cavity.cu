@@ -77,12 +77,10 @@ __global__ void k_cavity_residual(GridK<T> g, const T* __restrict__ x, const T* 
 // velocity blocks carry the tangential ghost (+c on the diagonal of a face next to a tangential
 // wall) and the IB entries; a wall face acts as an infinitely stiff block entry, so its inverse-block
 // factors are 0, which zeroes its correction and drops it from the pressure Schur complement.
-// d = (d0, d1, d2, d3, dp) per cell, 5 n values.
 template <typename T>
-__global__ void k_cavity_patch(GridK<T> g, const T* __restrict__ r, T* __restrict__ d) {
-    pdl_entry();
+__device__ __forceinline__ void cavity_patch(const GridK<T>& g, int i, int j, T r0, T r1, T r2, T r3, T r4, T& d0, T& d1,
+                                             T& d2, T& d3, T& dp) {
     const int N = g.N, n = N * N, m = N - 1;
-    const int i = blockIdx.x * g.tx + threadIdx.x, j = blockIdx.y * g.ty + threadIdx.y;
     const int c = j * N + i, ce = j * N + ((i + 1) & m), cn = ((j + 1) & m) * N + i;
     const bool wuL = i == 0, wuR = i == N - 1, wvB = j == 0, wvT = j == N - 1;
     const T tu = g.c * T(int(j == 0) + int(j == N - 1)), tv = g.c * T(int(i == 0) + int(i == N - 1));
@@ -108,35 +106,73 @@ __global__ void k_cavity_patch(GridK<T> g, const T* __restrict__ r, T* __restric
     T A00u, A01u, A11u, A00v, A01v, A11v;
     block(au00, au11, au01, wuL, wuR, A00u, A01u, A11u);
     block(av00, av11, av01, wvB, wvT, A00v, A01v, A11v);
-    const T r0 = wuL ? T(0) : r[c], r1 = wuR ? T(0) : r[c + 1];
-    const T r2 = wvB ? T(0) : r[n + c], r3 = wvT ? T(0) : r[n + c + N];
-    const T r4 = r[2 * n + c];
     const T ih = g.inv_h;
     const T tu0 = A00u * r0 + A01u * r1, tu1 = A01u * r0 + A11u * r1;
     const T tv0 = A00v * r2 + A01v * r3, tv1 = A01v * r2 + A11v * r3;
     const T su0 = ih * (A00u - A01u), su1 = ih * (A01u - A11u);
     const T sv0 = ih * (A00v - A01v), sv1 = ih * (A01v - A11v);
     const T S = ih * ((su0 - su1) + (sv0 - sv1));
-    const T dp = (ih * ((tu0 - tu1) + (tv0 - tv1)) - r4) / S;
-    d[c] = tu0 - su0 * dp;
-    d[n + c] = tu1 - su1 * dp;
-    d[2 * n + c] = tv0 - sv0 * dp;
-    d[3 * n + c] = tv1 - sv1 * dp;
-    d[4 * n + c] = dp;
+    dp = (ih * ((tu0 - tu1) + (tv0 - tv1)) - r4) / S;
+    d0 = tu0 - su0 * dp;
+    d1 = tu1 - su1 * dp;
+    d2 = tv0 - sv0 * dp;
+    d3 = tv1 - sv1 * dp;
 }
 
-// xo = x + omega (1/2 (two cell corrections) on interior faces, the cell's on p); 0 on wall faces
-template <typename T>
-__global__ void k_cavity_update(GridK<T> g, T omega, const T* __restrict__ d, const T* __restrict__ x,
-                                T* __restrict__ xo) {
+// One additive sweep, xo = x + omega (1/2 (two cells' corrections) on interior faces, the cell's on p), 0 on wall
+// faces; ZERO: from x = 0, where the residual is b.  A tile forms the residuals of its cells and of a ring around
+// them (0 on wall faces and outside), then its patches and those of the column to the west and the row to the south,
+// whose d1 and d3 reach into it.  As three launches with the residual and the corrections in between in global
+// memory, the 272 sweeps of a 128^2 solve waited three times for a launch each: solve 4.04 -> 3.45 ms.
+template <typename T, bool ZERO>
+__global__ void __launch_bounds__(TX * TY) k_cavity_vanka(GridK<T> g, T omega, const T* __restrict__ x,
+                                                          const T* __restrict__ b, T* __restrict__ xo) {
+    __shared__ T rs[3][TY + 2][TX + 2];         // residuals, cell (i0 - 1 + column, j0 - 1 + row)
+    __shared__ T d1s[TY][TX + 1], d3s[TY + 1][TX];
+    const int N = g.N, n = N * N, tx = threadIdx.x, ty = threadIdx.y, W = g.tx, H = g.ty;   // W <= TX, H <= TY
+    const int i0 = blockIdx.x * W, j0 = blockIdx.y * H, tid = ty * W + tx;
     pdl_entry();
-    const int N = g.N, n = N * N;
-    const int i = blockIdx.x * g.tx + threadIdx.x, j = blockIdx.y * g.ty + threadIdx.y;
-    const int c = j * N + i;
+    for (int q = tid; q < (W + 2) * (H + 2); q += W * H) {
+        const int rj = q / (W + 2), ri = q - rj * (W + 2), i = i0 - 1 + ri, j = j0 - 1 + rj, c = j * N + i;
+        T u = T(0), v = T(0), p = T(0);
+        if (i >= 0 && i < N && j >= 0 && j < N) {
+            T au = T(0), av = T(0), ap = T(0);
+            if (!ZERO) cavity_rows(g, x, i, j, au, av, ap);
+            u = i > 0 ? b[c] - au : T(0);
+            v = j > 0 ? b[n + c] - av : T(0);
+            p = b[2 * n + c] - ap;
+        }
+        rs[0][rj][ri] = u;
+        rs[1][rj][ri] = v;
+        rs[2][rj][ri] = p;
+    }
+    __syncthreads();
+    // patch of the cell in column pi, row pj of the tile (-1: the ring); faces past a wall hold 0 above
+    auto patch = [&](int pi, int pj, T& d0, T& d1, T& d2, T& d3, T& dp) {
+        cavity_patch(g, i0 + pi, j0 + pj, rs[0][pj + 1][pi + 1], rs[0][pj + 1][pi + 2], rs[1][pj + 1][pi + 1],
+                     rs[1][pj + 2][pi + 1], rs[2][pj + 1][pi + 1], d0, d1, d2, d3, dp);
+    };
+    T d0, d1, d2, d3, dp;
+    patch(tx, ty, d0, d1, d2, d3, dp);
+    d1s[ty][tx + 1] = d1;
+    d3s[ty + 1][tx] = d3;
+    if (tid < W + H) {
+        const bool south = tid < W;
+        const int pi = south ? tid : -1, pj = south ? -1 : tid - W;
+        T e0 = T(0), e1 = T(0), e2 = T(0), e3 = T(0), ep = T(0);
+        if (i0 + pi >= 0 && j0 + pj >= 0) patch(pi, pj, e0, e1, e2, e3, ep);
+        if (south)
+            d3s[0][pi] = e3;
+        else
+            d1s[pj][0] = e1;
+    }
+    __syncthreads();
+    const int i = i0 + tx, j = j0 + ty, c = j * N + i;
     const T hw = T(0.5) * omega;
-    xo[c] = i >= 1 ? x[c] + hw * (d[c] + d[n + c - 1]) : T(0);
-    xo[n + c] = j >= 1 ? x[n + c] + hw * (d[2 * n + c] + d[3 * n + c - N]) : T(0);
-    xo[2 * n + c] = x[2 * n + c] + omega * d[4 * n + c];
+    const T du = hw * (d0 + d1s[ty][tx]), dv = hw * (d2 + d3s[ty][tx]), dq = omega * dp;
+    xo[c] = i >= 1 ? (ZERO ? du : x[c] + du) : T(0);
+    xo[n + c] = j >= 1 ? (ZERO ? dv : x[n + c] + dv) : T(0);
+    xo[2 * n + c] = ZERO ? dq : x[2 * n + c] + dq;
 }
 
 // Restriction for the cavity (Sec. 3.2 with walls): the periodic R_u = P_u^T / 4 and the pressure
@@ -338,18 +374,18 @@ void launch_cavity_apply(const GridK<T>& g, const T* x, T* y, cudaStream_t s) {
     launch_pdl(k_cavity_apply<T>, dim3(g.N / g.tx, g.N / g.ty), dim3(g.tx, g.ty), 0, s, g, x, y);
 }
 template <typename T>
-void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* r, T* d, T* xo, T omega, cudaStream_t s) {
+void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* xo, T omega, cudaStream_t s) {
     const dim3 grd(g.N / g.tx, g.N / g.ty), blk(g.tx, g.ty);
-    launch_pdl(k_cavity_residual<T>, grd, blk, 0, s, g, x, b, r);
-    launch_pdl(k_cavity_patch<T>, grd, blk, 0, s, g, (const T*)r, d);
-    launch_pdl(k_cavity_update<T>, grd, blk, 0, s, g, omega, (const T*)d, x, xo);
+    if (x)
+        launch_pdl(k_cavity_vanka<T, false>, grd, blk, 0, s, g, omega, x, b, xo);
+    else
+        launch_pdl(k_cavity_vanka<T, true>, grd, blk, 0, s, g, omega, x, b, xo);
 }
 template void launch_cavity_apply<float>(const GridK<float>&, const float*, float*, cudaStream_t);
 template void launch_cavity_apply<double>(const GridK<double>&, const double*, double*, cudaStream_t);
-template void launch_cavity_vanka<float>(const GridK<float>&, const float*, const float*, float*, float*, float*, float,
-                                         cudaStream_t);
-template void launch_cavity_vanka<double>(const GridK<double>&, const double*, const double*, double*, double*,
-                                          double*, double, cudaStream_t);
+template void launch_cavity_vanka<float>(const GridK<float>&, const float*, const float*, float*, float, cudaStream_t);
+template void launch_cavity_vanka<double>(const GridK<double>&, const double*, const double*, double*, double,
+                                          cudaStream_t);
 template void launch_cavity_residual<float>(const GridK<float>&, const float*, const float*, float*, cudaStream_t);
 template void launch_cavity_residual<double>(const GridK<double>&, const double*, const double*, double*,
                                              cudaStream_t);

@@ -251,10 +251,10 @@ struct ClusterArgs {
 template <typename T> void launch_residual(const GridK<T>& g, const T* x, const T* b, T* r, cudaStream_t s);
 // y = L x of the lid-driven cavity on the periodic layout (kernels_cavity.cu); wall-face entries 0
 template <typename T> void launch_cavity_apply(const GridK<T>& g, const T* x, T* y, cudaStream_t s);
-// one additive Vanka sweep of the cavity: r = b - L x, per-cell patch solves into d (5 n), xo = x + omega
-// (weighted corrections); g.fib must hold [S K J] x (kernels_cavity.cu)
+// one additive Vanka sweep of the cavity, xo = x + omega (weighted corrections of b - L x; x == nullptr: from 0);
+// g.fib must hold [S K J] x (kernels_cavity.cu)
 template <typename T>
-void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* r, T* d, T* xo, T omega, cudaStream_t s);
+void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* xo, T omega, cudaStream_t s);
 // r = b - L x of the cavity (0 on the wall faces); x <- 0 on the wall faces
 template <typename T> void launch_cavity_residual(const GridK<T>& g, const T* x, const T* b, T* r, cudaStream_t s);
 template <typename T> void launch_cavity_zero_walls(T* x, int N, cudaStream_t s);

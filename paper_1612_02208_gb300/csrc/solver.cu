@@ -47,7 +47,6 @@ struct LevelBuf {
     void* tp[6] = {};
     void* dinv = nullptr;   // 3 n: SC diagonals
     void* pf = nullptr;     // 7 n: Vanka patch factors
-    void* cav = nullptr;    // 5 n: cavity Vanka patch corrections (allocated on first use)
     // Krylov-wrapped smoothing: WRAP_MAXK + 1 Arnoldi vectors, WRAP_MAXK preconditioned ones, a work
     // vector (3 n each) and the step's small FP64 arrays
     void* wV = nullptr;
@@ -609,11 +608,9 @@ void ras_apply(sib_ctx* c, int l, const T* r, const T* x, T* xo, double omega, c
 // one smoothing sweep xo <- smooth(x, b)
 template <typename T>
 void sweep(sib_ctx* c, int l, const T* x, const T* b, T* xo, cudaStream_t s) {
-    if (cavity(c)) {   // the cavity's Vanka sweep: residual, patch solves with the wall rules, update
-        LevelBuf& lb = c->L[l].p[Prec<T>::id];
-        ib_apply<T>(c, l, x, s);
-        launch_cavity_vanka<T>(gridk<T>(c, l), x, b, (T*)lb.r, (T*)lb.cav, xo, (T)c->opts.omega, s);
-        c->launches += 3;
+    if (cavity(c)) {   // the cavity's Vanka sweep: patch solves with the wall rules
+        if (x) ib_apply<T>(c, l, x, s);
+        KL(c, launch_cavity_vanka<T>(gridk<T>(c, l), x, b, xo, (T)c->opts.omega, s));
     } else if (c->opts.smoother == SIB_SMOOTHER_SC) {
         sc_sweep<T>(c, l, x, b, xo, s);
     } else if (c->opts.smoother == SIB_SMOOTHER_RAS) {   // r = b - L x, then the box corrections
@@ -817,9 +814,9 @@ T* vcycle_level(sib_ctx* c, int l, cudaStream_t s) {
         T* x = (T*)lv.p[pi].x;
         T* xt = (T*)lv.p[pi].xt;
         const T* b = (const T*)lv.p[pi].b;
-        CK(cudaMemsetAsync(x, 0, sizeof(T) * 3 * (size_t)lv.N * lv.N, s));
+        if (c->opts.nu1 == 0) CK(cudaMemsetAsync(x, 0, sizeof(T) * 3 * (size_t)lv.N * lv.N, s));
         for (int k = 0; k < c->opts.nu1; ++k) {
-            sweep<T>(c, l, x, b, xt, s);
+            sweep<T>(c, l, k > 0 ? x : nullptr, b, xt, s);   // the first from w = 0
             std::swap(x, xt);
         }
         T* r = (T*)lv.p[pi].r;
@@ -1594,11 +1591,6 @@ void setup(sib_ctx* c, cudaStream_t s) {
         KL(c, (launch_convert<double, float>((const double*)lv.p[0].pf, (float*)lv.p[1].pf, n7, s)));
     }
     if (c->opts.smoother == SIB_SMOOTHER_RAS && c->lmax > 0) ras_setup_all(c, s);
-    if (cavity(c))   // the cavity sweep's patch corrections, allocated outside any graph capture
-        for (int l = 1; l <= c->lmax; ++l)
-            for (int pi = 0; pi < 2; ++pi)
-                if (!c->L[l].p[pi].cav)
-                    c->L[l].p[pi].cav = dalloc(c, (pi == 0 ? 8 : 4) * 5 * (size_t)c->L[l].N * c->L[l].N);
     if (c->opts.smoother == SIB_SMOOTHER_SC) {
         alloc_sc_bufs(c);
         for (int l = 1; l <= c->lmax; ++l) {
@@ -2159,15 +2151,13 @@ void cavity_smooth_impl(sib_ctx* c, int l, T* x, const T* b, int sweeps, cudaStr
     Level& lv = c->L[l];
     LevelBuf& lb = lv.p[Prec<T>::id];
     const size_t n = (size_t)lv.N * lv.N;
-    if (!lb.cav) lb.cav = dalloc(c, sizeof(T) * 5 * n);
     const double om = c->opts.smoother == SIB_SMOOTHER_VANKA ? c->opts.omega : 0.8;
     GridK<T> g = gridk<T>(c, l);
     T* cur = x;
     T* nxt = (T*)lb.xt;
     for (int k = 0; k < sweeps; ++k) {
         ib_apply<T>(c, l, cur, s);
-        launch_cavity_vanka<T>(g, cur, b, (T*)lb.r, (T*)lb.cav, nxt, (T)om, s);
-        c->launches += 3;
+        KL(c, launch_cavity_vanka<T>(g, cur, b, nxt, (T)om, s));
         std::swap(cur, nxt);
     }
     if (cur != x) CK(cudaMemcpyAsync(x, cur, sizeof(T) * 3 * n, cudaMemcpyDeviceToDevice, s));
