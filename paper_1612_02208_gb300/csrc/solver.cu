@@ -791,9 +791,11 @@ int cluster_top(sib_ctx* c, ClusterArgs* a, size_t* smem) {
     return *smem <= (size_t)c->smemOptin && vcycle_cluster_fits(*smem) ? top : 0;
 }
 
-// Alg. 1 on level l with right-hand side in the level's b; returns the buffer holding w.
+// Alg. 1 on level l with right-hand side in the level's b; returns the buffer holding w.  bUser: the right-hand
+// side instead of the level's b, zUser: the buffer of the last post-smoothing sweep (vcycle_direct; such calls meet
+// neither the Krylov-wrapped nor the cavity's form, nor a level of the small-level kernels).
 template <typename T>
-T* vcycle_level(sib_ctx* c, int l, cudaStream_t s) {
+T* vcycle_level(sib_ctx* c, int l, cudaStream_t s, const T* bUser = nullptr, T* zUser = nullptr) {
     Level& lv = c->L[l];
     const int pi = Prec<T>::id;
     if (l > 0 && lv.N <= CV_MAXN) {
@@ -851,7 +853,7 @@ T* vcycle_level(sib_ctx* c, int l, cudaStream_t s) {
     const int64_t n3 = 3LL * lv.N * lv.N;
     T* x = (T*)lv.p[pi].x;
     T* xt = (T*)lv.p[pi].xt;
-    const T* b = (const T*)lv.p[pi].b;
+    const T* b = bUser ? bUser : (const T*)lv.p[pi].b;
     int k0 = 0;
     if (c->opts.smoother == SIB_SMOOTHER_VANKA && c->opts.nu1 > 0) {
         KL(c, launch_vanka_zero<T>(gridk<T>(c, l), b, xt, s));   // first sweep from w = 0
@@ -877,6 +879,7 @@ T* vcycle_level(sib_ctx* c, int l, cudaStream_t s) {
     T* ec = vcycle_level<T>(c, l - 1, s);
     KL(c, launch_prolong_add<T>(c->L[l - 1].N, ec, x, s));
     for (int k = 0; k < c->opts.nu2; ++k) {
+        if (zUser && k + 1 == c->opts.nu2) xt = zUser;
         sweep<T>(c, l, x, b, xt, s);
         std::swap(x, xt);
     }
@@ -2002,6 +2005,24 @@ int solve_impl(sib_ctx* c, const double* g, double* w, sib_stats* st, cudaStream
     return rc;
 }
 
+// A caller's V-cycle on large grids: the kernels launched one by one, the finest level's on the caller's own arrays.
+// The captured graph works on the level's, so b is copied in and z out: 121 of the 1,265 us of an FP32 V-cycle at
+// 4096^2 (1,140 so).  From 2048^2 on the finest level's kernels run longer than the host takes
+// to enqueue the rest; below, the graph's launches are worth more than the copies.  False: not for these arguments
+// (arrays that overlap, that 16-byte and TMA loads cannot take, or a stream in capture).
+template <typename T>
+bool vcycle_direct(sib_ctx* c, const T* b, T* z, cudaStream_t s) {
+    const uintptr_t pb = (uintptr_t)b, pz = (uintptr_t)z, bytes = sizeof(T) * (uintptr_t)n3f(c);
+    if (c->L[c->lmax].N < 2048 || cavity(c) || c->opts.smooth_krylov || c->opts.nu2 < 1 || c->opts.l2_persist ||
+        (pb | pz) % 16 != 0 || (pb < pz + bytes && pz < pb + bytes))
+        return false;
+    cudaStreamCaptureStatus st;
+    CK(cudaStreamIsCapturing(s, &st));
+    if (st != cudaStreamCaptureStatusNone) return false;
+    vcycle_level<T>(c, c->lmax, s, b, z);
+    return true;
+}
+
 bool valid_prec(int p) { return p == SIB_PREC_FP64 || p == SIB_PREC_FP32; }
 void check_level(sib_ctx* c, int l, int lo) {
     if (l < lo || l > c->lmax) throw SibError(SIB_ERR_ARG, "level out of range");
@@ -2665,7 +2686,9 @@ int sib_vcycle(sib_ctx* c, int prec, const void* b, void* z, void* stream) {
     cudaStream_t s = S(stream);
     const int64_t n = n3f(c);
     Level& lv = c->L[c->lmax];
-    if (prec == SIB_PREC_FP64) {
+    if (prec == SIB_PREC_FP64 ? vcycle_direct(c, (const double*)b, (double*)z, s)
+                              : vcycle_direct(c, (const float*)b, (float*)z, s)) {
+    } else if (prec == SIB_PREC_FP64) {
         CK(cudaMemcpyAsync(lv.p[0].b, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
         double* out = vcycle<double>(c, s);
         CK(cudaMemcpyAsync(z, out, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));

@@ -165,3 +165,19 @@ def test_arnoldi_lengths(N, n_min, restart):
         its.append(S.stats.iterations)
         S.close()
     assert abs(its[0] - its[1]) <= 1, its
+
+
+# The V-cycle on the caller's arrays (grids from 2048^2 on) and on the level's (an array that is not aligned, an
+# output that is the input) are the same kernels on the same values
+@pytest.mark.parametrize("dtype,smoother", [(torch.float32, 0), (torch.float64, 0), (torch.float32, sib.SMOOTHER_RAS)])
+def test_vcycle_on_the_callers_arrays(dtype, smoother):
+    N = 2048
+    S = sib.solver_for(I.thin_ellipse_re(N, kappa=1e2), smoother=smoother, restart=1, max_it=1)
+    b = torch.randn(3 * N * N + 1, device="cuda", dtype=dtype)
+    z = S.vcycle(b[:-1])
+    off = b[:-1].new_empty(3 * N * N + 1)
+    off[1:] = b[:-1]
+    assert torch.equal(S.vcycle(off[1:]), z)
+    same = b[:-1].clone()
+    assert S.vcycle(same, same) is same and torch.equal(same, z)
+    S.close()
