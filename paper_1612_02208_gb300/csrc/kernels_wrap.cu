@@ -7,7 +7,11 @@
 // timing.  The classical Gram-Schmidt update of each pass is fused with the inner products that
 // follow it (the second pass's coefficients, or the norm).  The small Hessenberg least-squares
 // problem is solved in FP64 by one thread.
+#include <cooperative_groups.h>
+
 #include "sib_internal.h"
+
+namespace cg = cooperative_groups;
 
 namespace sib {
 
@@ -343,98 +347,125 @@ __global__ void __launch_bounds__(WT) k_wreduce_lsq(const double* __restrict__ p
     }
 }
 
-// Levels small enough for one block (n <= WRAP_ONE_MAX): each reduction finishes in the block that
-// forms it, so no separate reduce kernel runs.  k_wnorm_one: beta2 = |r0|^2 and V0 = r0 / |r0|.
-template <typename T>
-__global__ void __launch_bounds__(WT) k_wnorm_one(const T* __restrict__ r0, int64_t n, double* __restrict__ beta2,
-                                                  T* __restrict__ V0) {
+// Levels of up to wrap_cluster_max values: a whole orthogonalisation step in one cluster of eight blocks.  w stays
+// in registers (E vectors of 16 bytes a thread); the two Gram-Schmidt passes h = V^T w, w -= V h and the norm each
+// end with every block's sums in every block's shared memory and one cluster barrier; then Vnext = w / |w|
+// (Vnext != nullptr) and, on the stage's last step (lsq_k > 0), its least-squares solve into y.  cnt = 0: the norm
+// alone, of the stage's residual.  Bound by latency: seven launches of 2.5 us each did a step (three on levels
+// of up to 32^2, in one block).  Solves with wrapped Schur-complement sweeps, disk, FP32: 32^2 2.35 -> 2.25 ms,
+// 128^2 6.49 -> 6.17, 256^2 11.75 -> 11.33.  FP64 levels take it up to 32^2 (3.67 -> 3.35): above, eight SMs' FP64 pipes
+// are slower than the launches (128^2: 10.6 against 11.0 ms with it).
+constexpr int WC = 8;
+template <typename T, int KC, int E>
+__global__ void __launch_bounds__(WT) k_wstep_cluster(const T* __restrict__ V, int64_t n, int cnt, const T* __restrict__ w,
+                                                      double* hA, double* hB, double* nr, T* __restrict__ Vnext,
+                                                      int lsq_k, const double* hAll, const double* hBll,
+                                                      const double* nrAll, const double* beta2, double* y) {
     using VT = typename WVec<T>::type;
     constexpr int VN = WVec<T>::n;
-    pdl_entry();
+    __shared__ double part[3][WC][KC], ws[KC][WW], sum[KC];
     __shared__ T scale;
-    double acc[1] = {0.0};
-    const int64_t nv = n / VN;
-    for (int64_t e = threadIdx.x; e < nv; e += WT) {
-        const VT y = reinterpret_cast<const VT*>(r0)[e];
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < VN; ++c) s = fma(wv<T>(y, c), wv<T>(y, c), s);
-        acc[0] += (double)s;
-    }
-    for (int64_t e = nv * VN + threadIdx.x; e < n; e += WT) acc[0] += (double)r0[e] * (double)r0[e];
-    block_partials<1>(acc, 1, beta2);
-    __syncthreads();
-    if (threadIdx.x == 0) scale = (T)(beta2[0] > 0.0 ? 1.0 / sqrt(beta2[0]) : 0.0);
-    __syncthreads();
-    const T sc = scale;
-    for (int64_t e = threadIdx.x; e < nv; e += WT) {
-        VT y = reinterpret_cast<const VT*>(r0)[e];
-#pragma unroll
-        for (int c = 0; c < VN; ++c) wset<T>(y, c, wv<T>(y, c) * sc);
-        reinterpret_cast<VT*>(V0)[e] = y;
-    }
-    for (int64_t e = nv * VN + threadIdx.x; e < n; e += WT) V0[e] = r0[e] * sc;
-}
-
-// One block: w -= sum_{i < cnt} coef[i] V_i and nr = |w|^2 (the second Gram-Schmidt pass and the
-// norm), then Vnext = w / sqrt(nr) (Vnext != nullptr) and, on the stage's last step (lsq_k > 0), the
-// least-squares solve of the stage into y.
-template <typename T, int KC>
-__global__ void __launch_bounds__(WT) k_wgs2_one(const T* __restrict__ V, int64_t ld, int cnt,
-                                                 const double* __restrict__ coef, T* w, int64_t n,
-                                                 double* __restrict__ nr, T* __restrict__ Vnext, int lsq_k,
-                                                 const double* __restrict__ hA, const double* __restrict__ hB,
-                                                 const double* __restrict__ nrAll, const double* __restrict__ beta2,
-                                                 double* __restrict__ y) {
-    using VT = typename WVec<T>::type;
-    constexpr int VN = WVec<T>::n;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int nv = (int)(n / VN), e0 = rank * WT + tid;   // n = 3 N^2 is a multiple of VN
     pdl_entry();
-    __shared__ T scale;
-    T cf[KC];
+    cl.sync();   // every block has started: its shared memory may be written
+    VT x[E];
 #pragma unroll
-    for (int i = 0; i < KC; ++i) cf[i] = i < cnt ? (T)coef[i] : T(0);
-    double acc[1] = {0.0};
-    const int64_t nv = n / VN;
-    for (int64_t e = threadIdx.x; e < nv; e += WT) {
-        VT yv = reinterpret_cast<const VT*>(w)[e];
+    for (int q = 0; q < E; ++q) {
+        const int e = e0 + q * WC * WT;
+        if (e < nv) {
+            x[q] = reinterpret_cast<const VT*>(w)[e];
+        } else {
 #pragma unroll
-        for (int i = 0; i < KC; ++i) {
-            if (i < cnt) {
-                const VT vi = reinterpret_cast<const VT*>(V + (int64_t)i * ld)[e];
-#pragma unroll
-                for (int c = 0; c < VN; ++c) wset<T>(yv, c, fma(-cf[i], wv<T>(vi, c), wv<T>(yv, c)));
-            }
+            for (int c = 0; c < VN; ++c) wset<T>(x[q], c, T(0));
         }
-        reinterpret_cast<VT*>(w)[e] = yv;
-        T s = T(0);
-#pragma unroll
-        for (int c = 0; c < VN; ++c) s = fma(wv<T>(yv, c), wv<T>(yv, c), s);
-        acc[0] += (double)s;
     }
-    for (int64_t e = nv * VN + threadIdx.x; e < n; e += WT) {
-        T yv = w[e];
+    // sums over the cluster of acc[i], i < m, into sum[] (every block, in rank order)
+    auto reduce = [&](double (&acc)[KC], int m, int slot) {
 #pragma unroll
         for (int i = 0; i < KC; ++i)
-            if (i < cnt) yv = fma(-cf[i], V[(int64_t)i * ld + e], yv);
-        w[e] = yv;
-        acc[0] += (double)yv * (double)yv;
-    }
-    block_partials<1>(acc, 1, nr);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        scale = (T)(nr[0] > 0.0 ? 1.0 / sqrt(nr[0]) : 0.0);
-        if (lsq_k > 0) wlsq_solve(hA, hB, nrAll, beta2, lsq_k, y);
-    }
-    __syncthreads();
-    if (Vnext) {
-        const T sc = scale;
-        for (int64_t e = threadIdx.x; e < nv; e += WT) {
-            VT yv = reinterpret_cast<const VT*>(w)[e];
+            if (i < m) {
+                double v = acc[i];
+                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (lane == 0) ws[i][wid] = v;
+            }
+        __syncthreads();
+        if (tid < m) {
+            double v = 0.0;
 #pragma unroll
-            for (int c = 0; c < VN; ++c) wset<T>(yv, c, wv<T>(yv, c) * sc);
-            reinterpret_cast<VT*>(Vnext)[e] = yv;
+            for (int q = 0; q < WW; ++q) v += ws[tid][q];
+            for (int r = 0; r < WC; ++r) *cl.map_shared_rank(&part[slot][rank][tid], r) = v;
         }
-        for (int64_t e = nv * VN + threadIdx.x; e < n; e += WT) Vnext[e] = w[e] * sc;
+        cl.sync();
+        if (tid < m) {
+            double v = 0.0;
+#pragma unroll
+            for (int r = 0; r < WC; ++r) v += part[slot][r][tid];
+            sum[tid] = v;
+        }
+        __syncthreads();
+    };
+    if (cnt > 0) {
+        for (int pass = 0; pass < 2; ++pass) {
+            double acc[KC] = {};
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                const int e = e0 + q * WC * WT;
+#pragma unroll
+                for (int i = 0; i < KC; ++i)
+                    if (i < cnt && e < nv) {
+                        const VT v = reinterpret_cast<const VT*>(V + (int64_t)i * n)[e];
+                        T s = T(0);
+#pragma unroll
+                        for (int c = 0; c < VN; ++c) s = fma(wv<T>(v, c), wv<T>(x[q], c), s);
+                        acc[i] += (double)s;
+                    }
+            }
+            reduce(acc, cnt, pass);
+            if (rank == 0 && tid < cnt) (pass == 0 ? hA : hB)[tid] = sum[tid];
+            T cf[KC];
+#pragma unroll
+            for (int i = 0; i < KC; ++i) cf[i] = i < cnt ? (T)sum[i] : T(0);
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                const int e = e0 + q * WC * WT;
+#pragma unroll
+                for (int i = 0; i < KC; ++i)
+                    if (i < cnt && e < nv) {
+                        const VT v = reinterpret_cast<const VT*>(V + (int64_t)i * n)[e];
+#pragma unroll
+                        for (int c = 0; c < VN; ++c) wset<T>(x[q], c, fma(-cf[i], wv<T>(v, c), wv<T>(x[q], c)));
+                    }
+            }
+            __syncthreads();   // sum[] is read
+        }
+    }
+    double acc[KC] = {};
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+        T s = T(0);
+#pragma unroll
+        for (int c = 0; c < VN; ++c) s = fma(wv<T>(x[q], c), wv<T>(x[q], c), s);
+        acc[0] += (double)s;
+    }
+    reduce(acc, 1, 2);
+    if (rank == 0 && tid == 0) {
+        nr[0] = sum[0];
+        if (lsq_k > 0) wlsq_solve(hAll, hBll, nrAll, beta2, lsq_k, y);
+    }
+    if (!Vnext) return;
+    if (tid == 0) scale = (T)(sum[0] > 0.0 ? 1.0 / sqrt(sum[0]) : 0.0);
+    __syncthreads();
+    const T sc = scale;
+#pragma unroll
+    for (int q = 0; q < E; ++q) {
+        const int e = e0 + q * WC * WT;
+        if (e < nv) {
+#pragma unroll
+            for (int c = 0; c < VN; ++c) wset<T>(x[q], c, wv<T>(x[q], c) * sc);
+            reinterpret_cast<VT*>(Vnext)[e] = x[q];
+        }
     }
 }
 
@@ -466,14 +497,14 @@ int wrap_blocks(int64_t n) {
 
 template <typename T>
 int launch_wdots(const T* V, int64_t ld, int cnt, const T* w, int64_t n, double* partials, cudaStream_t s) {
-    const int nb = n <= WRAP_ONE_MAX ? 1 : wrap_blocks<T>(n);
+    const int nb = wrap_blocks<T>(n);
     SIB_WRAP_KC(cnt, launch_pdl(k_wdots<T, KC>, nb, WT, 0, s, V, ld, cnt, w, n, partials));
     return nb;
 }
 template <typename T>
 int launch_wgs(const T* V, int64_t ld, int cnt, const double* coef, const T* win, T* wout, int64_t n, int mode,
                double* partials, cudaStream_t s) {
-    const int nb = n <= WRAP_ONE_MAX ? 1 : wrap_blocks<T>(n);
+    const int nb = wrap_blocks<T>(n);
     if (mode == 1)
         SIB_WRAP_KC(cnt, launch_pdl(k_wgs<T, 1, KC>, nb, WT, 0, s, V, ld, cnt, coef, win, wout, n, partials));
     else
@@ -481,15 +512,33 @@ int launch_wgs(const T* V, int64_t ld, int cnt, const double* coef, const T* win
     return nb;
 }
 template <typename T>
-void launch_wnorm_one(const T* r0, int64_t n, double* beta2, T* V0, cudaStream_t s) {
-    launch_pdl(k_wnorm_one<T>, 1, WT, 0, s, r0, n, beta2, V0);
-}
-template <typename T>
-void launch_wgs2_one(const T* V, int64_t ld, int cnt, const double* coef, T* w, int64_t n, double* nr, T* Vnext,
-                     int lsq_k, const double* hA, const double* hB, const double* nrAll, const double* beta2, double* y,
-                     cudaStream_t s) {
-    SIB_WRAP_KC(cnt, launch_pdl(k_wgs2_one<T, KC>, 1, WT, 0, s, V, ld, cnt, coef, w, n, nr, Vnext, lsq_k, hA, hB,
-                                nrAll, beta2, y));
+void launch_wstep_cluster(const T* V, int64_t n, int cnt, const T* w, double* hA, double* hB, double* nr, T* Vnext,
+                          int lsq_k, const double* hAll, const double* hBll, const double* nrAll, const double* beta2,
+                          double* y, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(WC);
+    cfg.blockDim = dim3(WT);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = WC;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    // vectors of 16 bytes a thread for levels of up to 32^2, and for the largest
+    constexpr int VN = WVec<T>::n, ESMALL = 4 / VN, ELARGE = (int)(wrap_cluster_max<T> / VN / (WC * WT));
+    if constexpr (ELARGE > ESMALL) {
+        if (n > (int64_t)ESMALL * VN * WC * WT) {
+            SIB_WRAP_KC(cnt, cudaLaunchKernelEx(&cfg, k_wstep_cluster<T, KC, ELARGE>, V, n, cnt, w, hA, hB, nr, Vnext,
+                                                lsq_k, hAll, hBll, nrAll, beta2, y));
+            return;
+        }
+    }
+    SIB_WRAP_KC(cnt, cudaLaunchKernelEx(&cfg, k_wstep_cluster<T, KC, ESMALL>, V, n, cnt, w, hA, hB, nr, Vnext, lsq_k,
+                                        hAll, hBll, nrAll, beta2, y));
 }
 void launch_wreduce(const double* partials, int cnt, int nblk, double* out, cudaStream_t s) {
     launch_pdl(k_wreduce, cnt, WT, 0, s, partials, nblk, out);
@@ -514,11 +563,10 @@ void launch_wreduce_lsq(const double* partials, int nblk, double* out, const dou
                                cudaStream_t);                                                               \
     template void launch_wmaxpy<T>(const T*, int64_t, int, const double*, double, const T*, T*, int64_t,      \
                                    cudaStream_t);                                                           \
-    template void launch_wscale<T>(const T*, const double*, T*, int64_t, cudaStream_t);                      \
-    template void launch_wnorm_one<T>(const T*, int64_t, double*, T*, cudaStream_t);                         \
-    template void launch_wgs2_one<T>(const T*, int64_t, int, const double*, T*, int64_t, double*, T*, int,   \
-                                     const double*, const double*, const double*, const double*, double*,     \
-                                     cudaStream_t);
+    template void launch_wscale<T>(const T*, const double*, T*, int64_t, cudaStream_t); \
+    template void launch_wstep_cluster<T>(const T*, int64_t, int, const T*, double*, double*, double*, T*, int, \
+                                          const double*, const double*, const double*, const double*, double*, \
+                                          cudaStream_t);
 SIB_WRAP_INST(float)
 SIB_WRAP_INST(double)
 

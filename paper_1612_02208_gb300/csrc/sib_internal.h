@@ -330,15 +330,15 @@ void launch_wreduce(const double* partials, int cnt, int nblk, double* out, cuda
 // the stage's last norm (one product) and then its least-squares solve, in one single-block launch
 void launch_wreduce_lsq(const double* partials, int nblk, double* out, const double* hA, const double* hB,
                         const double* nrAll, const double* beta2, int k, double* y, cudaStream_t s);
-// Levels of at most WRAP_ONE_MAX values: one block forms each inner product completely (launch_wdots
-// and launch_wgs return nblk = 1 and write the sums themselves), the normalisations are fused
-// (launch_wnorm_one: beta2 = |r0|^2, V0 = r0 / |r0|; launch_wgs2_one: the second Gram-Schmidt pass,
-// the norm, the next Arnoldi vector and, with lsq_k > 0, the stage's least-squares solve).
-constexpr int64_t WRAP_ONE_MAX = 3 * 32 * 32;
-template <typename T> void launch_wnorm_one(const T* r0, int64_t n, double* beta2, T* V0, cudaStream_t s);
-template <typename T> void launch_wgs2_one(const T* V, int64_t ld, int cnt, const double* coef, T* w, int64_t n,
-                                           double* nr, T* Vnext, int lsq_k, const double* hA, const double* hB,
-                                           const double* nrAll, const double* beta2, double* y, cudaStream_t s);
+// Levels of at most wrap_cluster_max values (128^2 in FP32, 32^2 in FP64): an orthogonalisation step in one launch.  h (hA + hB: the two
+// passes' coefficients) against the cnt vectors V, n apart, and nr = |w|^2 afterwards; Vnext = w / |w|; lsq_k > 0: the
+// stage's least-squares solve into y.  cnt = 0: nr and Vnext alone.
+template <typename T>
+constexpr int64_t wrap_cluster_max = sizeof(T) == 4 ? 3 * 128 * 128 : 3 * 32 * 32;
+template <typename T>
+void launch_wstep_cluster(const T* V, int64_t n, int cnt, const T* w, double* hA, double* hB, double* nr, T* Vnext,
+                          int lsq_k, const double* hAll, const double* hBll, const double* nrAll, const double* beta2,
+                          double* y, cudaStream_t s);
 template <typename T> void launch_wmaxpy(const T* V, int64_t ld, int cnt, const double* coef, double sign, const T* yin,
                                          T* yout, int64_t n, cudaStream_t s);
 template <typename T> void launch_wscale(const T* w, const double* nrm2, T* v, int64_t n, cudaStream_t s);

@@ -691,13 +691,8 @@ void wrapped_smooth(sib_ctx* c, int l, const T* x, const T* b, T* xo, int k, cud
     double* beta2 = nr + WRAP_MAXK;
     double* y = beta2 + 1;
     double* part = y + WRAP_MAXK;
-    // small levels: one block forms every inner product and norm, without a reduce kernel
-    const bool one = n3 <= WRAP_ONE_MAX;
+    const bool one = n3 <= wrap_cluster_max<T>;   // a step's inner products, updates and norm in one launch
     auto dots = [&](const T* Vs, int cnt, const T* v, double* out) {
-        if (one) {
-            KL(c, launch_wdots<T>(Vs, n3, cnt, v, n3, out, s));
-            return;
-        }
         const int nb = launch_wdots<T>(Vs, n3, cnt, v, n3, part, s);
         KL(c, launch_wreduce(part, cnt, nb, out, s));
         ++c->launches;
@@ -708,7 +703,7 @@ void wrapped_smooth(sib_ctx* c, int l, const T* x, const T* b, T* xo, int k, cud
         r0 = w;
     }
     if (one) {
-        KL(c, launch_wnorm_one<T>(r0, n3, beta2, V, s));
+        KL(c, launch_wstep_cluster<T>(V, n3, 0, r0, nullptr, nullptr, beta2, V, 0, hA, hB, nr, beta2, y, s));
     } else {
         dots(r0, 1, r0, beta2);
         KL(c, launch_wscale<T>(r0, beta2, V, n3, s));
@@ -726,15 +721,14 @@ void wrapped_smooth(sib_ctx* c, int l, const T* x, const T* b, T* xo, int k, cud
             KL(c, launch_vanka_zero<T>(g, Vj, Zj, s));
         ib_apply<T>(c, l, Zj, s);
         KL(c, launch_residual<T>(gridk<T>(c, l), Zj, nullptr, w, s));   // w = L z_j
-        // CGS2: h = V^T w; w -= V h and h' = V^T w in one pass; w -= V h' and |w|^2 in one pass
-        dots(V, j + 1, w, hA + j * K1);
         if (one) {
-            KL(c, launch_wgs<T>(V, n3, j + 1, hA + j * K1, w, w, n3, 1, hB + j * K1, s));
-            KL(c, launch_wgs2_one<T>(V, n3, j + 1, hB + j * K1, w, n3, nr + j,
-                                     j + 1 < k ? V + (size_t)(j + 1) * n3 : nullptr, j + 1 < k ? 0 : k, hA, hB, nr,
-                                     beta2, y, s));
+            KL(c, launch_wstep_cluster<T>(V, n3, j + 1, w, hA + j * K1, hB + j * K1, nr + j,
+                                          j + 1 < k ? V + (size_t)(j + 1) * n3 : nullptr, j + 1 < k ? 0 : k, hA, hB, nr,
+                                          beta2, y, s));
             continue;
         }
+        // CGS2: h = V^T w; w -= V h and h' = V^T w in one pass; w -= V h' and |w|^2 in one pass
+        dots(V, j + 1, w, hA + j * K1);
         int nb = launch_wgs<T>(V, n3, j + 1, hA + j * K1, w, w, n3, 1, part, s);
         KL(c, launch_wreduce(part, j + 1, nb, hB + j * K1, s));
         nb = launch_wgs<T>(V, n3, j + 1, hB + j * K1, w, w, n3, 2, part, s);

@@ -5,7 +5,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from oracle import ib, multigrid  # noqa: E402
+from oracle import ib, multigrid, system  # noqa: E402
 from paper_1612_02208_gb300 import inputs as I  # noqa: E402
 from paper_1612_02208_gb300 import sib  # noqa: E402
 
@@ -180,4 +180,18 @@ def test_vcycle_on_the_callers_arrays(dtype, smoother):
     assert torch.equal(S.vcycle(off[1:]), z)
     same = b[:-1].clone()
     assert S.vcycle(same, same) is same and torch.equal(same, z)
+    S.close()
+
+
+# Orthogonalisation steps in a cluster: levels of up to 128^2 (the largest it takes) and 256^2 (above), stages of one
+# to five steps, both precisions; the V-cycle to the repository's bars
+@pytest.mark.parametrize("N,nu1,nu2", [(16, 1, 1), (32, 2, 3), (128, 2, 2), (128, 5, 1), (256, 1, 2)])
+def test_wrapped_steps_in_a_cluster(N, nu1, nu2):
+    prob = I.disk_stokes(N, kappa=1e2, seed=1)
+    H = multigrid.Hierarchy(prob, smoother="vanka", krylov=True, nu1=nu1, nu2=nu2)
+    S = sib.solver_for(prob, smooth_krylov=1, nu1=nu1, nu2=nu2)
+    b = system.rhs(prob).astype(np.float32).astype(np.float64)
+    ref = H.vcycle(b)
+    assert rel(host(S.vcycle(cu(b))), ref) < TOL64
+    assert rel(host(S.vcycle(cu(b, torch.float32))), ref) < 1e-4
     S.close()
