@@ -76,8 +76,9 @@ typedef struct {
     int    restart;       /* FGMRES restart length (100)                                             */
     int    add_SKXn;      /* 1: right-hand side g + S K X^n (paper form), 0: g only (1)              */
     int    use_graphs;    /* 1: replay the V-cycle as a CUDA graph (1)                               */
-    int    fuse_small;    /* 1: levels 1 and 0 of the V-cycle run as one single-block kernel when
-                             level 1 (at most 16 x 16) fits in shared memory; 0: one kernel per step (1) */
+    int    fuse_small;    /* 1: the smallest levels of the V-cycle run as one launch where they fit in shared
+                             memory: FP32 Vanka up to 32 x 32, else levels 1 (at most 16 x 16) and 0;
+                             0: one kernel per step (1)                                               */
     int    smooth_krylov; /* 1: every pre- and post-smoothing stage of nu sweeps is nu iterations of
                              flexible GMRES on the level's residual equation, each preconditioned by
                              one undamped basic sweep (Sec. 3.3; nu <= 8); 0: nu damped sweeps (0)    */
