@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(512) k_gj_panel_wide(const double* __restrict_
     float* fac = Wp + (size_t)n * GJ_B;                   // n: column t before the pivot's elimination
     int* usedS = reinterpret_cast<int*>(fac + n);         // n
     __shared__ float prowv[GJ_B];
-    __shared__ float wv[32];
+    __shared__ unsigned wv[32];
     __shared__ int wi[32];
     __shared__ int pS[GJ_B];
     const int ld = 2 * n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -346,40 +346,32 @@ __global__ void __launch_bounds__(512) k_gj_panel_wide(const double* __restrict_
     for (int r = threadIdx.x; r < n; r += blockDim.x) usedS[r] = c0 == 0 ? 0 : w.used[r];
     __syncthreads();
     for (int t = 0; t < GJ_B; ++t) {
-        float best = -1.0f;
+        // magnitudes order as their bits do; 0: no candidate, 1: a zero (or not a number), so that a row of the matrix is
+        // chosen whatever its values
+        unsigned best = 0u;
         int bi = n;
+        auto take = [&](unsigned key, int row) {   // ties to the lower row
+            if (key > best || (key == best && row < bi)) {
+                best = key;
+                bi = row;
+            }
+        };
         for (int r = threadIdx.x; r < n; r += blockDim.x) {
             if (usedS[r]) continue;
-            const float a = fabsf(Wp[r * GJ_B + t]);
-            if (a > best) {
-                best = a;
-                bi = r;
-            }
+            const float m = fabsf(Wp[r * GJ_B + t]);
+            take(m >= 0.0f ? __float_as_uint(m) + 1u : 1u, r);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-            if (ob > best || (ob == best && oi < bi)) {
-                best = ob;
-                bi = oi;
-            }
-        }
+        for (int o = 16; o > 0; o >>= 1) take(__shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
         if (lane == 0) {
             wv[wid] = best;
             wi[wid] = bi;
         }
         __syncthreads();
         if (wid == 0) {
-            best = lane < nw ? wv[lane] : -1.0f;
+            best = lane < nw ? wv[lane] : 0u;
             bi = lane < nw ? wi[lane] : n;
-            for (int o = 16; o > 0; o >>= 1) {
-                const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-                if (ob > best || (ob == best && oi < bi)) {
-                    best = ob;
-                    bi = oi;
-                }
-            }
+            for (int o = 16; o > 0; o >>= 1)
+                take(__shfl_xor_sync(0xffffffffu, best, o), __shfl_xor_sync(0xffffffffu, bi, o));
             if (lane == 0) {
                 pS[t] = bi;
                 usedS[bi] = 1;
