@@ -196,7 +196,8 @@ void launch_assemble_L0(int N0, double rho, double mu, double dt, const double* 
 //   3. every other row r becomes  A_r - A_rQ W  there (A_rQ: its panel entries before the panel's
 //      elimination), and its panel entries 0 (the pivot rows' panel entries become unit vectors).
 // Rows are never swapped: piv[k] is the pivot row of column k and row k of A^{-1} is
-// Aug[piv[k]][n:].  info = 0, or k + 1 for the first pivot column without a nonzero candidate.
+// Aug[piv[k]][n:].  A zero *info (the caller clears it, once for a series of inversions that share the word) becomes
+// k + 1 for the first pivot column without a nonzero candidate.
 // The panel steps are sequential but tiny; the O(n^3) work of step 3 spreads over the GPU, whose
 // FP64 rate is low per SM.
 constexpr int GJ_B = 16;
@@ -273,7 +274,6 @@ __global__ void __launch_bounds__(GJ_MAXN) k_gj_panel(const double* __restrict__
     __shared__ int crow[2][32];
     __shared__ int pS[GJ_B];
     const int r = threadIdx.x, lane = r & 31, wid = r >> 5, nw = blockDim.x >> 5;
-    if (c0 == 0 && r == 0) *info = 0;
     float a[GJ_B] = {};
     bool used = true;
     if (r < n) {
@@ -337,7 +337,6 @@ __global__ void __launch_bounds__(512) k_gj_panel_wide(const double* __restrict_
     __shared__ int wi[32];
     __shared__ int pS[GJ_B];
     const int ld = 2 * n, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (c0 == 0 && threadIdx.x == 0) *info = 0;
     for (int q = threadIdx.x; q < n * GJ_B; q += blockDim.x) {
         const double v = A[(size_t)(q / GJ_B) * ld + c0 + (q % GJ_B)];
         Wp[q] = (float)v;

@@ -1574,6 +1574,7 @@ void setup(sib_ctx* c, cudaStream_t s) {
         else
             KL(c, launch_assemble_L0(c->L[0].N, c->rho, c->mu, c->dt, c->B0, c->Aug, s));
         CK(cudaEventRecord(c->evFork, s));
+        CK(cudaMemsetAsync(c->info, 0, sizeof(int), c->aux));
         CK(cudaStreamWaitEvent(c->aux, c->evFork, 0));
         KL(c, launch_gauss_jordan(c->Aug, n, c->info, c->piv, c->gjWork, c->aux));
         // the gauge's Z Z^T comes off the pressure block alone in the cavity (passed as rho != 0)

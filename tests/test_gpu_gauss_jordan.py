@@ -63,3 +63,18 @@ def test_pivot_rows(n, where):
     assert np.array_equal(np.sort(piv), np.arange(n))
     if where == "nowhere":   # backward stable up to growth: a few n eps of condition number <= 3
         assert np.abs(inv @ A - np.eye(n)).max() < 64 * n * 2.0 ** -53
+
+
+# A singular matrix (a zero column: its pivot is exactly zero) reports its column, and a regular one inverted
+# after it with the same word leaves the report; both panels
+@pytest.mark.parametrize("n", [48, 784])
+def test_singular_report_stays(n):
+    I = Inversion()
+    I.run(matrix(n, 1))
+    assert I.info.item() == 0
+    A = matrix(n, 2)
+    A[:, 20] = 0.0
+    I.run(A)
+    assert I.info.item() == 21
+    I.run(matrix(n, 3))
+    assert I.info.item() == 21
