@@ -1023,11 +1023,7 @@ void launch_residual_restrict(const GridK<T>& g, const T* x, const T* b, T* bc, 
         if (g.N >= RR_MIN) {
             const int Nc = g.N / 2;
             const size_t smem = sizeof(T) * (size_t)RR_WORDS + 128;   // 128: room to align the staged tile
-            static thread_local bool enabled = false;
-            if (!enabled) {
-                cudaFuncSetAttribute(k_residual_restrict_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-                enabled = true;
-            }
+            allow_smem(k_residual_restrict_tiled, smem);
             CUtensorMap mx, mb, mf;
             std::memset(&mx, 0, sizeof(mx));
             std::memset(&mb, 0, sizeof(mb));

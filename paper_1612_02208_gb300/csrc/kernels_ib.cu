@@ -959,7 +959,7 @@ void launch_dense_ib(const IBK<double>& k, const int* adjStart, const int* adjNb
     int threads = 256;
     while (threads > 32 && (size_t)threads * n0 * sizeof(double) > 128 * 1024) threads /= 2;
     const size_t smem = (size_t)threads * n0 * sizeof(double);
-    cudaFuncSetAttribute(k_dense_ib, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_dense_ib, smem);
     launch_pdl(k_dense_ib, dim3(n0, 2), dim3(threads), smem, s, k, adjStart, adjNbr, adjKap, B);
 }
 

@@ -448,7 +448,7 @@ void launch_gauss_jordan(double* Aug, int n, int* info, int* piv, void* work, cu
     const GjWork w = gj_work(work, n);
     const size_t smem = sizeof(float) * ((size_t)n * GJ_B + n) + sizeof(int) * (size_t)n;
     const bool wide = n > GJ_MAXN;   // the box smoothers' largest subdomains
-    if (wide) cudaFuncSetAttribute(k_gj_panel_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (wide) allow_smem(k_gj_panel_wide, smem);
     const int ld = 2 * n;
     for (int c0 = 0; c0 < n; c0 += GJ_B) {
         if (wide)
@@ -700,7 +700,7 @@ void launch_multidot_dev(const double* V, int64_t ld, const double* w, int64_t n
                          const FgDev* st, cudaStream_t s) {
     const int64_t nb = (FG_MAXM + MD_G - 1) / MD_G * ((n + MD_SLICE - 1) / MD_SLICE);
     const bool wave = n >= (int64_t)MD_SLICE * MD_BLOCKS;
-    if (wave) cudaFuncSetAttribute(k_multidot_dev, cudaFuncAttributeMaxDynamicSharedMemorySize, GS_RESERVE);
+    if (wave) allow_smem(k_multidot_dev, GS_RESERVE);
     launch_pdl(k_multidot_dev, (int)std::min<int64_t>(MD_BLOCKS, nb), 256, wave ? GS_RESERVE : 0, s, V, ld, w, n, partials,
                st, wave);
 }
@@ -776,7 +776,7 @@ int launch_gs_update_dev(const double* V, int64_t ld, const double* dots, double
     const int nb = std::min(num_blocks_for(n / 2), GS_BLOCKS);
     const bool wave = n >= (int64_t)MD_SLICE * MD_BLOCKS;   // as k_multidot_dev
     auto kern = partials ? k_gs_update_dev<true> : k_gs_update_dev<false>;
-    if (wave) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GS_RESERVE);
+    if (wave) allow_smem(kern, GS_RESERVE);
     launch_pdl(kern, nb, 256, wave ? GS_RESERVE : 0, s, V, ld, dots, h, y, n, st, partials, wave);
     return nb;
 }

@@ -1791,9 +1791,9 @@ void launch_ras_setup_be(int N, int b, int o, const RasIB& ib, double a0, double
     const size_t nu = be_nu(G.e), np = (size_t)G.e * G.e;
     const size_t sv = sizeof(double) * (nu * (nu + 1) / 2 + 2 * nu), sp = sizeof(double) * (np * (np + 1) / 2 + 2 * np);
     const size_t so = sizeof(double) * (2 * BE_ROWS * np + (size_t)BE_KC * BE_COLS);
-    cudaFuncSetAttribute(k_ras_be_velocity, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sv);
-    cudaFuncSetAttribute(k_ras_be_pressure, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sp);
-    cudaFuncSetAttribute(k_ras_be_owned, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)so);
+    allow_smem(k_ras_be_velocity, sv);
+    allow_smem(k_ras_be_pressure, sp);
+    allow_smem(k_ras_be_owned, so);
     k_ras_be_velocity<<<dim3(count, 2), BE_THREADS, sv, s>>>(G, ib, a0, c, dt, list, first, work, info);
     k_ras_be_pressure<<<count, BE_THREADS, sp, s>>>(G, inv_h, work, info);
     k_ras_be_owned<<<dim3(count, (G.nown + BE_ROWS - 1) / BE_ROWS), BE_THREADS, so, s>>>(G, inv_h, work, first, inv64,
@@ -1815,11 +1815,7 @@ void launch_ras_apply_big(const RasGeo& G, const int* slotOfBox, const T* inv, T
                           cudaStream_t s) {
     using TL = RasTile<T>;
     const size_t smem = sizeof(T) * ((size_t)RAS_KC * G.nown + (size_t)RAS_KC * TL::NBX) + sizeof(int) * G.ne;
-    static thread_local size_t allowed = 48 * 1024;   // dynamic shared memory the kernel is enabled for
-    if (smem > allowed) {
-        cudaFuncSetAttribute(k_ras_apply_big<T, RA>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        allowed = smem;
-    }
+    allow_smem(k_ras_apply_big<T, RA>, smem);
     const int tiles = (G.nbs * G.nbs + TL::NBX - 1) / TL::NBX;
     launch_pdl(k_ras_apply_big<T, RA>, dim3(tiles), dim3(32 * RAS_BW), smem, s, G, slotOfBox, inv, omega, r, x, xo);
 }
@@ -1875,14 +1871,10 @@ bool launch_ras_apply_tc(int N, int b, int o, const int* slotOfBox, const float*
     nsb = std::min(nsb, RT_MAXSB);
     if (nsb < 2) return false;   // b + 2 o <= 16 leaves room for three inverse stages in 227 KB
     const size_t smem = fixed + (size_t)nsb * bChunk;
-    static thread_local size_t allowed[2] = {48 * 1024, 48 * 1024};
-    if (smem > allowed[nc == 48]) {
-        if (nc == 48)
-            cudaFuncSetAttribute(k_ras_apply_tc<48, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        else
-            cudaFuncSetAttribute(k_ras_apply_tc<16, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        allowed[nc == 48] = smem;
-    }
+    if (nc == 48)
+        allow_smem(k_ras_apply_tc<48, 1>, smem);
+    else
+        allow_smem(k_ras_apply_tc<16, 2>, smem);
     const int ntiles = (G.nbs * G.nbs + RT_NB - 1) / RT_NB;
     // 16 worker warps and the issuing warp; row groups (16 x 16 boxes) side by side along y
     const dim3 grd(std::min(ntiles, sms), groups), blk(RT_THREADS + 32);
@@ -1923,7 +1915,7 @@ void launch_ras_wb_setup(int N, int b, int o, const RasIB& ib, double dt, const 
     const int nw = RAS_WB_THREADS / 32;
     const size_t smem = sizeof(double) * (3 * (size_t)mmax + 32) +
                         sizeof(int) * (32 + nw * WIN_SIZE + ((nw * WIN_SIZE) & 1)) + sizeof(double) * nw * WIN_SIZE;
-    if (smem > 48 * 1024) cudaFuncSetAttribute(k_ras_wb_setup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(k_ras_wb_setup, smem);
     k_ras_wb_setup<<<nIB, RAS_WB_THREADS, smem, s>>>(ras_geo(N, b, o), ib, dt, list, offT, T, offW, inv0, work, W,
                                                      info, mOneMax);
 }
@@ -1963,11 +1955,7 @@ void launch_ras_huge_apply(int N, int b, int o, const T* inv, T omega, const T* 
     if (count <= 0) return;
     const RasGeo G = ras_geo(N, b, o);
     const size_t smem = sizeof(T) * RH_BX * (size_t)G.ne;
-    static thread_local size_t allowed = 48 * 1024;
-    if (smem > allowed) {
-        cudaFuncSetAttribute(k_ras_huge_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        allowed = smem;
-    }
+    allow_smem(k_ras_huge_apply<T>, smem);
     // row splits: about two blocks per SM in all, at most one warp's row per split and warp
     const int boxBlocks = (count + RH_BX - 1) / RH_BX, nw = RH_THREADS / 32;
     const int splits = std::max(1, std::min((2 * 152 + boxBlocks - 1) / boxBlocks, (G.nown + nw - 1) / nw));
@@ -2168,12 +2156,8 @@ void launch_ras_wb_apply32(int N, int b, int o, const int* list, int nIB, const 
     float2* yT = reinterpret_cast<float2*>(rk + (size_t)st * nIB);
     const int groups = (nIB + WB_BX - 1) / WB_BX, nw = WB_THREADS / 32;
     const size_t smem1 = sizeof(float) * WB_BX * (size_t)st, smem3 = 2 * smem1;
-    static thread_local size_t allowed = 0;
-    if (smem3 > allowed) {
-        cudaFuncSetAttribute(k_ras_wb_rows<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem1);
-        cudaFuncSetAttribute(k_ras_wb_rows<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem3);
-        allowed = smem3;
-    }
+    allow_smem(k_ras_wb_rows<false>, smem1);
+    allow_smem(k_ras_wb_rows<true>, smem3);
     // rows per block: one wave of the blocks that shared memory lets an SM hold, a row per warp at least
     auto rows_for = [&](int total, int perSM) {
         const int blocks = std::max(1, perSM * 152 / groups);
@@ -2196,11 +2180,7 @@ void launch_ras_wb_apply64(int N, int b, int o, const RasIB& ib, double a0, doub
     if (nIB <= 0) return;
     const RasGeo G = ras_geo(N, b, o);
     const size_t smem = sizeof(double) * (4 * (size_t)G.ne + (size_t)mmax);
-    static thread_local size_t allowed = 48 * 1024;
-    if (smem > allowed) {
-        cudaFuncSetAttribute(k_ras_wb_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        allowed = smem;
-    }
+    allow_smem(k_ras_wb_apply, smem);
     launch_pdl(k_ras_wb_apply, dim3(nIB), dim3(256), smem, s, G, ib, a0, c, inv_h, dt, list, offT, Tl, offW, W,
                inv0, omega, r, xo);
 }
@@ -2231,7 +2211,7 @@ int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list,
         const int nb = ngroups > 0 ? RAS_SP_NB : 1;
         const size_t smem = sizeof(T) * nb * ((size_t)G.ne + (size_t)p.ks * p.rc);
         auto kern = ngroups > 0 ? k_ras_apply_split<T, true> : k_ras_apply_split<T, false>;
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        allow_smem(kern, smem);
         launch_pdl(kern, dim3((nIB + ngroups) * p.chunks), dim3(p.threads), smem, s, G, p, list, nIB,
                    slotOfBox, inv, omega, r, x, xo);
     };
@@ -2268,7 +2248,7 @@ int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list,
         static thread_local size_t cachedSmem = 0;   // persistent grid: the blocks resident at once, per size
         static thread_local int resident = 1;
         if (smem != cachedSmem) {
-            cudaFuncSetAttribute(k_ras_apply<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            allow_smem(k_ras_apply<T>, smem);
             int dev = 0, sms = 0, per = 0;
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

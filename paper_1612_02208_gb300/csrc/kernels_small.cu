@@ -645,7 +645,7 @@ bool vcycle_cluster_fits(size_t smem) {
     cudaLaunchConfig_t cfg = cluster_config(smem, attr);
     cfg.numAttrs = 1;
     int clusters = 0;
-    if (cudaFuncSetAttribute(k_vcycle_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(k_vcycle_cluster, smem) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&clusters, k_vcycle_cluster, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -653,7 +653,7 @@ bool vcycle_cluster_fits(size_t smem) {
     return clusters > 0;
 }
 cudaError_t launch_vcycle_cluster(const ClusterArgs& a, size_t smem, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_vcycle_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_vcycle_cluster, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = cluster_config(smem, attr);
@@ -670,7 +670,7 @@ size_t vcycle_small_smem(int N1, int n0, int nTiles, int per, int ntiles) {
 // if such a cluster cannot be resident with `smem` bytes per block.
 template <typename T>
 int vcycle_small_cluster(size_t smem) {
-    if (cudaFuncSetAttribute(k_vcycle_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    if (allow_smem(k_vcycle_small<T>, smem) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
@@ -695,7 +695,7 @@ int vcycle_small_cluster(size_t smem) {
 
 template <typename T>
 cudaError_t launch_vcycle_small(const SmallArgs<T>& a, size_t smem, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_vcycle_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k_vcycle_small<T>, smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(SMALL_CLUSTER);

@@ -3,7 +3,10 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <map>
+#include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "sib.h"
@@ -53,6 +56,32 @@ inline void launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t sme
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+// Lets `kern` be launched with `bytes` of dynamic shared memory.  That limit belongs to the function and is shared by
+// every host thread and context of the process, so it is only ever raised: set to each launch's own size, a thread with
+// a smaller case would lower it under another's launch.
+inline cudaError_t allow_smem_of(const void* kern, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<int, const void*>, size_t> limits;   // by device and function
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = limits.find({dev, kern});
+    if (it == limits.end()) {
+        cudaFuncAttributes fa;
+        if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
+        it = limits.emplace(std::make_pair(dev, kern), (size_t)fa.maxDynamicSharedSizeBytes).first;
+    }
+    if (bytes <= it->second) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) it->second = bytes;
+    return e;
+}
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kern)(KArgs...), size_t bytes) {
+    return allow_smem_of(reinterpret_cast<const void*>(kern), bytes);
 }
 
 // ------------------------------------------------------------------------------------------
