@@ -6,6 +6,7 @@
 #include <cstring>
 #include <stdexcept>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "sib_internal.h"
@@ -127,7 +128,7 @@ struct sib_ctx {
     int smemOptin = 0;           // largest dynamic shared memory of one block
     int64_t bytes = 0;
     double setup_ms = 0.0;
-    std::vector<void*> allocs;
+    std::vector<std::pair<void*, size_t>> allocs;
     cudaStream_t cap = nullptr;
     void* gjWork = nullptr;              // work arrays of the blocked Gauss-Jordan inversion
     cudaStream_t aux = nullptr;          // set-up work that runs beside the main stream
@@ -212,14 +213,15 @@ void* dalloc(sib_ctx* c, size_t bytes) {
         cudaGetLastError();
         throw SibError(SIB_ERR_ALLOC, "cudaMalloc of " + std::to_string(bytes) + " bytes failed");
     }
-    c->allocs.push_back(p);
+    c->allocs.emplace_back(p, bytes);
     c->bytes += (int64_t)bytes;
     return p;
 }
 void dfree(sib_ctx* c, void* p) {
     if (!p) return;
     for (size_t k = 0; k < c->allocs.size(); ++k)
-        if (c->allocs[k] == p) {
+        if (c->allocs[k].first == p) {
+            c->bytes -= (int64_t)c->allocs[k].second;
             c->allocs.erase(c->allocs.begin() + k);
             break;
         }
@@ -2292,7 +2294,7 @@ int sib_create(sib_ctx** out, int N, int n_min) {
 void sib_destroy(sib_ctx* c) {
     if (!c) return;
     invalidate_graphs(c);
-    for (void* p : c->allocs) cudaFree(p);
+    for (const auto& a : c->allocs) cudaFree(a.first);
     c->allocs.clear();
     if (c->hbuf) cudaFreeHost(c->hbuf);
     if (c->herr) cudaFreeHost(c->herr);
