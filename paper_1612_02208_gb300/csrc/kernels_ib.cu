@@ -691,13 +691,55 @@ __global__ void __launch_bounds__(TX * (TY + SP_MAXW - 1))
     f[(size_t)c * k.N * k.N + (size_t)(j0 + r) * k.N + i0 + x] = k.inv_h2 * sum;
 }
 
+// The same with a warp per face, whose lanes share each bin's markers: structures with crowded cells
+// (spread_crowded), which k_spread_tile walks with one thread per column and bin row.
+template <typename T>
+__global__ void __launch_bounds__(256) k_spread_crowded(IBK<T> k, const T* __restrict__ F, T* __restrict__ f,
+                                                        const int* __restrict__ tiles, const int* __restrict__ nTiles,
+                                                        const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
+    pdl_entry();
+    const int lane = threadIdx.x & 31, face = blockIdx.y * 8 + (threadIdx.x >> 5), per = tx * ty, mk = k.N - 1, W = k.W;
+    if ((int)blockIdx.x >= *nTiles || face >= 2 * per) return;
+    const int c = face >= per, q = face - c * per, t = tiles[rowSlots ? rowSlots[blockIdx.x] : blockIdx.x];
+    const int i = (t % ntx) * tx + q % tx, j = (t / ntx) * ty + q / tx;
+    const int* bs = c ? k.binStart[1] : k.binStart[0];
+    const int* srt = c ? k.sorted[1] : k.sorted[0];
+    const T* wg = c ? k.wgt[1] : k.wgt[0];
+    const T* Fc = F + c * k.M;
+    int s[SP_MAXW * SP_MAXW], e[SP_MAXW * SP_MAXW];   // the bins' ranges first: independent loads
+#pragma unroll
+    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n) {
+        const int a = n % SP_MAXW, b = n / SP_MAXW;
+        s[n] = e[n] = 0;
+        if (a < W && b < W) {
+            const uint32_t bin = morton((i - a) & mk, (j - b) & mk);
+            s[n] = bs[bin];
+            e[n] = bs[bin + 1];
+        }
+    }
+    T acc = T(0);
+#pragma unroll
+    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n)
+        for (int p = s[n] + lane; p < e[n]; p += 32) {
+            const int m = srt[p];
+            acc += wg[8 * m + 4 + n / SP_MAXW] * (wg[8 * m + n % SP_MAXW] * Fc[m]);
+        }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) f[(size_t)c * k.N * k.N + (size_t)j * k.N + i] = k.inv_h2 * acc;
+}
+
 // With rowSlots (nRow its count, maxTiles its host bound) only the tiles that a marker stencil touches
 // are written; the caller keeps f at zero on the other active tiles.
 template <typename T>
 void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles, int maxTiles, int tx,
-                   int ty, int ntx, cudaStream_t s, const int* rowSlots, const int* nRow) {
+                   int ty, int ntx, bool crowded, cudaStream_t s, const int* rowSlots, const int* nRow) {
     if (maxTiles == 0) return;
     const int* cnt = rowSlots ? nRow : nTiles;
+    if (crowded) {
+        launch_pdl(k_spread_crowded<T>, dim3(maxTiles, (2 * tx * ty + 7) / 8), 256, 0, s, k, F, f, tiles, cnt, rowSlots, tx,
+                   ty, ntx);
+        return;
+    }
     launch_pdl(k_spread_tile<T>, dim3(maxTiles, 2), dim3(tx, ty + k.W - 1), 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty,
                ntx);
 }
@@ -1472,7 +1514,7 @@ void launch_grad_X(const double* X, int M, int N, const double* w, const double*
     template void launch_interp<T>(const IBK<T>&, const T*, T*, cudaStream_t);                                  \
     template void launch_spring<T>(const int*, const int*, const T*, int, const T*, T*, cudaStream_t);           \
     template void launch_spread<T>(const IBK<T>&, const T*, T*, const int*, const int*, int, int, int, int,      \
-                                   cudaStream_t, const int*, const int*);
+                                   bool, cudaStream_t, const int*, const int*);
 SIB_IB_INST(float)
 SIB_IB_INST(double)
 

@@ -407,8 +407,15 @@ template <typename T> void launch_spring(const int* start, const int* nbr, const
                                          cudaStream_t s);
 // rowSlots != nullptr: only the tiles of that slot list (count *nRow, at most maxTiles) are written
 template <typename T> void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles,
-                                         int maxTiles, int tx, int ty, int ntx, cudaStream_t s,
+                                         int maxTiles, int tx, int ty, int ntx, bool crowded, cudaStream_t s,
                                          const int* rowSlots = nullptr, const int* nRow = nullptr);
+// Structures whose M markers take the form with a warp per face, by the largest number in one cell: the other waits for
+// one thread to walk its W bins (about 1.8 us per marker of the largest), this one reads every marker for each of its W^2
+// faces (0.3 ns a marker and 15 us).  FP64, us with a thread per column and bin row / a warp per face: 128^2, 5,000
+// markers in one cell 1,592 / 44, 78 a cell in 16 x 16 cells 167 / 42; along a line 16 a cell 37 / 23, 195 a cell 359 / 39
+// (512^2: 8 a cell 28 / 35, 16 a cell 40 / 34, 195 a cell 367 / 71); evenly over 128^2 4 a cell 29 / 92, 40 a cell 186 / 212,
+// 128 a cell 644 / 666.
+inline bool spread_crowded(int most, int M) { return most > 24 + M / 6000; }
 // the spreading's walk stored at set-up (rows: faces of the stencil-touched tiles, entries in the
 // gather's order, cap = 2 M W^2), then applied as one ordered dot product per face
 void launch_spread_store(const IBK<double>& k, const float* w32u, const float* w32v, const int* tiles,
