@@ -252,7 +252,8 @@ int sib_time_kernel(sib_ctx* ctx, int kernel, int level, int prec, int reps, voi
 
 /* ---- spreading without device allocation ----------------------------------------------------- */
 /* f = S F on an N x N grid for markers X (M x 2) and forces F (M x 2), written to the caller's
- * f (2 N^2 values [f_u | f_v]); the same result as sib_spread without a solver context.
+ * f (2 N^2 values [f_u | f_v]); the same result as sib_spread without a solver context
+ * (to rounding where one cell holds more than 24 markers).
  * The paper has no counterpart: this is for callers that cannot allocate device memory, such as
  * programs whose device memory is owned by their own pool allocator (a raw cudaMalloc would fail
  * or fragment it) and latency-critical loops that cannot afford the device-wide synchronisation

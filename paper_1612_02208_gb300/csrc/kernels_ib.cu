@@ -631,11 +631,45 @@ void launch_spring(const int* start, const int* nbr, const T* kap, int M, const 
 // bins of four markers.  1024^2 disk and ellipse, 3e5 markers, FP64: interpolation, spreading and operator
 // together 722 us with the warp per face (598 us of it the spreading), 204 us so (66 us).
 constexpr int SP_MAXW = 4;
+constexpr int SP_CROWD = 24;   // markers of a crowded cell
+constexpr int SP_BLOCKS = 8;
 template <typename T>
 struct alignas(16) Wgt4 {   // half of a marker's eight weights: 16 bytes (FP32) or 32 (FP64), aligned to them
     T v[4];
 };
+// The sum of face (i, j) of component c by a warp, whose lanes share each bin's markers
 template <typename T>
+__device__ __forceinline__ T spread_face_sum(const IBK<T>& k, const T* __restrict__ F, int c, int i, int j, int lane) {
+    const int mk = k.N - 1, W = k.W;
+    const int* bs = c ? k.binStart[1] : k.binStart[0];
+    const int* srt = c ? k.sorted[1] : k.sorted[0];
+    const T* wg = c ? k.wgt[1] : k.wgt[0];
+    const T* Fc = F + c * k.M;
+    int s[SP_MAXW * SP_MAXW], e[SP_MAXW * SP_MAXW];   // the bins' ranges first: independent loads
+#pragma unroll
+    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n) {
+        const int a = n % SP_MAXW, b = n / SP_MAXW;
+        s[n] = e[n] = 0;
+        if (a < W && b < W) {
+            const uint32_t bin = morton((i - a) & mk, (j - b) & mk);
+            s[n] = bs[bin];
+            e[n] = bs[bin + 1];
+        }
+    }
+    T acc = T(0);
+#pragma unroll
+    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n)
+        for (int p = s[n] + lane; p < e[n]; p += 32) {
+            const int m = srt[p];
+            acc += wg[8 * m + 4 + n / SP_MAXW] * (wg[8 * m + n % SP_MAXW] * Fc[m]);
+        }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    return acc;
+}
+// BYTILE: a tile with a crowded cell is summed a warp per face here, by the blocks along z, for the caller that does not
+// know the cells' counts on the host (sib_spread_noalloc at 64^2, the call: one cell of 4,000 markers 1,554 -> 179 us,
+// 39 a cell along a line 209 -> 163, 16,384 evenly 214 -> 215).
+template <typename T, bool BYTILE>
 __global__ void __launch_bounds__(TX * (TY + SP_MAXW - 1))
     k_spread_tile(IBK<T> k, const T* __restrict__ F, T* __restrict__ f, const int* __restrict__ tiles,
                   const int* __restrict__ nTiles, const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
@@ -664,6 +698,20 @@ __global__ void __launch_bounds__(TX * (TY + SP_MAXW - 1))
         total += e0 - s0;
         end[a] = total;
     }
+    if (BYTILE && tx == TX) {   // full warps, one bin row each; the blocks along z share a crowded tile's faces
+        int most = end[0];
+#pragma unroll
+        for (int a = 1; a < SP_MAXW; ++a) most = max(most, end[a] - end[a - 1]);
+        if (__syncthreads_or(most > SP_CROWD)) {
+            for (int q = r + blockIdx.z * blockDim.y; q < tx * ty; q += gridDim.z * blockDim.y) {
+                const int i = i0 + q % tx, j = j0 + q / tx;
+                const T sum = spread_face_sum(k, F, c, i, j, x);
+                if (x == 0) f[(size_t)c * k.N * k.N + (size_t)j * k.N + i] = k.inv_h2 * sum;
+            }
+            return;
+        }
+        if (blockIdx.z > 0) return;
+    }
     // face rows of the tile that this bin row reaches: r - (W - 1) + b in [0, ty)
     const int blo = max(0, W - 1 - r), bhi = min(W, ty + W - 1 - r);
     T acc[SP_MAXW];
@@ -691,57 +739,36 @@ __global__ void __launch_bounds__(TX * (TY + SP_MAXW - 1))
     f[(size_t)c * k.N * k.N + (size_t)(j0 + r) * k.N + i0 + x] = k.inv_h2 * sum;
 }
 
-// The same with a warp per face, whose lanes share each bin's markers: structures with crowded cells
-// (spread_crowded), which k_spread_tile walks with one thread per column and bin row.
+// The same with a warp per face: structures with crowded cells (spread_crowded), which k_spread_tile walks with one
+// thread per column and bin row.
 template <typename T>
 __global__ void __launch_bounds__(256) k_spread_crowded(IBK<T> k, const T* __restrict__ F, T* __restrict__ f,
                                                         const int* __restrict__ tiles, const int* __restrict__ nTiles,
                                                         const int* __restrict__ rowSlots, int tx, int ty, int ntx) {
     pdl_entry();
-    const int lane = threadIdx.x & 31, face = blockIdx.y * 8 + (threadIdx.x >> 5), per = tx * ty, mk = k.N - 1, W = k.W;
+    const int lane = threadIdx.x & 31, face = blockIdx.y * 8 + (threadIdx.x >> 5), per = tx * ty;
     if ((int)blockIdx.x >= *nTiles || face >= 2 * per) return;
     const int c = face >= per, q = face - c * per, t = tiles[rowSlots ? rowSlots[blockIdx.x] : blockIdx.x];
     const int i = (t % ntx) * tx + q % tx, j = (t / ntx) * ty + q / tx;
-    const int* bs = c ? k.binStart[1] : k.binStart[0];
-    const int* srt = c ? k.sorted[1] : k.sorted[0];
-    const T* wg = c ? k.wgt[1] : k.wgt[0];
-    const T* Fc = F + c * k.M;
-    int s[SP_MAXW * SP_MAXW], e[SP_MAXW * SP_MAXW];   // the bins' ranges first: independent loads
-#pragma unroll
-    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n) {
-        const int a = n % SP_MAXW, b = n / SP_MAXW;
-        s[n] = e[n] = 0;
-        if (a < W && b < W) {
-            const uint32_t bin = morton((i - a) & mk, (j - b) & mk);
-            s[n] = bs[bin];
-            e[n] = bs[bin + 1];
-        }
-    }
-    T acc = T(0);
-#pragma unroll
-    for (int n = 0; n < SP_MAXW * SP_MAXW; ++n)
-        for (int p = s[n] + lane; p < e[n]; p += 32) {
-            const int m = srt[p];
-            acc += wg[8 * m + 4 + n / SP_MAXW] * (wg[8 * m + n % SP_MAXW] * Fc[m]);
-        }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) f[(size_t)c * k.N * k.N + (size_t)j * k.N + i] = k.inv_h2 * acc;
+    const T sum = spread_face_sum(k, F, c, i, j, lane);
+    if (lane == 0) f[(size_t)c * k.N * k.N + (size_t)j * k.N + i] = k.inv_h2 * sum;
 }
 
 // With rowSlots (nRow its count, maxTiles its host bound) only the tiles that a marker stencil touches
 // are written; the caller keeps f at zero on the other active tiles.
 template <typename T>
 void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles, int maxTiles, int tx,
-                   int ty, int ntx, bool crowded, cudaStream_t s, const int* rowSlots, const int* nRow) {
+                   int ty, int ntx, SpreadForm form, cudaStream_t s, const int* rowSlots, const int* nRow) {
     if (maxTiles == 0) return;
     const int* cnt = rowSlots ? nRow : nTiles;
-    if (crowded) {
+    const dim3 blk(tx, ty + k.W - 1);
+    if (form == SPREAD_CROWDED)
         launch_pdl(k_spread_crowded<T>, dim3(maxTiles, (2 * tx * ty + 7) / 8), 256, 0, s, k, F, f, tiles, cnt, rowSlots, tx,
                    ty, ntx);
-        return;
-    }
-    launch_pdl(k_spread_tile<T>, dim3(maxTiles, 2), dim3(tx, ty + k.W - 1), 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty,
-               ntx);
+    else if (form == SPREAD_BY_TILE)
+        launch_pdl(k_spread_tile<T, true>, dim3(maxTiles, 2, tx == TX ? SP_BLOCKS : 1), blk, 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty, ntx);
+    else
+        launch_pdl(k_spread_tile<T, false>, dim3(maxTiles, 2), blk, 0, s, k, F, f, tiles, cnt, rowSlots, tx, ty, ntx);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1514,7 +1541,7 @@ void launch_grad_X(const double* X, int M, int N, const double* w, const double*
     template void launch_interp<T>(const IBK<T>&, const T*, T*, cudaStream_t);                                  \
     template void launch_spring<T>(const int*, const int*, const T*, int, const T*, T*, cudaStream_t);           \
     template void launch_spread<T>(const IBK<T>&, const T*, T*, const int*, const int*, int, int, int, int,      \
-                                   bool, cudaStream_t, const int*, const int*);
+                                   SpreadForm, cudaStream_t, const int*, const int*);
 SIB_IB_INST(float)
 SIB_IB_INST(double)
 

@@ -136,6 +136,6 @@ extern "C" int sib_spread_noalloc(int N, int M, const double* X, const double* F
     }
     k.inv_h2 = (double)N * N;
     // one block per tile; blocks past the active-tile count return at once
-    launch_spread<double>(k, Fc, f, tiles, nTiles, ntiles, tx, ty, ntx, false, s);
+    launch_spread<double>(k, Fc, f, tiles, nTiles, ntiles, tx, ty, ntx, SPREAD_BY_TILE, s);
     return cudaGetLastError() == cudaSuccess ? SIB_OK : SIB_ERR_CUDA;
 }

@@ -405,9 +405,10 @@ template <typename T> void launch_adj_kappa(const int* eid, const double* kappa,
 template <typename T> void launch_interp(const IBK<T>& k, const T* u, T* U, cudaStream_t s);
 template <typename T> void launch_spring(const int* start, const int* nbr, const T* kap, int M, const T* U, T* F,
                                          cudaStream_t s);
+enum SpreadForm { SPREAD_TILES, SPREAD_CROWDED, SPREAD_BY_TILE };   // kernels_ib.cu; by tile: chosen on the device
 // rowSlots != nullptr: only the tiles of that slot list (count *nRow, at most maxTiles) are written
 template <typename T> void launch_spread(const IBK<T>& k, const T* F, T* f, const int* tiles, const int* nTiles,
-                                         int maxTiles, int tx, int ty, int ntx, bool crowded, cudaStream_t s,
+                                         int maxTiles, int tx, int ty, int ntx, SpreadForm form, cudaStream_t s,
                                          const int* rowSlots = nullptr, const int* nRow = nullptr);
 // Structures whose M markers take the form with a warp per face, by the largest number in one cell: the other waits for
 // one thread to walk its W bins (about 1.8 us per marker of the largest), this one reads every marker for each of its W^2

@@ -151,7 +151,7 @@ struct sib_ctx {
     uint64_t* keys = nullptr;
     int* binSums = nullptr;      // scratch of the marker binning
     int* binMost = nullptr;      // most markers of one fine bin
-    bool crowded = false;        // the spreading's form on the finest level
+    SpreadForm spreadForm = SPREAD_TILES;   // of the finest level
     int* sorted[2] = {nullptr, nullptr};
     uint32_t* mkey[2] = {nullptr, nullptr};
     int* adjStart = nullptr;
@@ -335,7 +335,7 @@ void spread_apply(sib_ctx* c, const Level& lv, const IBK<T>& k, const T* F, T* f
         return;
     }
     KL(c, launch_spread<T>(k, F, f, lv.tiles, lv.nTiles, lv.hnRowTiles, lv.tx, lv.ty, lv.ntx,
-                           c->crowded && &lv == &c->L[c->lmax], s, lv.rowSlots, lv.nRowTiles));
+                           &lv == &c->L[c->lmax] ? c->spreadForm : SPREAD_TILES, s, lv.rowSlots, lv.nRowTiles));
 }
 
 // f = [S K J]^l u (velocity part of x), written into the level's fib (only IB-active tiles)
@@ -1443,7 +1443,7 @@ void setup(sib_ctx* c, cudaStream_t s) {
             CK(cudaMemcpyAsync(&cnt[2 * l + 1], c->L[l].nRowTiles, sizeof(int), cudaMemcpyDeviceToHost, s));
         }
         CK(cudaStreamSynchronize(s));
-        c->crowded = spread_crowded(most, c->M);
+        c->spreadForm = spread_crowded(most, c->M) ? SPREAD_CROWDED : SPREAD_TILES;
         if (most > BIN_MAX) {   // a crowded cell: the order by the sorting network instead
             int Mpad = 1;
             while (Mpad < c->M) Mpad <<= 1;
@@ -1962,7 +1962,7 @@ void build_rhs(sib_ctx* c, const double* g, bool addSKX, cudaStream_t s) {
         double* F = (double*)c->F[0];
         KL(c, launch_spring<double>(c->adjStart, c->adjNbr, c->kap64, c->M, c->Xc, F, s));
         KL(c, launch_spread<double>(k, F, (double*)lv.p[0].fib, lv.tiles, lv.nTiles, lv.hnTiles, lv.tx, lv.ty, lv.ntx,
-                                    c->crowded, s));
+                                    c->spreadForm, s));
         KL(c, launch_axpby<double>(1.0, c->rhs, 1.0, (const double*)lv.p[0].fib, c->rhs, nv, s));
     }
     if (cavity(c)) {   // the walls are not unknowns; the moving lid enters through the ghost values
@@ -2746,7 +2746,7 @@ int sib_spread(sib_ctx* c, const double* F, double* f, void* stream) {
     KL(c, launch_deinterleave(F, c->M, (double*)c->F[0], s));
     CK(cudaMemsetAsync(lv.p[0].fib, 0, sizeof(double) * nv, s));
     KL(c, launch_spread<double>(k, (const double*)c->F[0], (double*)lv.p[0].fib, lv.tiles, lv.nTiles, lv.hnTiles,
-                                lv.tx, lv.ty, lv.ntx, c->crowded, s));
+                                lv.tx, lv.ty, lv.ntx, c->spreadForm, s));
     CK(cudaMemcpyAsync(f, lv.p[0].fib, sizeof(double) * nv, cudaMemcpyDeviceToDevice, s));
     kcheck(c);
     return SIB_OK;

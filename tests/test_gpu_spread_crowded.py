@@ -73,3 +73,25 @@ def test_time_of_a_crowded_cell():
         times.append(best)
         S.close()
     assert times[1] < 40 * times[0], times
+
+
+# the call without allocations, whose tiles choose their form on the device: crowded tiles beside ordinary ones, the
+# largest cell on both sides of the line, a grid below a tile
+@pytest.mark.parametrize("N,per", [(64, 24), (64, 25), (64, 2000), (32, 100), (256, 40), (16, 100)])
+def test_crowded_cells_without_allocations(N, per):
+    import ctypes
+
+    rng = np.random.default_rng(2000 * N + per)
+    X = np.concatenate([(np.array([1, N // 2]) + 0.55 + 0.4 * rng.uniform(0.0, 1.0, (per, 2))) / N,
+                        rng.uniform(0.0, 1.0, (500, 2))])
+    M = len(X)
+    F = rng.standard_normal((M, 2))
+    Xd, Fd, f = cu(X), cu(F), torch.full((2 * N * N,), 7.0, dtype=torch.float64, device="cuda")
+    p = lambda t: ctypes.c_void_p(t.data_ptr())  # noqa: E731
+    rc = sib.load().sib_spread_noalloc(N, M, p(Xd), p(Fd), p(f),
+                                       ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == sib.SIB_OK
+    ref = ib.spread_force(N, X, F)
+    mag = np.concatenate([abs(ib.spread_matrix(N, X, c)) @ np.abs(F[:, c]) for c in (0, 1)])
+    tol = (2 * M + 8) * EPS * mag + 64 * EPS * N * N * np.abs(F).max()
+    assert (np.abs(f.cpu().numpy() - ref) <= tol).all()
