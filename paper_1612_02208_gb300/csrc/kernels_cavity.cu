@@ -122,8 +122,8 @@ __device__ __forceinline__ void cavity_patch(const GridK<T>& g, int i, int j, T 
 // One additive sweep, xo = x + omega (1/2 (two cells' corrections) on interior faces, the cell's on p), 0 on wall
 // faces; ZERO: from x = 0, where the residual is b.  A tile forms the residuals of its cells and of a ring around
 // them (0 on wall faces and outside), then its patches and those of the column to the west and the row to the south,
-// whose d1 and d3 reach into it.  As three launches with the residual and the corrections in between in global
-// memory, the 272 sweeps of a 128^2 solve waited three times for a launch each: solve 4.04 -> 3.45 ms.
+// whose d1 and d3 reach into it.  As three launches (below) with the residual and the corrections in between in
+// global memory, the 272 sweeps of a 128^2 solve in FP32 waited three times for a launch each: solve 4.04 -> 3.45 ms.
 template <typename T, bool ZERO>
 __global__ void __launch_bounds__(TX * TY) k_cavity_vanka(GridK<T> g, T omega, const T* __restrict__ x,
                                                           const T* __restrict__ b, T* __restrict__ xo) {
@@ -173,6 +173,35 @@ __global__ void __launch_bounds__(TX * TY) k_cavity_vanka(GridK<T> g, T omega, c
     xo[c] = i >= 1 ? (ZERO ? du : x[c] + du) : T(0);
     xo[n + c] = j >= 1 ? (ZERO ? dv : x[n + c] + dv) : T(0);
     xo[2 * n + c] = ZERO ? dq : x[2 * n + c] + dq;
+}
+
+// The same sweep in three launches, residual, patches and update, with the corrections d = (d0, d1, d2, d3, dp) of
+// every cell in memory (5 n values).  r: the residual, or b where x = 0 (its wall-face entries are not read).
+template <typename T>
+__global__ void k_cavity_patches(GridK<T> g, const T* __restrict__ r, T* __restrict__ d) {
+    pdl_entry();
+    const int N = g.N, n = N * N;
+    const int i = blockIdx.x * g.tx + threadIdx.x, j = blockIdx.y * g.ty + threadIdx.y, c = j * N + i;
+    const T r0 = i == 0 ? T(0) : r[c], r1 = i == N - 1 ? T(0) : r[c + 1];
+    const T r2 = j == 0 ? T(0) : r[n + c], r3 = j == N - 1 ? T(0) : r[n + c + N];
+    T d0, d1, d2, d3, dp;
+    cavity_patch(g, i, j, r0, r1, r2, r3, r[2 * n + c], d0, d1, d2, d3, dp);
+    d[c] = d0;
+    d[n + c] = d1;
+    d[2 * n + c] = d2;
+    d[3 * n + c] = d3;
+    d[4 * n + c] = dp;
+}
+template <typename T, bool ZERO>
+__global__ void k_cavity_update(GridK<T> g, T omega, const T* __restrict__ d, const T* __restrict__ x,
+                                T* __restrict__ xo) {
+    pdl_entry();
+    const int N = g.N, n = N * N;
+    const int i = blockIdx.x * g.tx + threadIdx.x, j = blockIdx.y * g.ty + threadIdx.y, c = j * N + i;
+    const T hw = T(0.5) * omega;
+    xo[c] = i >= 1 ? (ZERO ? T(0) : x[c]) + hw * (d[c] + d[n + c - 1]) : T(0);
+    xo[n + c] = j >= 1 ? (ZERO ? T(0) : x[n + c]) + hw * (d[2 * n + c] + d[3 * n + c - N]) : T(0);
+    xo[2 * n + c] = (ZERO ? T(0) : x[2 * n + c]) + omega * d[4 * n + c];
 }
 
 // Restriction for the cavity (Sec. 3.2 with walls): the periodic R_u = P_u^T / 4 and the pressure
@@ -374,18 +403,29 @@ void launch_cavity_apply(const GridK<T>& g, const T* x, T* y, cudaStream_t s) {
     launch_pdl(k_cavity_apply<T>, dim3(g.N / g.tx, g.N / g.ty), dim3(g.tx, g.ty), 0, s, g, x, y);
 }
 template <typename T>
-void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* xo, T omega, cudaStream_t s) {
+int launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* r, T* d, T* xo, T omega, cudaStream_t s) {
     const dim3 grd(g.N / g.tx, g.N / g.ty), blk(g.tx, g.ty);
+    if (!d) {
+        if (x)
+            launch_pdl(k_cavity_vanka<T, false>, grd, blk, 0, s, g, omega, x, b, xo);
+        else
+            launch_pdl(k_cavity_vanka<T, true>, grd, blk, 0, s, g, omega, x, b, xo);
+        return 1;
+    }
+    if (x) launch_pdl(k_cavity_residual<T>, grd, blk, 0, s, g, x, b, r);
+    launch_pdl(k_cavity_patches<T>, grd, blk, 0, s, g, x ? (const T*)r : b, d);
     if (x)
-        launch_pdl(k_cavity_vanka<T, false>, grd, blk, 0, s, g, omega, x, b, xo);
+        launch_pdl(k_cavity_update<T, false>, grd, blk, 0, s, g, omega, (const T*)d, x, xo);
     else
-        launch_pdl(k_cavity_vanka<T, true>, grd, blk, 0, s, g, omega, x, b, xo);
+        launch_pdl(k_cavity_update<T, true>, grd, blk, 0, s, g, omega, (const T*)d, x, xo);
+    return x ? 3 : 2;
 }
 template void launch_cavity_apply<float>(const GridK<float>&, const float*, float*, cudaStream_t);
 template void launch_cavity_apply<double>(const GridK<double>&, const double*, double*, cudaStream_t);
-template void launch_cavity_vanka<float>(const GridK<float>&, const float*, const float*, float*, float, cudaStream_t);
-template void launch_cavity_vanka<double>(const GridK<double>&, const double*, const double*, double*, double,
-                                          cudaStream_t);
+template int launch_cavity_vanka<float>(const GridK<float>&, const float*, const float*, float*, float*, float*, float,
+                                        cudaStream_t);
+template int launch_cavity_vanka<double>(const GridK<double>&, const double*, const double*, double*, double*, double*,
+                                         double, cudaStream_t);
 template void launch_cavity_residual<float>(const GridK<float>&, const float*, const float*, float*, cudaStream_t);
 template void launch_cavity_residual<double>(const GridK<double>&, const double*, const double*, double*,
                                              cudaStream_t);

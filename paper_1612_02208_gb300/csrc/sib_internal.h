@@ -281,9 +281,17 @@ template <typename T> void launch_residual(const GridK<T>& g, const T* x, const 
 // y = L x of the lid-driven cavity on the periodic layout (kernels_cavity.cu); wall-face entries 0
 template <typename T> void launch_cavity_apply(const GridK<T>& g, const T* x, T* y, cudaStream_t s);
 // one additive Vanka sweep of the cavity, xo = x + omega (weighted corrections of b - L x; x == nullptr: from 0);
-// g.fib must hold [S K J] x (kernels_cavity.cu)
+// g.fib must hold [S K J] x (kernels_cavity.cu).  d == nullptr: one launch; else three, with r (3 n) and d (5 n) in
+// between.  Returns the number of launches.
 template <typename T>
-void launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* xo, T omega, cudaStream_t s);
+int launch_cavity_vanka(const GridK<T>& g, const T* x, const T* b, T* r, T* d, T* xo, T omega, cudaStream_t s);
+// Which form a level takes.  The one launch forms a tile's ring of residuals and patches anew: FP64 levels are bound by
+// that work, large FP32 ones by its loads, smaller ones by the launches.  us a sweep in one launch / in three, annulus and
+// no structure: FP32 128^2 14.2 / 15.0 and 4.2 / 6.0, 256^2 21.0 / 19.0 and 4.5 / 6.1, 512^2 40.4 / 33.8 and 8.4 / 8.3,
+// 2048^2 191 / 168 and 115 / 98; FP64 32^2 24.3 / 21.8 and 13.1 / 11.1, 128^2 25.9 / 23.6 and 12.9 / 10.9, 2048^2 1,190 / 983
+// and 970 / 763.
+template <typename T>
+constexpr bool cavity_in_three(int N, bool ib) { return sizeof(T) == 8 || N >= (ib ? 256 : 512); }
 // r = b - L x of the cavity (0 on the wall faces); x <- 0 on the wall faces
 template <typename T> void launch_cavity_residual(const GridK<T>& g, const T* x, const T* b, T* r, cudaStream_t s);
 template <typename T> void launch_cavity_zero_walls(T* x, int N, cudaStream_t s);

@@ -48,6 +48,7 @@ struct LevelBuf {
     void* tp[6] = {};
     void* dinv = nullptr;   // 3 n: SC diagonals
     void* pf = nullptr;     // 7 n: Vanka patch factors
+    void* cav = nullptr;    // 5 n: cavity Vanka patch corrections, where its sweep is three launches
     // Krylov-wrapped smoothing: WRAP_MAXK + 1 Arnoldi vectors, WRAP_MAXK preconditioned ones, a work
     // vector (3 n each) and the step's small FP64 arrays
     void* wV = nullptr;
@@ -609,12 +610,23 @@ void ras_apply(sib_ctx* c, int l, const T* r, const T* x, T* xo, double omega, c
                                        (const T*)lv.rasInv[pi], (T)omega, r, x, xo, s, tc, c->herr);
 }
 
+// the patch corrections of the cavity's sweep, where the level's form has them in memory
+template <typename T>
+void cavity_corrections(sib_ctx* c, int l) {
+    Level& lv = c->L[l];
+    LevelBuf& lb = lv.p[Prec<T>::id];
+    if (cavity_in_three<T>(lv.N, c->haveIB) && !lb.cav) lb.cav = dalloc(c, sizeof(T) * 5 * (size_t)lv.N * lv.N);
+}
+
 // one smoothing sweep xo <- smooth(x, b)
 template <typename T>
 void sweep(sib_ctx* c, int l, const T* x, const T* b, T* xo, cudaStream_t s) {
     if (cavity(c)) {   // the cavity's Vanka sweep: patch solves with the wall rules
+        LevelBuf& lb = c->L[l].p[Prec<T>::id];
         if (x) ib_apply<T>(c, l, x, s);
-        KL(c, launch_cavity_vanka<T>(gridk<T>(c, l), x, b, xo, (T)c->opts.omega, s));
+        c->launches += launch_cavity_vanka<T>(gridk<T>(c, l), x, b, (T*)lb.r,
+                                              cavity_in_three<T>(c->L[l].N, c->haveIB) ? (T*)lb.cav : nullptr, xo,
+                                              (T)c->opts.omega, s);
     } else if (c->opts.smoother == SIB_SMOOTHER_SC) {
         sc_sweep<T>(c, l, x, b, xo, s);
     } else if (c->opts.smoother == SIB_SMOOTHER_RAS) {   // r = b - L x, then the box corrections
@@ -1594,6 +1606,11 @@ void setup(sib_ctx* c, cudaStream_t s) {
         KL(c, (launch_convert<double, float>((const double*)lv.p[0].pf, (float*)lv.p[1].pf, n7, s)));
     }
     if (c->opts.smoother == SIB_SMOOTHER_RAS && c->lmax > 0) ras_setup_all(c, s);
+    if (cavity(c))   // outside any graph capture
+        for (int l = 1; l <= c->lmax; ++l) {
+            cavity_corrections<double>(c, l);
+            cavity_corrections<float>(c, l);
+        }
     if (c->opts.smoother == SIB_SMOOTHER_SC) {
         alloc_sc_bufs(c);
         for (int l = 1; l <= c->lmax; ++l) {
@@ -2174,12 +2191,14 @@ void cavity_smooth_impl(sib_ctx* c, int l, T* x, const T* b, int sweeps, cudaStr
     LevelBuf& lb = lv.p[Prec<T>::id];
     const size_t n = (size_t)lv.N * lv.N;
     const double om = c->opts.smoother == SIB_SMOOTHER_VANKA ? c->opts.omega : 0.8;
+    cavity_corrections<T>(c, l);
     GridK<T> g = gridk<T>(c, l);
     T* cur = x;
     T* nxt = (T*)lb.xt;
     for (int k = 0; k < sweeps; ++k) {
         ib_apply<T>(c, l, cur, s);
-        KL(c, launch_cavity_vanka<T>(g, cur, b, nxt, (T)om, s));
+        c->launches += launch_cavity_vanka<T>(g, cur, b, (T*)lb.r,
+                                              cavity_in_three<T>(lv.N, c->haveIB) ? (T*)lb.cav : nullptr, nxt, (T)om, s);
         std::swap(cur, nxt);
     }
     if (cur != x) CK(cudaMemcpyAsync(x, cur, sizeof(T) * 3 * n, cudaMemcpyDeviceToDevice, s));
