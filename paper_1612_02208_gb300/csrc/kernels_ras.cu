@@ -902,6 +902,37 @@ __global__ void __launch_bounds__(RAS_SP_T) k_ras_apply_split(RasGeo G, RasSplit
     }
 }
 
+// The IB boxes of few dofs (1 x 1 boxes with overlap 0 or 1): a warp each, whose lanes are four rows, three of them
+// owned, by eight parts of the dofs.  A block of k_ras_apply_split has two products a thread to do there and is all
+// set-up.  Annulus, overlap 0, a sweep of the finest level: FP64 128^2 48.7 -> 36.2 us, 512^2 331 -> 237; FP32 512^2
+// 161 -> 104.  (2 x 2 boxes with overlap 0, a warp each: 128^2 FP32 16.4 -> 18.6, so those stay there.)
+constexpr int RAS_FEW = 33;
+template <typename T>
+__global__ void __launch_bounds__(256) k_ras_apply_ib_few(RasGeo G, const int* __restrict__ list, int nIB,
+                                                         const T* __restrict__ inv, T omega, const T* __restrict__ r,
+                                                         const T* x, T* xo) {
+    constexpr int R = 4;
+    const int lane = threadIdx.x & 31, s = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int row = lane % R, part = lane / R;
+    const int k = s < nIB ? list[s] : 0;   // set-up data
+    pdl_entry();
+    if (s >= nIB) return;
+    const int N = G.N, n = N * N, m = N - 1, I = k % G.nbs, J = k / G.nbs;
+    const T* M = inv + (size_t)(s + 1) * G.ne * G.nown;
+    T acc = T(0);
+#pragma unroll 4
+    for (int q = part; q < G.ne; q += 32 / R) {
+        int comp, ii, jj;
+        ras_dof(G, q, comp, ii, jj);
+        const T v = r[(size_t)comp * n + (size_t)((J - G.o + jj) & m) * N + ((I - G.o + ii) & m)];
+        if (row < G.nown) acc += M[(size_t)q * G.nown + row] * v;
+    }
+    for (int o = R; o < 32; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (part > 0 || row >= G.nown) return;
+    const size_t d = (size_t)row * n + (size_t)J * N + I;
+    xo[d] = (x ? x[d] : T(0)) + omega * acc;
+}
+
 // ---- tensor-core correction of the IB-free boxes on FP32 levels ---------------------------------
 // The boxes without IB terms share one inverse, so their correction is the product
 //   C^T (boxes x owned rows) = R^T (boxes x ne) Inv^T (ne x owned rows).
@@ -2206,7 +2237,7 @@ template <typename T>
 int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list, int nIB, const T* inv, T omega,
                      const T* r, const T* x, T* xo, cudaStream_t s, const float* tcPack, int* err) {
     const RasGeo G = ras_geo(N, b, o);
-    auto split = [&](int ngroups) {
+    auto split = [&](int ngroups, int nIB) {
         const RasSplit p = ras_split(G, ngroups == 0);
         const int nb = ngroups > 0 ? RAS_SP_NB : 1;
         const size_t smem = sizeof(T) * nb * ((size_t)G.ne + (size_t)p.ks * p.rc);
@@ -2215,18 +2246,41 @@ int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list,
         launch_pdl(kern, dim3((nIB + ngroups) * p.chunks), dim3(p.threads), smem, s, G, p, list, nIB,
                    slotOfBox, inv, omega, r, x, xo);
     };
-    // Which form (us per correction, thin circle, the other forms with one block per IB box / all boxes split):
-    //   FP32  4x4 o1: 64^2 14.5 / 4.8, 128^2 13.8 / 8.0, 256^2 14.8 / 17.1, 512^2 19.6 / 53.9
-    //         2x2 o2: 64^2 13.2 / 4.7, 128^2 14.9 / 8.9, 256^2 16.8 / 21.4, 512^2 41.2 / 67.2
-    //         8x8 o2: 64^2 77 / 7.8, 128^2 87 / 11.6, 256^2 79 / 27.8, 512^2 154 / 79, 1024^2 165 / 272
-    //   FP64  4x4 o1: 64^2 45 / 12, 128^2 45 / 24, 256^2 73 / 72, 512^2 262 / 252, 1024^2 858 / 987
-    //         2x2 o2: 256^2 258 / 88, 512^2 879 / 310;  8x8 o2: 256^2 825 / 219, 1024^2 2998 / 2692
-    // FP32 levels above 128^2 fill the GPU with tiles of boxes; FP64 is bound by the FP64 pipe in either form,
-    // and the persistent kernel's staged inverse pays only where its 64 lanes of owned rows are filled.
-    const bool all = sizeof(T) == 4 ? N <= 128 : !(G.e <= RAS_EMAX_SMEM && G.nown >= 32 && N > 256);
+    // Which form.  us a sweep of the finest level (IB pass, residual, correction), the other forms / all boxes split:
+    //               no structure                                     paper's annulus
+    //   FP32  8x8 o2: 128^2 45.8 / 11.7, 256^2 35.7 / 23.1, 512^2 37.3 / 66.7;  65.6 / 27.4, 77.0 / 54.6, 148 / 148
+    //         4x4 o1: 128^2 13.7 / 8.1, 256^2 14.2 / 16.9, 512^2 16.0 / 50.0;   28.9 / 22.1, 36.9 / 41.6, 88.3 / 116
+    //         2x2 o2: 128^2 13.7 / 8.8, 256^2 15.0 / 19.7;                      29.1 / 24.0, 38.5 / 46.8
+    //         2x2 o0: 64^2 6.6 / 6.3, 128^2 7.0 / 7.6;                          19.8 / 15.5, 19.7 / 21.5
+    //         1x1 o0: 32^2 6.3 / 6.4, 64^2 6.7 / 7.4, 128^2 9.7 / 17.5;         15.7 / 14.1, 18.0 / 21.4, 22.9 / 38.8
+    //         1x1 o2: 64^2 12.3 / 8.3, 128^2 12.9 / 18.8;                       27.4 / 24.7, 34.3 / 45.3
+    //         1x1 o7: 128^2 44.4 / 28.1;                                        89.0 / 77.5
+    //   FP64  4x4 o1: 256^2 107 / 78, 512^2 296 / 273, 1024^2 886 / 1046;       256^2 139 / 119, 512^2 400 / 402
+    //         2x2 o1: 128^2 49.3 / 20.9, 1024^2 1618 / 900;                     71.0 / 47.0
+    //         2x2 o0: 64^2 12.3 / 9.1, 128^2 17.3 / 18.1, 1024^2 529 / 643;     28.7 / 25.3, 34.0 / 37.7
+    //         1x1 o0: 32^2 8.7 / 10.7, 128^2 18.6 / 54.4, 512^2 185 / 738;      21.5 / 26.9, 36.2 / 113, 237 / 1312
+    //         1x1 o1: 64^2 24.1 / 19.3, 128^2 75.4 / 56.8;                      40.3 / 35.9, 94.5 / 66.9
+    // FP32 levels above 128^2 fill the GPU with tiles of boxes (8x8 boxes do so from 512^2 on only).  FP64 is bound by the
+    // FP64 pipe in either form, and the persistent kernel's staged inverse pays only where its 64 lanes of owned rows
+    // are filled.  A split block serves eight boxes, of few dofs too: many such boxes are cheaper in the other forms.
+    const int nboxes = G.nbs * G.nbs;
+    bool all;
+    if (sizeof(T) == 4)
+        all = N <= 128 && !(nboxes >= 4096 && G.ne <= (tcPack ? 16 : RAS_FEW)) &&
+              !(nboxes >= 16384 && G.ne <= (tcPack ? 200 : 100));
+    else
+        all = !(nboxes >= (G.ne <= 5 ? 1024 : 4096) && G.ne <= 16) &&
+              !(G.e <= RAS_EMAX_SMEM && G.nown >= 32 && N > 256);
+    // one-cell IB boxes in a launch of their own: 1x1 o1 annulus, in it / apart, FP32 32^2 16.7 / 17.6, 64^2 22.5 / 21.2; FP64
+    // 32^2 31.6 / 25.9, 128^2 125 / 66.9, 512^2 1395 / 762
+    const bool few = G.b == 1 && G.ne <= RAS_FEW && nIB > 0 && (!all || nboxes >= (sizeof(T) == 4 ? 4096 : 1024));
+    auto apply_few = [&]() {
+        launch_pdl(k_ras_apply_ib_few<T>, dim3((nIB + 7) / 8), dim3(256), 0, s, G, list, nIB, inv, omega, r, x, xo);
+        return 2;
+    };
     if (all) {
-        split((G.nbs * G.nbs + RAS_SP_NB - 1) / RAS_SP_NB);
-        return 1;
+        split((nboxes + RAS_SP_NB - 1) / RAS_SP_NB, few ? 0 : nIB);
+        return few ? apply_few() : 1;
     }
     bool done = false;
     if constexpr (sizeof(T) == 4) {
@@ -2262,7 +2316,8 @@ int launch_ras_apply(int N, int b, int o, const int* slotOfBox, const int* list,
         launch_pdl(k_ras_apply<T>, dim3(blocks), dim3(32 * RAS_WARPS), smem, s, G, slotOfBox, inv, omega, r, x, xo);
     }
     if (nIB == 0) return 1;
-    split(0);   // the IB boxes
+    if (few) return apply_few();
+    split(0, nIB);   // the IB boxes
     return 2;
 }
 template int launch_ras_apply<float>(int, int, int, const int*, const int*, int, const float*, float, const float*,
