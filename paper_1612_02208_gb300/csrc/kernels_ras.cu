@@ -2210,7 +2210,11 @@ void launch_ras_wb_apply64(int N, int b, int o, const RasIB& ib, double a0, doub
                            cudaStream_t s) {
     if (nIB <= 0) return;
     const RasGeo G = ras_geo(N, b, o);
-    const size_t smem = sizeof(double) * (4 * (size_t)G.ne + (size_t)mmax);
+    // With fewer boxes than SMs each takes an SM to itself, by reserving more than half of its shared memory: launched
+    // beside the end of the shared correction, up to three crowd the SMs that it leaves first, and how many changes from
+    // process to process (128^2 circle, a sweep: 3.4 to 6.4 ms, 2.81 so; annulus 7.3 to 8.6, 4.3; 256^2 circle 8.0, 3.9).
+    const size_t need = sizeof(double) * (4 * (size_t)G.ne + (size_t)mmax);
+    const size_t smem = nIB <= 152 ? std::max<size_t>(need, 116 * 1024) : need;
     allow_smem(k_ras_wb_apply, smem);
     launch_pdl(k_ras_wb_apply, dim3(nIB), dim3(256), smem, s, G, ib, a0, c, inv_h, dt, list, offT, Tl, offW, W,
                inv0, omega, r, xo);
