@@ -18,7 +18,7 @@ Output: one JSON line (rank 0).  `value` is device time per step (ms) over the w
 runs its own replica); `e2e` is the same step through the autograd binding with g, kappa and X copied
 from pinned host memory and the loss and gradients copied back.  The other workloads of the build
 (32^2 to 512^2, the paper's own structures, the lid-driven cavity, the 4096^2 V-cycle roofline) are
-reported beside it, each result with its error against the FP64 oracle.
+reported on stderr as one JSON object, each result with its error against the FP64 oracle.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl native|reference] [--cpu-breadth]
 """
@@ -760,13 +760,17 @@ def run_native(args):
                        "max_it": 100, "parallelism": f"replicas x{world}",
                        "l2": "flushed between timed steps (inputs exceed L2: FGMRES basis 2.5 GB)",
                        "timing": "CUDA events per step on the launching stream"},
-            "headline": {"first_timed_step": first, "phase_ms_median": phase_ms,
-                         "oracle_checks": checks.get("headline") if checks else None},
-            "variants": variants, "legs": legs,
-            "oracle_checks": checks.get("legs") if checks else None,
-            "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
-            "gpu_launches": int(launches), "clocks": clk, "wall_s": round(wall, 3),
+            "roofline": {k: roofline[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
+                                                  "launch_ms", "peak_source") if k in roofline},
+            "cpu_baseline": {k: v for k, v in cpu.items() if not isinstance(v, (dict, list))} if cpu else None,
+            "e2e": e2e, "gpu_launches": int(launches), "clocks": clk, "wall_s": round(wall, 3),
         }
+        # the other workloads, the variants and the oracle's checks, apart from the result line
+        details = {"headline": {"first_timed_step": first, "phase_ms_median": phase_ms,
+                                "oracle_checks": checks.get("headline") if checks else None},
+                   "variants": variants, "legs": legs, "oracle_checks": checks.get("legs") if checks else None,
+                   "roofline": roofline, "cpu_baseline": cpu}
+        print(json.dumps({"details": details}), file=sys.stderr, flush=True)
         print(json.dumps(line), flush=True)
 
 
