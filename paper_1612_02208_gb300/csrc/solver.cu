@@ -1185,7 +1185,7 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     double* Aug = (double*)dalloc(c, sizeof(double) * (size_t)n * 2 * n);
     void* work = dalloc(c, gauss_jordan_work_bytes(n));
     int* piv = (int*)dalloc(c, sizeof(int) * (size_t)n);
-    tmp.insert(tmp.end(), {Aug, work, piv});
+    std::vector<void*> own = {Aug, work, piv};   // the level's temporaries
     const double h = lv.h, a0 = c->rho / c->dt + 4.0 * c->mu / (h * h), cc = c->mu / (h * h);
     KL(c, launch_ras_huge_assemble(lv.N, b, o, a0, cc, 1.0 / h, Aug, s));
     KL(c, launch_gauss_jordan(Aug, n, ginfo, piv, work, s));
@@ -1217,10 +1217,13 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     lv.wbOffW = nullptr;
     lv.wbW = nullptr;
     lv.wbMmax = 0;
-    if (nIB == 0) return;
+    if (nIB == 0) {
+        tmp.insert(tmp.end(), own.begin(), own.end());
+        return;
+    }
     const RasIB ib{lv.slotOf, (const double*)lv.win[0], lv.tx, lv.ty, lv.ntx};
     int* dcnt = (int*)dalloc(c, sizeof(int) * (size_t)nIB);
-    tmp.push_back(dcnt);
+    own.push_back(dcnt);
     KL(c, launch_ras_wb_count(lv.N, b, o, ib, lv.rasList, nIB, dcnt, s));
     std::vector<int> cnt(nIB), offT(nIB + 1, 0);
     std::vector<long long> offW(nIB, 0);
@@ -1238,11 +1241,8 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
     lv.wbT = (int*)dalloc(c, sizeof(int) * (size_t)std::max(1, offT[nIB]));
     lv.wbW = (double*)dalloc(c, sizeof(double) * (size_t)std::max(1LL, wTot));
     lv.wbScratch = (double*)dalloc(c, sizeof(double) * (2 * ras_wb_row(b, o) + (size_t)lv.wbMmax) * nIB);
-    lv.hugeSplit = dalloc(c, 2 * sizeof(float) * (size_t)ne * ras_wb_row(b, o));
-    lv.wbWs = dalloc(c, 2 * sizeof(float) * (size_t)std::max(1LL, wTot));
-    lv.wbPos = (int*)dalloc(c, sizeof(int) * (size_t)ne * nIB);
     double* wwork = (double*)dalloc(c, sizeof(double) * (size_t)std::max(1LL, 2 * wTot));
-    tmp.push_back(wwork);
+    own.push_back(wwork);
     CK(cudaMemcpyAsync(lv.wbOffT, offT.data(), sizeof(int) * (size_t)(nIB + 1), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(lv.wbOffW, offW.data(), sizeof(long long) * (size_t)nIB, cudaMemcpyHostToDevice, s));
     KL(c, launch_ras_wb_fill(lv.N, b, o, ib, lv.rasList, nIB, lv.wbOffT, lv.wbT, s));
@@ -1258,16 +1258,22 @@ void ras_huge_setup(sib_ctx* c, int l, int nIB, std::vector<void*>& tmp, int* gi
         double* augB = (double*)dalloc(c, sizeof(double) * (size_t)m16 * 2 * m16);
         int* pivB = (int*)dalloc(c, sizeof(int) * (size_t)m16);
         void* workB = dalloc(c, gauss_jordan_work_bytes(m16));
-        tmp.insert(tmp.end(), {augB, pivB, workB});
+        own.insert(own.end(), {augB, pivB, workB});
         for (int k = 0; k < nIB; ++k)
             if (cnt[k] > RAS_WB_ONE_MAX) {
                 launch_ras_wb_big(wwork + 2 * offW[k], cnt[k], augB, pivB, workB, c->rasInfo, lv.wbW + offW[k], s);
                 c->launches += 2 + 3 * ((cnt[k] + 15) / 16);
             }
     }
+    // the temporaries, twice the size of W, go before the pairs of floats come: a set-up then holds no more at a time than
+    // it would without the pairs
+    CK(cudaStreamSynchronize(s));   // (the host vectors above are the copies' sources)
+    for (void* p : own) dfree(c, p);
+    lv.hugeSplit = dalloc(c, 2 * sizeof(float) * (size_t)ne * ras_wb_row(b, o));
+    lv.wbWs = dalloc(c, 2 * sizeof(float) * (size_t)std::max(1LL, wTot));
+    lv.wbPos = (int*)dalloc(c, sizeof(int) * (size_t)ne * nIB);
     launch_ras_wb_split(b, o, (const double*)lv.hugeInv[0], lv.hugeSplit, lv.wbW, (size_t)wTot, lv.wbWs, nIB, lv.wbOffT,
                         lv.wbT, lv.wbPos, s);
-    CK(cudaStreamSynchronize(s));   // the host vectors above are the copies' sources
     c->launches += 6;
 }
 
