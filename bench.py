@@ -762,7 +762,7 @@ def run_native(args):
                        "timing": "CUDA events per step on the launching stream"},
             "roofline": {k: roofline[k] for k in ("bound", "kernel", "achieved", "peak", "unit", "frac", "traffic",
                                                   "launch_ms", "peak_source") if k in roofline},
-            "cpu_baseline": {k: v for k, v in cpu.items() if not isinstance(v, (dict, list))} if cpu else None,
+            "cpu_baseline": {k: cpu[k] for k in ("value", "unit", "cores", "kind")} if cpu else None,
             "e2e": e2e, "gpu_launches": int(launches), "clocks": clk, "wall_s": round(wall, 3),
         }
         # the other workloads, the variants and the oracle's checks, apart from the result line

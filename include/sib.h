@@ -75,7 +75,8 @@ typedef struct {
     int    max_it;        /* iteration cap (100, the paper's cap)                                    */
     int    restart;       /* FGMRES restart length (100)                                             */
     int    add_SKXn;      /* 1: right-hand side g + S K X^n (paper form), 0: g only (1)              */
-    int    use_graphs;    /* 1: replay the V-cycle as a CUDA graph (1)                               */
+    int    use_graphs;    /* 1: replay the V-cycle as a CUDA graph (1); sib_vcycle from 2048 x 2048 up
+                             launches its kernels one by one either way, on the caller's arrays     */
     int    fuse_small;    /* 1: the smallest levels of the V-cycle run as one launch where they fit in shared
                              memory: FP32 Vanka up to 32 x 32, else levels 1 (at most 16 x 16) and 0;
                              0: one kernel per step (1)                                               */

@@ -13,9 +13,9 @@
 // Boxes whose subdomain meets no IB window all have the same operator (the grid is uniform and
 // periodic): one shared inverse per level serves them.  Subdomains up to RAS_BE_EMAX cells wide are
 // inverted by block elimination in shared memory, wider ones (and those whose blocks are not positive
-// definite) by Gauss-Jordan with partial pivoting in a global workspace.  Subdomains up to RAS_EMAX_SMEM
-// cells wide are corrected by a persistent kernel, wider ones (the paper's 8 x 8 boxes with overlap 2
-// and up) by a batched product over tiles of boxes.
+// definite) by Gauss-Jordan with partial pivoting in a global workspace.  The correction spreads a box's owned rows over
+// blocks (k_ras_apply_split); levels of many boxes take a persistent kernel (narrow boxes), tiles of boxes (wide ones)
+// or the tensor cores (launch_ras_apply says which).
 #include <algorithm>
 #include <type_traits>
 
@@ -218,12 +218,9 @@ __global__ void k_box_slots(const int* __restrict__ list, const int* __restrict_
     if (s < *count) slotOfBox[list[s]] = s;
 }
 
-// ---- set-up with pivoting, and subdomains wider than RAS_EMAX_SMEM cells (e <= RAS_EMAX, ne <= 800) ----
-// The local operator takes up to 5 MB in FP64.  Each set-up block assembles its matrix in a global
-// workspace and eliminates there, with the pivot column and the scaled pivot row in shared memory.  For
-// the wide subdomains the shared-inverse correction becomes one batched product per level,
-// C (nown x boxes) = Inv (nown x ne) R (ne x boxes), over tiles of boxes; the IB boxes keep one block
-// each.
+// ---- set-up with pivoting (any subdomain up to RAS_EMAX cells, ne <= 800) ------------------------------
+// The local operator takes up to 5 MB in FP64.  Each set-up block assembles its matrix in a global workspace and
+// eliminates there, with the pivot column and the scaled pivot row in shared memory.
 
 // Row q of L_k for the subdomain with corner cell (i0, j0), added into `row` (zeroed by the caller).
 // Couplings go to dofs of the subdomain at local coordinates taken modulo N: on small grids a neighbour or
@@ -1768,8 +1765,6 @@ __global__ void k_ras_tc_pack_rows(RasGeo G, const double* __restrict__ inv0, in
 
 }  // namespace
 
-bool ras_big(int b, int o) { return b + 2 * o > RAS_EMAX_SMEM; }
-
 int ras_ne(int b, int o) { return ras_geo(16, b, o).ne; }
 
 void launch_ras_classify(int N, int b, int o, const RasIB& ib, int* list, int* count, cudaStream_t s) {
@@ -2005,13 +2000,15 @@ template void launch_ras_huge_apply<double>(int, int, int, const double*, double
 // were in FP64 (y on T and the owned rows, W y, Q_{own,T} z), bound by the FP64 pipe: 2 multiply-adds per SM and clock,
 // against 128 in FP32.  Here every value is a sum of two floats (Q and W split at set-up to 48 bits, r exact in one)
 // and every product and sum keeps its rounding error (two-product by FMA and Knuth's two-sum: Ogita, Rump and
-// Oishi's Dot2), twelve FP32 operations for one in FP64.  The rounding left is 2^-46 or so of the terms, and the
-// result is rounded to FP32 as before: one sweep's error against FP64 levels is the same to five digits from
-// gamma = 5 to 500 on 32^2 to 128^2, circle and annulus (2e-8 to 7e-8).
+// Oishi's Dot2), twelve FP32 operations for one in FP64.  The rounding left is 2^-46 or so of the terms (FP64: 2^-53), and
+// the result is rounded to FP32 as before: a sweep's error against FP64 levels, in ulp of the result, is the FP64 form's
+// to four digits, mean and largest, for residuals from 2^60 down to 2^-100 and gamma from 5 to 50,000 on 64^2 and 128^2,
+// circle and annulus.  Exponents are FP32's: products below 2^-125 or so lose their error terms (one to six of 49,000
+// results change at 2^-100).
 // A block holds the vectors of WB_BX boxes in shared memory, and a warp takes a row of Q for those of them that need
 // it, so that Q, 25 MB in all, is read from L2 once per group and not once per box; eight elements a lane at a time,
 // whose sums overlap.
-// 128^2 circle, 16 x 16 boxes with overlap 4, with the IB-free boxes listed (k_ras_huge_apply): solve 25.9 -> 11.1 ms.
+// 128^2 circle, 16 x 16 boxes with overlap 4, with the IB-free boxes listed (k_ras_huge_apply): solve 22.3 -> 10.9 ms.
 struct TwoFloat {
     float s, c;
 };

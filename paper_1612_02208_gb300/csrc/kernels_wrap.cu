@@ -352,8 +352,8 @@ __global__ void __launch_bounds__(WT) k_wreduce_lsq(const double* __restrict__ p
 // end with every block's sums in every block's shared memory and one cluster barrier; then Vnext = w / |w|
 // (Vnext != nullptr) and, on the stage's last step (lsq_k > 0), its least-squares solve into y.  cnt = 0: the norm
 // alone, of the stage's residual.  Bound by latency: seven launches of 2.5 us each did a step (three on levels
-// of up to 32^2, in one block).  Solves with wrapped Schur-complement sweeps, disk, FP32: 32^2 2.35 -> 2.25 ms,
-// 128^2 6.49 -> 6.17, 256^2 11.75 -> 11.33.  FP64 levels take it up to 32^2 (3.67 -> 3.35): above, eight SMs' FP64 pipes
+// of up to 32^2, in one block).  Solves with wrapped Schur-complement sweeps, disk, FP32: 32^2 2.35 -> 2.27 ms,
+// 128^2 6.49 -> 6.20, 256^2 11.75 -> 11.38.  FP64 levels take it up to 32^2 (3.67 -> 3.35): above, eight SMs' FP64 pipes
 // are slower than the launches (128^2: 10.6 against 11.0 ms with it).
 constexpr int WC = 8;
 template <typename T, int KC, int E>

@@ -153,13 +153,12 @@ struct RasIB {
     const double* win;       // FP64 windows of the level
     int tx, ty, ntx;         // tile geometry of the level
 };
-// Subdomains up to RAS_EMAX_SMEM cells wide are applied from shared memory; wider ones, up to RAS_EMAX
-// cells (ne <= 800), as a batched product.  Set-up: up to RAS_BE_EMAX cells wide (a packed velocity block
+// The persistent correction holds inverses of subdomains up to RAS_EMAX_SMEM cells wide in shared memory; those of
+// boxes below 16 cells are up to RAS_EMAX cells wide (ne <= 800).  Set-up: up to RAS_BE_EMAX cells wide (a packed velocity block
 // of 177 KB fits shared memory) by block elimination, else by pivoted elimination in a global workspace.
 constexpr int RAS_EMAX_SMEM = 6;
 constexpr int RAS_BE_EMAX = 14;
 constexpr int RAS_EMAX = 16;
-bool ras_big(int b, int o);
 int ras_ne(int b, int o);
 void launch_ras_classify(int N, int b, int o, const RasIB& ib, int* list, int* count, cudaStream_t s);
 void launch_box_slots(int nboxes, const int* list, const int* count, int* slotOfBox, cudaStream_t s);

@@ -1587,8 +1587,8 @@ void setup(sib_ctx* c, cudaStream_t s) {
         c->kappaDirty = false;
         c->fluidDirty = true;
     }
-    // coarsest pseudo-inverse (depends on rho, mu, dt and kappa).  The Gauss-Jordan inversion holds
-    // one 16-block cluster for about a millisecond; it runs on the auxiliary stream, beside the SC
+    // coarsest pseudo-inverse (depends on rho, mu, dt and kappa).  The Gauss-Jordan inversion is
+    // a chain of one-block panels (twelve at 8 x 8 cells, 16.5 us each) and their updates; it runs on the auxiliary stream, beside the SC
     // eigenvalue estimates below (which do not use it), and the main stream joins it at the end.
     {
         const int n = c->n0;
@@ -2032,7 +2032,10 @@ int solve_impl(sib_ctx* c, const double* g, double* w, sib_stats* st, cudaStream
 // A caller's V-cycle on large grids: the kernels launched one by one, the finest level's on the caller's own arrays.
 // The captured graph works on the level's, so b is copied in and z out: 121 of the 1,265 us of an FP32 V-cycle at
 // 4096^2 (1,140 so).  From 2048^2 on the finest level's kernels run longer than the host takes
-// to enqueue the rest; below, the graph's launches are worth more than the copies.  False: not for these arguments
+// to enqueue the rest; below, the graph's launches are worth more than the copies.  All at 2048^2, us before the form
+// (graph, copies and the kernels of then) / with it: Vanka FP32 551 / 436, FP64 3,331 / 3,093; SC, the most launches, FP32
+// 1,996 / 1,960, FP64 8,146 / 7,976; 4 x 4 boxes FP32 1,591 / 1,311, FP64 21,069 / 20,074; with other arrays at every call
+// the same.  False: not for these arguments
 // (arrays that overlap, that 16-byte and TMA loads cannot take, or a stream in capture).
 template <typename T>
 bool vcycle_direct(sib_ctx* c, const T* b, T* z, cudaStream_t s) {
@@ -2416,9 +2419,7 @@ int sib_set_stiffness(sib_ctx* c, const double* kappa, void* stream) {
     API_END(c)
 }
 
-// Widest box subdomain the options accept: up to RAS_EMAX_SMEM cells in shared memory, wider ones
-// (boxes of 8 cells with overlap 2, up to RAS_EMAX cells) through the global-workspace set-up and the
-// batched correction.
+// Widest box subdomain the options accept (boxes of 16 cells apart).
 constexpr int RAS_EMAX_ENABLED = RAS_EMAX;
 constexpr bool CAVITY_SOLVE_ENABLED = true;
 
