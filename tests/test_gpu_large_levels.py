@@ -115,3 +115,20 @@ def test_smallest_levels_are_one_launch():
         counts[key] = S.launch_count - before
         S.close()
     assert counts["cluster"] == 1 and min(counts["separate"], counts["fp64"], counts["sc"]) > 4, counts
+
+
+# a V-cycle from 2048^2 on copies nothing; one on an array off 16 bytes, or below that size, copies its input and its output
+@pytest.mark.parametrize("N,shift,copies", [(2048, 0, 0), (2048, 1, 2), (1024, 0, 2)])
+def test_copies_of_a_vcycle(N, shift, copies):
+    from torch.profiler import ProfilerActivity, profile
+
+    S = sib.solver_for(I.thin_ellipse_re(N, kappa=1e2), restart=1, max_it=1)
+    b = torch.randn(3 * N * N + 1, device="cuda")[shift: 3 * N * N + shift]
+    z = torch.empty_like(b)
+    S.vcycle(b, z)
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as p:
+        S.vcycle(b, z)
+        torch.cuda.synchronize()
+    assert sum(e.count for e in p.key_averages() if "Memcpy DtoD" in e.key) == copies
+    S.close()
